@@ -186,7 +186,7 @@ void free_all(hfcr_ctx *c) {
     c->eorder_n[0] = c->eorder_n[1] = 0;
     for (int i = 0; i < 2; ++i) {
         Bvh &b = c->bvh[i];
-        void *bp[] = {b.nodes, b.parent, b.flags, b.leaf_face, b.leaf_tri, b.keys, b.keys_alt,
+        void *bp[] = {b.nodes, b.parent, b.top, b.leaf_face, b.leaf_tri, b.keys, b.keys_alt,
                       b.vals_alt, b.bounds, b.bounds_part, b.d_rest};
         for (void *p : bp)
             if (p) cudaFree(p);
@@ -940,7 +940,7 @@ hfcr_status hfcr_reserve(hfcr_ctx *ctx, int64_t max_verts, int64_t max_tris, int
         b.cap = (int)T;
         CK(dalloc(&b.nodes, 4 * T));
         CK(dalloc(&b.parent, 2 * T));
-        CK(dalloc(&b.flags, T));
+        CK(dalloc(&b.top, T + 1));
         CK(dalloc(&b.leaf_face, T));
         CK(cudaMalloc(&b.leaf_tri, 80 * T));
         CK(dalloc(&b.keys, T));

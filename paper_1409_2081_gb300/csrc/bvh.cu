@@ -3,7 +3,8 @@
 //
 // The paper only says that detection uses tight bounding volumes (Sec. 1);
 // the hierarchy here is a binary radix tree over 30-bit Morton codes of the
-// face centroids (Karras 2012), refitted bottom-up with arrival counters.
+// face centroids (Karras 2012), refitted bottom-up: block by block in shared
+// memory, then the few nodes that span blocks.
 // Boxes are float32 and conservative: for float32 coordinates min/max are
 // exact, for float64 they are rounded outward, so box rejection never drops
 // a true intersection.
@@ -273,12 +274,22 @@ __device__ __forceinline__ int kdelta(const unsigned long long *K, int n, int i,
     return __clzll(ki ^ kj);
 }
 
+// Leaves per block of the refit.  A node is local when its leaf range lies
+// in one block [REFIT_BLOCK b, REFIT_BLOCK (b + 1)) (its index is an end of
+// that range, so the node does too); the others span blocks.
+constexpr int REFIT_BITS = 9;
+constexpr int REFIT_BLOCK = 1 << REFIT_BITS;
+
 // Karras 2012, one tree per segment: internal node l of the segment whose
 // faces start at t0 covers a key range found from the common-prefix lengths
 // of its neighbours.  Segment-local node l is stored at t0 + l, leaf c at
-// t0 + c (encoded ~(t0 + c)); each segment's root (l = 0) has parent -1.
+// t0 + c (encoded ~(t0 + c)).  Links carry the child's slot and whether the
+// parent is local: (parent << 2) | (local << 1) | (1 for the right child),
+// parents being below 2^29; roots (l = 0) keep the -1 the caller set.  The
+// nodes that span blocks are listed in top[1 ...], their number in top[0]
+// (zeroed by the caller).
 __global__ void k_karras(const unsigned long long *keys, int n_total, const int *segs, int col,
-                         int nseg, float4 *nodes, int *iparent, int *lparent) {
+                         int nseg, float4 *nodes, int *iparent, int *lparent, int *top) {
     HFCR_PDL_WAIT();
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= n_total) return;
@@ -305,14 +316,12 @@ __global__ void k_karras(const unsigned long long *keys, int n_total, const int 
     int gamma = i + s * d + min(d, 0);
     int left = (min(i, j) == gamma) ? ~(t0 + gamma) : t0 + gamma;
     int right = (max(i, j) == gamma + 1) ? ~(t0 + gamma + 1) : t0 + gamma + 1;
-    // child ids, then the node's leaf range (first, last; one end is gi), which
-    // the refit uses to keep a warp's own subtrees in shared memory
-    nodes[4 * gi + 3] = make_float4(__int_as_float(left), __int_as_float(right),
-                                    __int_as_float(t0 + min(i, j)), __int_as_float(t0 + max(i, j)));
-    // parent links carry the child's slot: (parent << 1) | (1 for the right child)
-    if (left < 0) lparent[~left] = gi << 1; else iparent[left] = gi << 1;
-    if (right < 0) lparent[~right] = (gi << 1) | 1; else iparent[right] = (gi << 1) | 1;
-    if (i == 0) iparent[gi] = -1;
+    nodes[4 * gi + 3] = make_float4(__int_as_float(left), __int_as_float(right), 0.f, 0.f);
+    const bool local = ((t0 + i) >> REFIT_BITS) == ((t0 + j) >> REFIT_BITS);
+    const int link = (gi << 2) | (local ? 2 : 0);
+    if (left < 0) lparent[~left] = link; else iparent[left] = link;
+    if (right < 0) lparent[~right] = link | 1; else iparent[right] = link | 1;
+    if (!local) top[1 + atomicAdd(top, 1)] = gi;
 }
 
 template <typename T>
@@ -337,101 +346,151 @@ __device__ __forceinline__ void pack_leaf<double>(void *leaf_tri, int j, const d
     L[4] = make_double2(c[2], __longlong_as_double((long long)f));
 }
 
-// Bottom-up refit, one thread per leaf, warp by warp: warp w owns leaves
-// [32 w, 32 w + 32).  A node whose leaf range lies in its warp's block (its
-// whole subtree does) is met by two lanes of that warp: they hand over
-// through shared memory (box slots and an arrival counter, block-scope
-// fences), and the second writes both child boxes of the node.  Above the
-// block, the second child to arrive at a node (an acquire-release atomic
-// counter in global memory) merges the two boxes.  Min and max are exact,
-// so the boxes do not depend on the arrival order.
-constexpr int REFIT_WARPS = 8;
-
+// Refit, first kernel: one CTA per block of REFIT_BLOCK leaves, one thread
+// per leaf.  The boxes of the block's local nodes are merged in shared
+// memory: both children of a local node are carried by threads of this CTA,
+// which meet at the node's slot (an arrival counter, block-scope fences);
+// the second carries the union upwards, its links read from shared memory.
+// Then thread t writes node base + t.  A box whose parent spans blocks goes
+// to the parent's child slot in global memory; the slot of a child that
+// itself spans blocks is set empty, for the second kernel.  Min and max are
+// exact, so the boxes do not depend on the order.
+// Bound by the latency of the position gathers, then by some ten shared-
+// memory steps; 512 leaves keep four CTAs on an SM.  With arrival counters in
+// global memory for every node above a warp's 32 leaves a level cost about
+// 2 us (fence, atomic, sibling read).  Both kernels together, against that
+// form: 327,680 float32 faces 71 -> 39 us, 262,144 51 -> 34, 1,280 float64
+// faces 24 -> 17, 5.06 million in 1,024 trees 503 -> 273.
 template <typename T>
-__global__ void __launch_bounds__(32 * REFIT_WARPS) k_refit(
+__global__ void __launch_bounds__(REFIT_BLOCK) k_refit_block(
     const T *x, const T *y, const T *z, int nv, const int *tris, const int *leaf_face, int n,
-    float4 *nodes, const int *iparent, const int *lparent, unsigned *flags, void *leaf_tri,
-    uint32_t *st) {
+    float4 *nodes, const int *iparent, const int *lparent, void *leaf_tri, uint32_t *st) {
     HFCR_PDL_WAIT();
-    __shared__ unsigned cnt[REFIT_WARPS][32];
-    __shared__ float sbox[REFIT_WARPS][32][12];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int base = (blockIdx.x * REFIT_WARPS + w) * 32;
-    cnt[w][lane] = 0u;
-    __syncwarp();
-    const int j = base + lane;
-    if (j >= n) return;
-    int f = leaf_face[j];
-    T a[3], b[3], c[3];
-    load3(x, y, z, chk(tris[3 * f], nv, st), a);
-    load3(x, y, z, chk(tris[3 * f + 1], nv, st), b);
-    load3(x, y, z, chk(tris[3 * f + 2], nv, st), c);
-    pack_leaf<T>(leaf_tri, j, a, b, c, f);
-    float lo[3], hi[3];
+    __shared__ float sb[12][REFIT_BLOCK];  // both child boxes of each local node
+    __shared__ int up[REFIT_BLOCK];
+    __shared__ unsigned cnt[REFIT_BLOCK];
+    const int t = threadIdx.x, base = blockIdx.x * REFIT_BLOCK, j = base + t;
+    const bool live = j < n;
+    int link = -1;
+    float lo[3] = {0.f, 0.f, 0.f}, hi[3] = {0.f, 0.f, 0.f};
+    cnt[t] = 0u;
+    up[t] = live ? iparent[j] : -1;
+    if (live) {
+        link = lparent[j];  // -1: the only face of its segment
+        const int f = leaf_face[j];
+        T a[3], b[3], c[3];
+        load3(x, y, z, chk(tris[3 * f], nv, st), a);
+        load3(x, y, z, chk(tris[3 * f + 1], nv, st), b);
+        load3(x, y, z, chk(tris[3 * f + 2], nv, st), c);
+        pack_leaf<T>(leaf_tri, j, a, b, c, f);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        lo[k] = lo_f(fmin(fmin(a[k], b[k]), c[k]));
-        hi[k] = hi_f(fmax(fmax(a[k], b[k]), c[k]));
+        for (int k = 0; k < 3; ++k) {
+            lo[k] = lo_f(fmin(fmin(a[k], b[k]), c[k]));
+            hi[k] = hi_f(fmax(fmax(a[k], b[k]), c[k]));
+        }
     }
-    int link = lparent[j];  // (parent << 1) | slot, -1 at a root
+    __syncthreads();
     // bounded by the tree depth (< 64 for unique 62-bit keys); the guard
     // only keeps a corrupted parent array from looping
-    for (int guard = 0; guard < 128 && link >= 0; ++guard) {
-        const int node = link >> 1;
-        const int side = link & 1;
-        const int up = iparent[node];  // read-only: load it before the handshake
-        float *nf = (float *)(nodes + 4 * node);
-        const float4 n3 = nodes[4 * node + 3];  // ids and leaf range: not written here
-        const int first = __float_as_int(n3.z), last = __float_as_int(n3.w);
-        // both children's lanes are in this warp when the range is: the
-        // node's slot q (one end of its range is the node's own index)
-        const int q = node - base;
-        if (first >= base && last < base + 32 && q >= 0 && q < 32) {
-            float *mine = sbox[w][q] + 6 * side;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                mine[k] = lo[k];
-                mine[3 + k] = hi[k];
-            }
-            __threadfence_block();
-            if (atomicAdd(&cnt[w][q], 1u) == 0u) return;
-            __threadfence_block();
-            const volatile float *sb = sbox[w][q];
-            float bx[12];
-#pragma unroll
-            for (int k = 0; k < 12; ++k) bx[k] = sb[k];
-            float4 *nd = nodes + 4 * node;
-            nd[0] = make_float4(bx[0], bx[1], bx[2], bx[3]);
-            nd[1] = make_float4(bx[4], bx[5], bx[6], bx[7]);
-            nd[2] = make_float4(bx[8], bx[9], bx[10], bx[11]);
-            const int o = 6 * (1 - side);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = fminf(lo[k], bx[o + k]);
-                hi[k] = fmaxf(hi[k], bx[o + 3 + k]);
-            }
-        } else {
-            const int slot = 6 * side;
-            nf[slot + 0] = lo[0];
-            nf[slot + 1] = lo[1];
-            nf[slot + 2] = lo[2];
-            nf[slot + 3] = hi[0];
-            nf[slot + 4] = hi[1];
-            nf[slot + 5] = hi[2];
-            // the first child to arrive leaves; the second (acquire) sees the
-            // first one's box (release) and carries the union upwards
-            unsigned old;
-            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;"
-                         : "=r"(old) : "l"(flags + node) : "memory");
-            if (old == 0) return;
-            const int sib = 6 - slot;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = fminf(lo[k], __ldcg(nf + sib + k));
-                hi[k] = fmaxf(hi[k], __ldcg(nf + sib + 3 + k));
-            }
+    for (int guard = 0; guard < 128 && link >= 0 && (link & 2); ++guard) {
+        const int q = (link >> 2) - base;
+        if ((unsigned)q >= (unsigned)REFIT_BLOCK) {  // unreachable: a local parent is in the block
+            atomicOr(st, ST_BAD_INDEX);
+            link = -1;
+            break;
         }
-        link = up;
+        const int o = (link & 1) ? 6 : 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            sb[o + k][q] = lo[k];
+            sb[o + 3 + k][q] = hi[k];
+        }
+        __threadfence_block();
+        if (atomicAdd(&cnt[q], 1u) == 0u) {
+            link = -1;  // the sibling's thread carries on
+            break;
+        }
+        __threadfence_block();
+        const volatile float *vs = &sb[0][0] + q;
+        const int so = 6 - o;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            lo[k] = fminf(lo[k], vs[(so + k) * REFIT_BLOCK]);
+            hi[k] = fmaxf(hi[k], vs[(so + 3 + k) * REFIT_BLOCK]);
+        }
+        link = up[q];
+    }
+    if (link >= 0) {
+        float2 *s = (float2 *)((float *)(nodes + 4 * (size_t)(link >> 2)) + ((link & 1) ? 6 : 0));
+        s[0] = make_float2(lo[0], lo[1]);
+        s[1] = make_float2(lo[2], hi[0]);
+        s[2] = make_float2(hi[1], hi[2]);
+    }
+    __syncthreads();
+    if (!live) return;
+    if (cnt[t] == 2u) {
+        float4 *nd = nodes + 4 * (size_t)j;
+        nd[0] = make_float4(sb[0][t], sb[1][t], sb[2][t], sb[3][t]);
+        nd[1] = make_float4(sb[4][t], sb[5][t], sb[6][t], sb[7][t]);
+        nd[2] = make_float4(sb[8][t], sb[9][t], sb[10][t], sb[11][t]);
+    } else if (up[t] >= 0) {  // a node that spans blocks (and is not a root)
+        const int l = up[t];
+        const float inf = __int_as_float(0x7f800000);
+        float2 *s = (float2 *)((float *)(nodes + 4 * (size_t)(l >> 2)) + ((l & 1) ? 6 : 0));
+        s[0] = make_float2(inf, inf);
+        s[1] = make_float2(inf, -inf);
+        s[2] = make_float2(-inf, -inf);
+    }
+}
+
+// *p = min(*p, v) / max(*p, v) of floats by integer atomics: non-negative
+// floats order as signed integers, negative ones in reverse as unsigned
+__device__ __forceinline__ void red_min(float *p, float v) {
+    const int b = __float_as_int(v);
+    if (b >= 0) atomicMin((int *)p, b);
+    else atomicMax((unsigned *)p, (unsigned)b);
+}
+__device__ __forceinline__ void red_max(float *p, float v) {
+    const int b = __float_as_int(v);
+    if (b >= 0) atomicMax((int *)p, b);
+    else atomicMin((unsigned *)p, (unsigned)b);
+}
+
+// Refit, second kernel: one thread per node that spans blocks.  It carries
+// the union of the child boxes it finds (those of local children, written by
+// the first kernel) up the tree, widening each ancestor's slot by atomics
+// that nothing waits for, and stops where the slot already holds its box:
+// whoever widened that slot carries the same bounds on, so every slot ends
+// as the union over its leaves.  There are about ten such nodes per block
+// boundary, and a step costs one read of the slot instead of a handshake.
+__global__ void __launch_bounds__(256) k_refit_top(float4 *nodes, const int *iparent,
+                                                   const int *top, int n) {
+    HFCR_PDL_WAIT();
+    const int nt = min(top[0], n);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += gridDim.x * blockDim.x) {
+        const int node = top[1 + i];
+        const float2 *c = (const float2 *)(nodes + 4 * (size_t)node);
+        float2 v[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = __ldcg(c + k);
+        const float lo[3] = {fminf(v[0].x, v[3].x), fminf(v[0].y, v[3].y), fminf(v[1].x, v[4].x)};
+        const float hi[3] = {fmaxf(v[1].y, v[4].y), fmaxf(v[2].x, v[5].x), fmaxf(v[2].y, v[5].y)};
+        int link = iparent[node];
+        for (int guard = 0; guard < 128 && link >= 0; ++guard) {
+            const int p = link >> 2;
+            float *s = (float *)(nodes + 4 * (size_t)p) + ((link & 1) ? 6 : 0);
+            const float2 a = __ldcg((const float2 *)s), b = __ldcg((const float2 *)s + 1),
+                         d = __ldcg((const float2 *)s + 2);
+            link = iparent[p];
+            bool wider = false;
+            if (lo[0] < a.x) { red_min(s, lo[0]); wider = true; }
+            if (lo[1] < a.y) { red_min(s + 1, lo[1]); wider = true; }
+            if (lo[2] < b.x) { red_min(s + 2, lo[2]); wider = true; }
+            if (hi[0] > b.y) { red_max(s + 3, hi[0]); wider = true; }
+            if (hi[1] > d.x) { red_max(s + 4, hi[1]); wider = true; }
+            if (hi[2] > d.y) { red_max(s + 5, hi[2]); wider = true; }
+            if (!wider) break;
+        }
     }
 }
 
@@ -544,10 +603,13 @@ void bvh_build(Bvh &b, const hfcr_mesh &m, const int *segs, int col, int nseg, S
         cudaMemcpyAsync(b.keys, b.keys_alt, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, s);
         cudaMemcpyAsync(b.leaf_face, b.vals_alt, sizeof(int) * n, cudaMemcpyDeviceToDevice, s);
     }
-    // leaves of one-face segments keep parent -1
+    // roots and leaves of one-face segments keep parent -1 (and so does
+    // whatever a malformed segment table leaves out of every tree)
+    cudaMemsetAsync(b.parent, 0xff, sizeof(int) * n, s);
     cudaMemsetAsync(b.parent + b.cap, 0xff, sizeof(int) * n, s);
+    cudaMemsetAsync(b.top, 0, sizeof(int), s);
     { launch_pdl(k_karras, nb, 256, 0, s, b.keys, n, segs, col, nseg, b.nodes, b.parent,
-                 b.parent + b.cap); note_launch(); }
+                 b.parent + b.cap, b.top); note_launch(); }
 }
 
 void edge_order(const int *edges, int ne, const hfcr_mesh &m, const int *segs, int col, int nseg,
@@ -579,20 +641,21 @@ void edge_order(const int *edges, int ne, const hfcr_mesh &m, const int *segs, i
 }
 
 void bvh_refit(Bvh &b, const hfcr_mesh &m, uint32_t *d_status, cudaStream_t s) {
-    int n = b.n;
+    const int n = b.n;
     if (n <= 0) return;
-    cudaMemsetAsync(b.flags, 0, sizeof(unsigned) * n, s);
-    int nb = (n + 32 * REFIT_WARPS - 1) / (32 * REFIT_WARPS);
+    const int nb = (n + REFIT_BLOCK - 1) / REFIT_BLOCK;
     if (m.dtype == HFCR_F32)
-        { launch_pdl(k_refit<float>, nb, 32 * REFIT_WARPS, 0, s, (const float *)m.x, (const float *)m.y,
-                     (const float *)m.z,
-                                          m.n_verts, m.tris, b.leaf_face, n, b.nodes, b.parent,
-                                          b.parent + b.cap, b.flags, b.leaf_tri, d_status); note_launch(); }
+        { launch_pdl(k_refit_block<float>, nb, REFIT_BLOCK, 0, s, (const float *)m.x,
+                     (const float *)m.y, (const float *)m.z, m.n_verts, m.tris, b.leaf_face, n,
+                     b.nodes, b.parent, b.parent + b.cap, b.leaf_tri, d_status); note_launch(); }
     else
-        { launch_pdl(k_refit<double>, nb, 32 * REFIT_WARPS, 0, s, (const double *)m.x, (const double *)m.y,
-                                           (const double *)m.z, m.n_verts, m.tris, b.leaf_face, n,
-                                           b.nodes, b.parent, b.parent + b.cap, b.flags, b.leaf_tri,
-                                           d_status); note_launch(); }
+        { launch_pdl(k_refit_block<double>, nb, REFIT_BLOCK, 0, s, (const double *)m.x,
+                     (const double *)m.y, (const double *)m.z, m.n_verts, m.tris, b.leaf_face, n,
+                     b.nodes, b.parent, b.parent + b.cap, b.leaf_tri, d_status); note_launch(); }
+    if (nb == 1) return;  // every node is local
+    int gt = (16 * nb + 255) / 256;  // about ten spanning nodes per block boundary
+    if (gt > 1216) gt = 1216;
+    { launch_pdl(k_refit_top, gt, 256, 0, s, b.nodes, b.parent, b.top, n); note_launch(); }
 }
 
 }  // namespace hfcr

@@ -97,8 +97,8 @@ struct Bvh {
     int n = 0;                  // leaves (faces)
     int cap = 0;
     float4 *nodes = nullptr;    // [4 * (cap - 1)]
-    int *parent = nullptr;      // [2 * cap - 1]: parent of internal i at [i], of leaf j at [cap - 1 + j]
-    unsigned *flags = nullptr;  // [cap - 1] arrival counters of the refit
+    int *parent = nullptr;      // [2 * cap]: link of internal i at [i], of leaf j at [cap + j] (k_karras)
+    int *top = nullptr;         // [1 + cap] nodes that span blocks of the refit, their number first
     int *leaf_face = nullptr;   // [cap]
     void *leaf_tri = nullptr;   // [cap] packed triangles in leaf order
     unsigned long long *keys = nullptr;      // [cap] (segment, Morton code) sort keys
