@@ -351,13 +351,10 @@ hfcr_status hfcr_resolve(hfcr_ctx *ctx, hfcr_mesh *A, hfcr_mesh *B, double d, in
  * the hierarchies for A and B (a batch laid out as in hfcr_detect_batch
  * when segs is given, one pair when segs is NULL and n_pairs is ignored),
  * times every traversal variant three times on this scene and makes the
- * fastest the context's choice for every later call.  The variants span:
- * the register budget (2, 3 or 4 CTAs of 256 threads per SM), the exact
- * narrow phase inline or out of line, one walk per edge or one per warp of
- * edges of the same mesh pair (0 to 4), and persistent walks fed by a
- * device work queue of edges, with 3 or 4 CTAs per SM and a warp refilling
- * its idle lanes once 8 or 16 are idle (5 to 8).  The stack depth is not
- * tuned: it is set by the deepest tree the build makes.  *chosen (host,
+ * fastest the context's choice for every later call.  The variants span
+ * how many edges a warp takes at a time (32, 16 or 8: variant mod 3) and the
+ * share of the resident CTAs that the walk is given (all, three quarters,
+ * half: variant / 3).  *chosen (host,
  * may be NULL) gets the chosen index; ms (host [n_ms], may be NULL) the
  * best time of each variant per traversal launch (one launch per direction
  * with edges, as a repair iteration of that direction runs it).

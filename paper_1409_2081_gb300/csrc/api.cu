@@ -119,7 +119,7 @@ struct hfcr_ctx {
 
 // device counter slots
 enum { C_PAIRS = 0, C_STENCILS = 1, C_EDGES_A = 2, C_EDGES_B = 3, C_N4 = 4, C_NPAIRS_IN = 5, C_PEFF = 6,
-       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 };
+       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 /* to 13: two words per direction */ };
 
 namespace {
 
@@ -453,7 +453,9 @@ void launch_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bool d
             a.cap = (int)ctx->max_pairs;
             a.stats = ctx->d_stats;
             a.variant = variant;
-            a.queue = ctx->d_cnt + C_QUEUE;
+            a.queue = ctx->d_cnt + C_QUEUE + 2 * d;
+            a.leaves = (int2 *)ctx->ekeys;  // free outside the edge builds
+            a.leaf_cap = (int)(3 * ctx->max_tris);
             detect_launch(a, s, ctx->d_status);
         }
         return;
@@ -496,7 +498,9 @@ void launch_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bool d
         a.cap = (int)ctx->max_pairs;
         a.stats = ctx->d_stats;
         a.variant = ctx->trav_variant;
-        a.queue = ctx->d_cnt + C_QUEUE;
+        a.queue = ctx->d_cnt + C_QUEUE + 2 * d;
+        a.leaves = (int2 *)ctx->ekeys;  // free outside the edge builds
+        a.leaf_cap = (int)(3 * ctx->max_tris);
         prof_begin(ctx, HFCR_STAGE_TRAVERSE, s);
         detect_launch(a, s, ctx->d_status);
         prof_end(ctx, HFCR_STAGE_TRAVERSE, s);
@@ -1347,6 +1351,7 @@ hfcr_status hfcr_autotune(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B,
         double vbest = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
             CK(cudaMemsetAsync(ctx->d_cnt + C_PAIRS, 0, sizeof(int), s));
+            CK(cudaMemsetAsync(ctx->d_cnt + C_QUEUE, 0, 4 * sizeof(int), s));
             CK(cudaEventRecord(e0, s));
             launch_detect(ctx, A, B, dir0, dir1, pl, built, s, true, v);
             CK(cudaEventRecord(e1, s));

@@ -1,12 +1,12 @@
 // Narrow and broad phase of the edge-face detection (Sec. 3) and the
 // penetration stencils (Sec. 4, Fig. 3).
 //
-// One thread per edge of the edge mesh walks the BVH of the oriented mesh's
-// faces with the edge's box, testing both children of a node with one
-// 64-byte node load; at a leaf the exact segment-triangle test decides.
-// Threads take the edges in the Morton order of their midpoints (a cached
-// permutation), so that a warp walks one region of the tree; the packet
-// variants walk a warp's edges together.
+// The broad phase (k_broad) walks the BVH of the oriented mesh's faces with
+// every edge's box, testing both children of a node with one 64-byte node
+// load, and lists the leaves met; the narrow phase (k_narrow) decides each by
+// the exact segment-triangle test.  The edges are taken in the Morton order
+// of their midpoints (a cached permutation), so that a warp walks one region
+// of the tree.
 // Hits are appended (one atomic per hit) as 64-bit keys
 // (dir | edge | face), which a radix sort turns into the lexicographic
 // (dir, v0, v1, face) order because the edges are sorted by (v0, v1).
@@ -80,321 +80,298 @@ __device__ __forceinline__ bool leaf_test_body(const T *p, const T *q, const Lea
     }
 }
 
-// the exact narrow phase out of line: the traversal loop then needs far
-// fewer registers (leaf tests are rare next to node visits)
-template <typename T, bool F32F>
-__device__ __noinline__ bool leaf_test_call(const T *p, const T *q, const Leaf<T> &L, DevStats *st) {
-    return leaf_test_body<T, F32F>(p, q, L, st);
+// ---------------------------------------------------------------------------
+// Broad phase: every warp keeps the pending visits of its edges (the edge's
+// box, its index and a node) on one stack in shared memory and takes the
+// newest 32 of them per step, one per lane, so an edge whose box overlaps
+// thousands of faces is walked by the whole warp instead of by one lane while
+// 31 wait.  While fewer than 32 visits are pending, the warp takes the next
+// edges of the traversal order (its first ones are fixed, the others come
+// from a device counter).  The leaves met, (edge, leaf), are appended to a
+// list for the narrow phase (k_narrow), 32 at a time.
+// Bound by the latency of dependent node loads and by how evenly the long
+// walks spread: one thread per edge with the exact test inline needed 125
+// registers (a quarter of the warps) and left a warp waiting for its longest
+// walk.  Without the test this kernel needs 38 registers, and its lanes stay
+// 95% busy.  Both phases against that form: a direction of 1,024 pairs of
+// spheres of 80 to 20,480 faces 1.61 -> 0.56 ms, of two 262,144-face tori
+// 50 -> 43 us, the 512 x 512 cloth over 327,680 faces 66 -> 50 us, the
+// 200 x 200 cloth over 65,536 faces 64 -> 37 us, two 1,280-face float64
+// spheres 131 -> 24 us.
+// ---------------------------------------------------------------------------
+constexpr int POOL_WARPS = 4;    // warps per CTA
+constexpr int POOL_CAP = 128;    // pending visits in shared memory per warp
+constexpr int POOL_SPILL = 128;  // blocks of 16 visits moved out to local memory at most
+static_assert((POOL_CAP & (POOL_CAP - 1)) == 0 && POOL_CAP >= 64 + 16,
+              "a step pushes up to 64 visits and moves out blocks of 16");
+
+struct PoolSmem {
+    float4 a[POOL_CAP];          // lo.xyz, hi.x
+    float4 b[POOL_CAP];          // hi.yz, edge, node
+    int2 leaf[32 + 64];          // fewer than 32 before a step, at most 64 more after it
+};
+
+// where the narrow phase puts its hits
+struct HitList {
+    unsigned long long *out;
+    int *count;
+    unsigned long long dirbit;
+    int cap, face_bits;
+    DevStats *st;
+};
+// the list between the two phases: n words of (edge, leaf), those beyond cap
+// not stored
+struct LeafList {
+    int2 *items;
+    int *n;
+    int cap;
+};
+
+template <typename T>
+__device__ __forceinline__ void edge_box(const T *p, const T *q, float *lo, float *hi) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = lo_f(p[k] < q[k] ? p[k] : q[k]);
+        hi[k] = hi_f(p[k] < q[k] ? q[k] : p[k]);
+    }
 }
 
-// Traversal variants (picked by hfcr_autotune): MINB = CTAs of 256 threads
-// the compiler must fit per SM (register budget), NOINL = narrow phase out
-// of line, PACKET = a warp whose edges all belong to one mesh pair walks
-// that pair's tree together (one broadcast load per node, a node entered
-// when any lane's box overlaps it, a shared stack per warp); each lane still
-// tests exactly the leaves its own box overlaps, because every box of the
-// tree contains its children's, so the tests and pairs are those of the
-// per-thread walk.  Warps that span two pairs walk per thread.
-template <typename T, bool F32F, int MINB, bool NOINL, bool PACKET>
-__global__ void __launch_bounds__(256, MINB) k_traverse(
-    const int2 *edges, const int *order, int ne, const T *ex, const T *ey, const T *ez, int nv,
-    const float4 *nodes, const void *leaf_tri, int nfaces, const int *segs, int nseg, int ecol,
-    int fcol, unsigned long long dirbit, int face_bits, unsigned long long *out, int *count, int cap,
-    DevStats *st, uint32_t *status) {
+// endpoints of an edge (out-of-range ids read vertex 0 and raise ST_BAD_INDEX)
+template <typename T>
+__device__ __forceinline__ void ld_edge(const int2 ev, const T *ex, const T *ey, const T *ez, int nv, T *p, T *q,
+                                        uint32_t *status) {
+    const int v0 = chk(ev.x, nv, status), v1 = chk(ev.y, nv, status);
+    p[0] = ex[v0]; p[1] = ey[v0]; p[2] = ez[v0];
+    q[0] = ex[v1]; q[1] = ey[v1]; q[2] = ez[v1];
+}
+
+// a node's 64 bytes by two 32-byte loads
+__device__ __forceinline__ void ld_node(const float4 *nodes, int i, float *f) {
+    const double4_32a *nd = (const double4_32a *)(nodes + 4 * (size_t)i);
+    const double4_32a u = nd[0], v = nd[1];
+    const double w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        f[2 * k] = __int_as_float(__double2loint(w[k]));
+        f[2 * k + 1] = __int_as_float(__double2hiint(w[k]));
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
+    const int2 *edges, const int *order, int ne, int chunk, const T *ex, const T *ey, const T *ez,
+    int nv, const float4 *nodes, int nfaces, const int *segs, int nseg, int ecol, int fcol, LeafList out,
+    int *queue, uint32_t *status) {
     HFCR_PDL_WAIT();
-    // thread t takes edge order[t] (a spatially coherent permutation of the
-    // edges, when there is one): a warp then walks neighbouring parts of the
-    // tree; the keys carry the edge's own index
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int e = t >= ne ? ne : (order ? order[t] : t);
+    // malformed input (reported by the host): its tree is not walked
+    if (__any_sync(0xffffffffu, (*(volatile uint32_t *)status & ST_BAD_INDEX) != 0)) return;
+    __shared__ PoolSmem smw[POOL_WARPS];
+    PoolSmem &sm = smw[threadIdx.x >> 5];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int hint = 0;               // segment of this lane's last edge
+    // pending visits: `n` of them in the ring ending at `top` (exclusive), and
+    // `spilled` blocks of 16 older ones in local memory (lanes 0 to 15); nl
+    // leaves wait (all the same in every lane)
+    int top = 0, n = 0, nl = 0, spilled = 0;
+    int2 spill[POOL_SPILL];
+    int base = (blockIdx.x * POOL_WARPS + (threadIdx.x >> 5)) * chunk;  // the next edges
+    // steps since the last edges were taken: guards against a corrupted tree
+    // (an edge visits each of the 2 nfaces - 1 nodes at most once)
+    unsigned steps = 0;
+    const unsigned most = (unsigned)min(64ll * nfaces + 256, 0xffffffffll);
+    while (true) {
+        if (++steps > most) {
+            if (lane == 0) atomicOr(status, ST_BAD_INDEX);
+            break;
+        }
+        const bool fresh = n < 32 && spilled == 0 && base < ne;
+        if (nl >= 32 || (nl > 0 && n == 0 && spilled == 0 && !fresh)) {
+            const int take = min(nl, 32);
+            nl -= take;
+            int at = 0;
+            if (lane == 0) {  // once over the capacity the count only has to stay there
+                at = *(volatile int *)out.n;
+                if (at <= out.cap) at = atomicAdd(out.n, take);
+            }
+            at = __shfl_sync(full, at, 0) + lane;
+            if (lane < take && at < out.cap) out.items[at] = sm.leaf[nl + lane];
+            __syncwarp();
+            continue;
+        }
+        bool on = false;
+        float lo[3] = {0.f, 0.f, 0.f}, hi[3] = {0.f, 0.f, 0.f};
+        int e = 0, node = 0;
+        if (fresh) {
+            const int i = base + lane;
+            int t0 = 0, nleaf = 0;
+            if (lane < chunk && i < ne) {
+                e = order ? order[i] : i;
+                const int2 ev = edges[e];
+                if (nseg > 1 && !(segs[4 * hint + ecol] <= ev.x && ev.x < segs[4 * (hint + 1) + ecol]))
+                    hint = seg_of(segs, ecol, nseg, ev.x);
+                seg_range(segs, fcol, hint, nfaces, t0, nleaf);
+                T p[3], q[3];
+                ld_edge(ev, ex, ey, ez, nv, p, q, status);
+                edge_box(p, q, lo, hi);
+            }
+            steps = 0;
+            if (lane == 0) base = gridDim.x * POOL_WARPS * chunk + atomicAdd(queue, chunk);
+            base = __shfl_sync(full, base, 0);
+            const bool one = nleaf == 1;  // a tree of one leaf: tested outright
+            const unsigned m = __ballot_sync(full, one);
+            if (one) sm.leaf[nl + __popc(m & below)] = make_int2(e, t0);
+            nl += __popc(m);
+            on = nleaf > 1;
+            node = t0;
+        } else if (n > 0) {
+            const int take = min(n, 32);
+            on = lane < take;
+            if (on) {
+                const int at = (top - take + lane) & (POOL_CAP - 1);
+                const float4 u = sm.a[at], w = sm.b[at];
+                lo[0] = u.x; lo[1] = u.y; lo[2] = u.z; hi[0] = u.w;
+                hi[1] = w.x; hi[2] = w.y;
+                e = __float_as_int(w.z);
+                node = __float_as_int(w.w);
+            }
+            top -= take;
+            n -= take;
+            __syncwarp();
+        } else if (spilled > 0) {
+            // a block of older visits back
+            --spilled;
+            if (lane < 16) {
+                const int2 s = spill[spilled];
+                T p[3], q[3];
+                ld_edge(edges[s.x], ex, ey, ez, nv, p, q, status);
+                edge_box(p, q, lo, hi);
+                e = s.x;
+                node = s.y;
+                on = true;
+            }
+        } else {
+            break;
+        }
+        // the visit: the node's two boxes against the edge's
+        int c0 = 0, c1 = 0;
+        bool h0 = false, h1 = false;
+        if (on) {
+            float f[16];
+            ld_node(nodes, node, f);
+            c0 = __float_as_int(f[12]);
+            c1 = __float_as_int(f[13]);
+            h0 = overlap(lo, hi, f[0], f[1], f[2], f[3], f[4], f[5]);
+            h1 = overlap(lo, hi, f[6], f[7], f[8], f[9], f[10], f[11]);
+        }
+        const unsigned l0 = __ballot_sync(full, h0 && c0 < 0), l1 = __ballot_sync(full, h1 && c1 < 0);
+        if (l0 | l1) {
+            if (h0 && c0 < 0) sm.leaf[nl + __popc(l0 & below)] = make_int2(e, ~c0);
+            if (h1 && c1 < 0) sm.leaf[nl + __popc(l0) + __popc(l1 & below)] = make_int2(e, ~c1);
+            nl += __popc(l0) + __popc(l1);
+        }
+        const unsigned i0 = __ballot_sync(full, h0 && c0 >= 0), i1 = __ballot_sync(full, h1 && c1 >= 0);
+        const int add = __popc(i0) + __popc(i1);
+        while (n + add > POOL_CAP) {  // the 16 oldest visits out of the ring
+            if (lane < 16) {
+                const float4 s = sm.b[(top - n + lane) & (POOL_CAP - 1)];
+                if (spilled < POOL_SPILL) spill[spilled] = make_int2(__float_as_int(s.z), __float_as_int(s.w));
+                else atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
+            }
+            spilled = min(spilled + 1, POOL_SPILL);
+            n -= 16;
+            __syncwarp();
+        }
+        const float4 u = make_float4(lo[0], lo[1], lo[2], hi[0]);
+        if (h0 && c0 >= 0) {
+            const int at = (top + __popc(i0 & below)) & (POOL_CAP - 1);
+            sm.a[at] = u;
+            sm.b[at] = make_float4(hi[1], hi[2], __int_as_float(e), __int_as_float(c0));
+        }
+        if (h1 && c1 >= 0) {
+            const int at = (top + __popc(i0) + __popc(i1 & below)) & (POOL_CAP - 1);
+            sm.a[at] = u;
+            sm.b[at] = make_float4(hi[1], hi[2], __int_as_float(e), __int_as_float(c1));
+        }
+        top += add;
+        n += add;
+        __syncwarp();
+    }
+}
+
+// leaf lf against an edge, the hit appended
+template <typename T, bool F32F>
+__device__ __forceinline__ void narrow_test(const T *p, const T *q, int e, int lf, const void *leaf_tri,
+                                            const HitList &o) {
+    Leaf<T> L;
+    L.load(leaf_tri, lf);
+    if (leaf_test_body<T, F32F>(p, q, L, o.st)) {
+        const int pos = atomicAdd(o.count, 1);
+        if (pos < o.cap)
+            o.out[pos] = o.dirbit | ((unsigned long long)e << o.face_bits) | (unsigned)L.face;
+    }
+}
+
+// Narrow phase: the exact test of every (edge, leaf) of the broad phase, one
+// per thread, consecutive warps' work on different CTAs (few tests spread
+// over many SMs: the float64 stages are slow on one).  When the list
+// overflowed, every edge is walked again from its root by one thread, each
+// leaf tested as it is met.
+template <typename T, bool F32F>
+__global__ void __launch_bounds__(128) k_narrow(
+    const int2 *edges, int ne, const T *ex, const T *ey, const T *ez, int nv, const float4 *nodes,
+    const void *leaf_tri, int nfaces, const int *segs, int nseg, int ecol, int fcol, HitList o, LeafList in,
+    uint32_t *status) {
+    HFCR_PDL_WAIT();
+    if (*(volatile uint32_t *)status & ST_BAD_INDEX) return;
+    const int n = *in.n, lane = threadIdx.x & 31;
+    const int first = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + lane, stride = gridDim.x * 128;
+    if (n <= in.cap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&o.st->narrow_tests, (unsigned long long)n);
+        for (int i = first; i < n; i += stride) {
+            const int2 l = in.items[i];
+            T p[3], q[3];
+            ld_edge(edges[l.x], ex, ey, ez, nv, p, q, status);
+            narrow_test<T, F32F>(p, q, l.x, l.y, leaf_tri, o);
+        }
+        return;
+    }
     unsigned tests = 0;
-    int2 ev = make_int2(0, 0);
-    int pair = 0, t0 = 0, nleaf = 0;
-    if (e < ne) {
-        ev = edges[e];
-        // the faces of this edge's own mesh pair form one tree
-        pair = seg_of(segs, ecol, nseg, ev.x);
-        seg_range(segs, fcol, pair, nfaces, t0, nleaf);
-    }
-    const bool active = e < ne && nleaf > 0;
-    bool walked = false;  // by the warp's packet walk
-    if constexpr (PACKET) {
-        const unsigned full = 0xffffffffu;
-        const unsigned act = __ballot_sync(full, active);
-        const int leader = act ? __ffs(act) - 1 : 0;
-        const int lt0 = __shfl_sync(full, t0, leader), lnl = __shfl_sync(full, nleaf, leader);
-        if (act && __all_sync(full, !active || (t0 == lt0 && nleaf == lnl))) {
-            walked = true;
-            __shared__ int pstack[256 / 32][STACK];
-            int *stk = pstack[threadIdx.x >> 5];
-            const int lane = threadIdx.x & 31;
-            T p[3] = {0, 0, 0}, q[3] = {0, 0, 0};
-            float lo[3] = {1.f, 1.f, 1.f}, hi[3] = {0.f, 0.f, 0.f};  // empty for idle lanes
-            if (active) {
-                const int i0 = chk(ev.x, nv, status), i1 = chk(ev.y, nv, status);
-                p[0] = ex[i0]; p[1] = ey[i0]; p[2] = ez[i0];
-                q[0] = ex[i1]; q[1] = ey[i1]; q[2] = ez[i1];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    lo[k] = lo_f(p[k] < q[k] ? p[k] : q[k]);
-                    hi[k] = hi_f(p[k] < q[k] ? q[k] : p[k]);
-                }
-            }
-            const unsigned long long ebits = ((unsigned long long)e) << face_bits;
-            int sp = 0;
-            int node = lnl == 1 ? ~lt0 : lt0;
-            int visits = 0;
-            const int max_visits = 2 * lnl + 8;
-            while (true) {
-                if (++visits > max_visits) {
-                    if (lane == 0) atomicOr(status, ST_BAD_INDEX);
-                    break;
-                }
-                int leaf0 = -1, leaf1 = -1, next = -1, push = -1;
-                bool m0 = false, m1 = false;
-                if (node < 0) {
-                    leaf0 = ~node;
-                    m0 = active;
-                } else {
-                    const float4 *nd = nodes + 4 * node;
-                    const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
-                    const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-                    const bool h0 = active && overlap(lo, hi, n0.x, n0.y, n0.z, n0.w, n1.x, n1.y);
-                    const bool h1 = active && overlap(lo, hi, n1.z, n1.w, n2.x, n2.y, n2.z, n2.w);
-                    const bool a0 = __any_sync(full, h0), a1 = __any_sync(full, h1);
-                    if (a0) {
-                        if (c0 < 0) { leaf0 = ~c0; m0 = h0; } else next = c0;
-                    }
-                    if (a1) {
-                        if (c1 < 0) { leaf1 = ~c1; m1 = h1; }
-                        else if (next < 0) next = c1;
-                        else push = c1;
-                    }
-                }
-#pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    const int lf = w ? leaf1 : leaf0;
-                    if (lf >= 0 && (w ? m1 : m0)) {
-                        Leaf<T> L;
-                        L.load(leaf_tri, lf);
-                        ++tests;
-                        bool hit;
-                        if constexpr (NOINL) hit = leaf_test_call<T, F32F>(p, q, L, st);
-                        else hit = leaf_test_body<T, F32F>(p, q, L, st);
-                        if (hit) {
-                            int pos = atomicAdd(count, 1);
-                            if (pos < cap) out[pos] = dirbit | ebits | (unsigned)L.face;
-                        }
-                    }
-                }
-                __syncwarp();
-                if (push >= 0) {
-                    if (sp < STACK) {
-                        if (lane == 0) stk[sp] = push;
-                        ++sp;
-                        __syncwarp();
-                    } else if (lane == 0) {
-                        atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
-                    }
-                }
-                if (next >= 0) {
-                    node = next;
-                    continue;
-                }
-                if (sp == 0) break;
-                node = stk[--sp];
-            }
-        }
-    }
-    if (active && !walked) {
-        int i0 = chk(ev.x, nv, status), i1 = chk(ev.y, nv, status);
-        T p[3] = {ex[i0], ey[i0], ez[i0]}, q[3] = {ex[i1], ey[i1], ez[i1]};
+    for (int e = first; e < ne; e += stride) {
+        const int2 ev = edges[e];
+        int t0, nleaf;
+        seg_range(segs, fcol, seg_of(segs, ecol, nseg, ev.x), nfaces, t0, nleaf);
+        if (nleaf < 1) continue;
+        T p[3], q[3];
+        ld_edge(ev, ex, ey, ez, nv, p, q, status);
         float lo[3], hi[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = lo_f(p[k] < q[k] ? p[k] : q[k]);
-            hi[k] = hi_f(p[k] < q[k] ? q[k] : p[k]);
-        }
-        const unsigned long long ebits = ((unsigned long long)e) << face_bits;
+        edge_box(p, q, lo, hi);
         int stack[STACK];
-        int sp = 0;
-        int node = nleaf == 1 ? ~t0 : t0;
-        // a tree of nleaf leaves has 2 nleaf - 1 nodes; each is visited at
-        // most once per edge, so the bound only guards a corrupted tree
-        int visits = 0;
-        const int max_visits = 2 * nleaf + 8;
+        int sp = 0, node = nleaf == 1 ? ~t0 : t0, visits = 0;
         while (true) {
-            if (++visits > max_visits) {
+            if (++visits > 2 * nleaf + 8) {  // a corrupted tree
                 atomicOr(status, ST_BAD_INDEX);
                 break;
             }
-            int leaf0 = -1, leaf1 = -1;
-            int next = -1, push = -1;
             if (node < 0) {
-                leaf0 = ~node;
+                narrow_test<T, F32F>(p, q, e, ~node, leaf_tri, o);
+                ++tests;
             } else {
-                const float4 *nd = nodes + 4 * node;
-                float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
-                int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-                bool h0 = overlap(lo, hi, n0.x, n0.y, n0.z, n0.w, n1.x, n1.y);
-                bool h1 = overlap(lo, hi, n1.z, n1.w, n2.x, n2.y, n2.z, n2.w);
-                if (h0) { if (c0 < 0) leaf0 = ~c0; else next = c0; }
-                if (h1) {
-                    if (c1 < 0) leaf1 = ~c1;
-                    else if (next < 0) next = c1;
-                    else push = c1;
+                float f[16];
+                ld_node(nodes, node, f);
+                if (sp + 2 > STACK) {
+                    atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
+                    break;
                 }
-            }
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-                int lf = w ? leaf1 : leaf0;
-                if (lf >= 0) {
-                    Leaf<T> L;
-                    L.load(leaf_tri, lf);
-                    ++tests;
-                    bool hit;
-                    if constexpr (NOINL) hit = leaf_test_call<T, F32F>(p, q, L, st);
-                    else hit = leaf_test_body<T, F32F>(p, q, L, st);
-                    if (hit) {
-                        int pos = atomicAdd(count, 1);
-                        if (pos < cap) out[pos] = dirbit | ebits | (unsigned)L.face;
-                    }
-                }
-            }
-            if (push >= 0) {
-                if (sp < STACK) stack[sp++] = push;
-                else atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
-            }
-            if (next >= 0) {
-                node = next;
-                continue;
+                if (overlap(lo, hi, f[6], f[7], f[8], f[9], f[10], f[11])) stack[sp++] = __float_as_int(f[13]);
+                if (overlap(lo, hi, f[0], f[1], f[2], f[3], f[4], f[5])) stack[sp++] = __float_as_int(f[12]);
             }
             if (sp == 0) break;
             node = stack[--sp];
         }
     }
-    unsigned tot = __reduce_add_sync(0xffffffffu, tests);
-    if ((threadIdx.x & 31) == 0 && tot) atomicAdd(&st->narrow_tests, (unsigned long long)tot);
-}
-
-// ---------------------------------------------------------------------------
-// Persistent traversal with a device work queue (variants 5 to 8): a grid
-// of as many CTAs as fit on the GPU at once; every warp keeps its lanes
-// busy by handing each lane whose walk has ended the next edge of the
-// traversal order from one global counter (one atomic per refill, once at
-// least FETCH lanes are idle).  Every lane then takes one node per step,
-// so short walks (edges that leave at the root of their pair's tree) no
-// longer idle their warp until its longest walk ends, and no CTA outlives
-// the others with a few long walks.  Edges are handed out in the Morton
-// order of their midpoints, so a warp still walks one region of a tree.
-// The pairs and tests are exactly those of the per-edge walk.
-// ---------------------------------------------------------------------------
-template <typename T, bool F32F, int MINB, int FETCH>
-__global__ void __launch_bounds__(256, MINB) k_traverse_q(
-    const int2 *edges, const int *order, int ne, const T *ex, const T *ey, const T *ez, int nv,
-    const float4 *nodes, const void *leaf_tri, int nfaces, const int *segs, int nseg, int ecol,
-    int fcol, unsigned long long dirbit, int face_bits, unsigned long long *out, int *count, int cap,
-    int *queue, DevStats *st, uint32_t *status) {
-    HFCR_PDL_WAIT();
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    bool active = false, drained = false;
-    int e = 0, node = 0, sp = 0, visits = 0, max_visits = 0;
-    T p[3] = {0, 0, 0}, q[3] = {0, 0, 0};
-    float lo[3] = {0.f, 0.f, 0.f}, hi[3] = {0.f, 0.f, 0.f};
-    unsigned long long ebits = 0;
-    int stack[STACK];
-    unsigned tests = 0;
-    while (true) {
-        // refill the idle lanes from the queue (warp-uniform decision)
-        const unsigned idle = __ballot_sync(full, !active);
-        if (!drained && __popc(idle) >= (idle == full ? 1 : FETCH)) {
-            const int leader = __ffs(idle) - 1;
-            int base = 0;
-            if (lane == leader) base = atomicAdd(queue, __popc(idle));
-            base = __shfl_sync(full, base, leader);
-            if (base + __popc(idle) >= ne) drained = true;
-            if (!active) {
-                const int t = base + __popc(idle & below);
-                if (t < ne) {
-                    e = order ? order[t] : t;
-                    const int2 ev = edges[e];
-                    const int pair = seg_of(segs, ecol, nseg, ev.x);
-                    int t0, nleaf;
-                    seg_range(segs, fcol, pair, nfaces, t0, nleaf);
-                    if (nleaf > 0) {
-                        const int i0 = chk(ev.x, nv, status), i1 = chk(ev.y, nv, status);
-                        p[0] = ex[i0]; p[1] = ey[i0]; p[2] = ez[i0];
-                        q[0] = ex[i1]; q[1] = ey[i1]; q[2] = ez[i1];
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            lo[k] = lo_f(p[k] < q[k] ? p[k] : q[k]);
-                            hi[k] = hi_f(p[k] < q[k] ? q[k] : p[k]);
-                        }
-                        ebits = ((unsigned long long)e) << face_bits;
-                        node = nleaf == 1 ? ~t0 : t0;
-                        sp = 0;
-                        visits = 0;
-                        // a tree of nleaf leaves has 2 nleaf - 1 nodes, each
-                        // visited at most once per edge: the bound only guards
-                        // a corrupted tree
-                        max_visits = 2 * nleaf + 8;
-                        active = true;
-                    }
-                }
-            }
-        }
-        if (!__any_sync(full, active)) {
-            if (drained) break;
-            continue;  // every fetched edge had an empty pair; fetch again
-        }
-        if (!active) continue;
-        // one step of this lane's walk
-        if (++visits > max_visits) {
-            atomicOr(status, ST_BAD_INDEX);
-            active = false;
-            continue;
-        }
-        int leaf0 = -1, leaf1 = -1, next = -1, push = -1;
-        if (node < 0) {
-            leaf0 = ~node;
-        } else {
-            const float4 *nd = nodes + 4 * node;
-            const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
-            const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-            const bool h0 = overlap(lo, hi, n0.x, n0.y, n0.z, n0.w, n1.x, n1.y);
-            const bool h1 = overlap(lo, hi, n1.z, n1.w, n2.x, n2.y, n2.z, n2.w);
-            if (h0) { if (c0 < 0) leaf0 = ~c0; else next = c0; }
-            if (h1) {
-                if (c1 < 0) leaf1 = ~c1;
-                else if (next < 0) next = c1;
-                else push = c1;
-            }
-        }
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            const int lf = w ? leaf1 : leaf0;
-            if (lf >= 0) {
-                Leaf<T> L;
-                L.load(leaf_tri, lf);
-                ++tests;
-                if (leaf_test_call<T, F32F>(p, q, L, st)) {
-                    const int pos = atomicAdd(count, 1);
-                    if (pos < cap) out[pos] = dirbit | ebits | (unsigned)L.face;
-                }
-            }
-        }
-        if (push >= 0) {
-            if (sp < STACK) stack[sp++] = push;
-            else atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
-        }
-        if (next >= 0) node = next;
-        else if (sp > 0) node = stack[--sp];
-        else active = false;
-    }
-    unsigned tot = __reduce_add_sync(full, tests);
-    if (lane == 0 && tot) atomicAdd(&st->narrow_tests, (unsigned long long)tot);
+    if (tests) atomicAdd(&o.st->narrow_tests, (unsigned long long)tests);
 }
 
 __global__ void k_keys_to_pairs(const unsigned long long *keys, const int *d_n, int cap,
@@ -555,19 +532,9 @@ void pair_products(const int *edges, int ne, const int *segs, int nseg, int ecol
                                                         fcol, nfaces, stats); note_launch(); }
 }
 
-template <typename T, bool F32F, int MINB, bool NOINL, bool PACKET>
-static void launch_traverse(const DetectArgs &a, const T *x, const T *y, const T *z, int nb,
-                            unsigned long long dirbit, cudaStream_t s, uint32_t *d_status) {
-    const hfcr_mesh &m = *a.edge_mesh;
-    { launch_pdl(k_traverse<T, F32F, MINB, NOINL, PACKET>, nb, 256, 0, s, (const int2 *)a.edges,
-                 a.order, a.n_edges, x, y, z, m.n_verts, a.bvh->nodes, a.bvh->leaf_tri,
-          a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, dirbit, a.face_bits, a.keys, a.d_count, a.cap,
-          a.stats, d_status); note_launch(); }
-}
-
-// resident CTAs of a persistent traversal kernel on this device (cached)
-template <typename K>
-static int resident_ctas(K kern) {
+// resident CTAs of the broad phase on this device (cached)
+template <typename T>
+static int broad_ctas() {
     static int dev_cache[64];
     static bool done[64];
     int dev = 0;
@@ -576,60 +543,46 @@ static int resident_ctas(K kern) {
     if (!done[dev]) {
         int sms = 0, per = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_broad<T>, 32 * POOL_WARPS, 0);
         dev_cache[dev] = sms * (per > 0 ? per : 1);
         done[dev] = true;
     }
     return dev_cache[dev];
 }
 
-template <typename T, bool F32F, int MINB, int FETCH>
-static void launch_queue(const DetectArgs &a, const T *x, const T *y, const T *z,
-                         unsigned long long dirbit, cudaStream_t s, uint32_t *d_status) {
-    const hfcr_mesh &m = *a.edge_mesh;
-    auto kern = k_traverse_q<T, F32F, MINB, FETCH>;
-    int grid = resident_ctas(kern);
-    const int need = (a.n_edges + 255) / 256;
-    if (grid > need) grid = need;
-    cudaMemsetAsync(a.queue, 0, sizeof(int), s);
-    { launch_pdl(kern, grid, 256, 0, s, (const int2 *)a.edges, a.order, a.n_edges, x, y, z,
-                 m.n_verts, a.bvh->nodes, a.bvh->leaf_tri, a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol,
-                 dirbit, a.face_bits, a.keys, a.d_count, a.cap, a.queue, a.stats, d_status);
-      note_launch(); }
-}
-
 template <typename T, bool F32F>
-static void launch_variant(const DetectArgs &a, const T *x, const T *y, const T *z, int nb,
-                           unsigned long long dirbit, cudaStream_t s, uint32_t *d_status) {
-    switch (a.variant) {
-        case 5: launch_queue<T, F32F, 3, 8>(a, x, y, z, dirbit, s, d_status); return;
-        case 6: launch_queue<T, F32F, 4, 8>(a, x, y, z, dirbit, s, d_status); return;
-        case 7: launch_queue<T, F32F, 3, 16>(a, x, y, z, dirbit, s, d_status); return;
-        case 8: launch_queue<T, F32F, 4, 16>(a, x, y, z, dirbit, s, d_status); return;
-        default: break;
-    }
-    switch (a.variant) {
-        case 1: launch_traverse<T, F32F, 4, true, false>(a, x, y, z, nb, dirbit, s, d_status); break;
-        case 2: launch_traverse<T, F32F, 3, true, false>(a, x, y, z, nb, dirbit, s, d_status); break;
-        case 3: launch_traverse<T, F32F, 2, false, true>(a, x, y, z, nb, dirbit, s, d_status); break;
-        case 4: launch_traverse<T, F32F, 4, true, true>(a, x, y, z, nb, dirbit, s, d_status); break;
-        default: launch_traverse<T, F32F, 2, false, false>(a, x, y, z, nb, dirbit, s, d_status); break;
-    }
+static void launch_phases(const DetectArgs &a, cudaStream_t s, uint32_t *d_status) {
+    const hfcr_mesh &m = *a.edge_mesh;
+    const T *x = (const T *)m.x, *y = (const T *)m.y, *z = (const T *)m.z;
+    const unsigned long long dirbit = (unsigned long long)a.dir << (a.edge_bits + a.face_bits);
+    // the variant: 32, 16 or 8 edges taken at a time, on all, 3/4 or half of
+    // the CTAs that fit; with few edges fewer at a time, so that every warp
+    // has some (down to 4: a tree's levels are walked one after the other
+    // however few edges a warp has)
+    int grid = broad_ctas<T>() * (4 - a.variant / 3) / 4;
+    if (grid < 1) grid = 1;
+    const int most = 32 >> (a.variant % 3);
+    int chunk = (a.n_edges + grid * POOL_WARPS - 1) / (grid * POOL_WARPS);
+    chunk = chunk < 4 ? 4 : (chunk > most ? most : chunk);
+    const int need = (a.n_edges + chunk * POOL_WARPS - 1) / (chunk * POOL_WARPS);
+    if (grid > need) grid = need;
+    const LeafList l = {a.leaves, a.queue + 1, a.leaf_cap};
+    { launch_pdl(k_broad<T>, grid, 32 * POOL_WARPS, 0, s, (const int2 *)a.edges, a.order, a.n_edges, chunk, x,
+                 y, z, m.n_verts, a.bvh->nodes, a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, l, a.queue, d_status);
+      note_launch(); }
+    const HitList o = {a.keys, a.d_count, dirbit, a.cap, a.face_bits, a.stats};
+    int gn = (a.n_edges + 127) / 128;
+    if (gn > 8 * 152) gn = 8 * 152;
+    { launch_pdl(k_narrow<T, F32F>, gn, 128, 0, s, (const int2 *)a.edges, a.n_edges, x, y, z, m.n_verts,
+                 a.bvh->nodes, a.bvh->leaf_tri, a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, o, l, d_status);
+      note_launch(); }
 }
 
 void detect_launch(const DetectArgs &a, cudaStream_t s, uint32_t *d_status) {
     if (a.n_edges <= 0 || a.bvh->n <= 0) return;
-    const hfcr_mesh &m = *a.edge_mesh;
-    int nb = (a.n_edges + 255) / 256;
-    unsigned long long dirbit = (unsigned long long)a.dir << (a.edge_bits + a.face_bits);
-    if (m.dtype == HFCR_F32) {
-        const float *x = (const float *)m.x, *y = (const float *)m.y, *z = (const float *)m.z;
-        if (a.f32_filter) launch_variant<float, true>(a, x, y, z, nb, dirbit, s, d_status);
-        else launch_variant<float, false>(a, x, y, z, nb, dirbit, s, d_status);
-    } else {
-        const double *x = (const double *)m.x, *y = (const double *)m.y, *z = (const double *)m.z;
-        launch_variant<double, false>(a, x, y, z, nb, dirbit, s, d_status);
-    }
+    if (a.edge_mesh->dtype != HFCR_F32) launch_phases<double, false>(a, s, d_status);
+    else if (a.f32_filter) launch_phases<float, true>(a, s, d_status);
+    else launch_phases<float, false>(a, s, d_status);
 }
 
 void keys_to_pairs(const unsigned long long *keys, const int *d_n, int cap, const int *edgesA,

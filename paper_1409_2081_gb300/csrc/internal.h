@@ -193,8 +193,10 @@ struct DetectArgs {
     int *d_count;
     int cap;
     DevStats *stats;
-    int variant = 0;  // traversal variant (0 to 8; see detect.cu)
-    int *queue = nullptr;  // work counter of the persistent variants (zeroed by the launch)
+    int variant = 0;       // traversal variant (0 to 8; see detect.cu)
+    int *queue = nullptr;  // [2] edges taken, leaves listed (zero before the launch)
+    int2 *leaves = nullptr;  // [leaf_cap] (edge, leaf) between the broad and the narrow phase
+    int leaf_cap = 0;
 };
 constexpr int N_TRAVERSE_VARIANTS = 9;
 void detect_launch(const DetectArgs &a, cudaStream_t s, uint32_t *d_status);
