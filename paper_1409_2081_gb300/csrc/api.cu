@@ -119,7 +119,8 @@ struct hfcr_ctx {
 
 // device counter slots
 enum { C_PAIRS = 0, C_STENCILS = 1, C_EDGES_A = 2, C_EDGES_B = 3, C_N4 = 4, C_NPAIRS_IN = 5, C_PEFF = 6,
-       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 /* to 13: two words per direction */ };
+       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 /* to 13: two words per direction */,
+       C_SLOW = 14 };
 
 namespace {
 
@@ -312,6 +313,31 @@ hfcr_status check_pair(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B) {
     return HFCR_OK;
 }
 
+hfcr_status read_back(hfcr_ctx *ctx, cudaStream_t s);
+
+// Unique edges of a triangle list into out (room for 3 n_tris), their number
+// to *ne; synchronises.  C_SLOW is zero before.
+hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts, int *out, int slot,
+                         int *ne, cudaStream_t s) {
+    // the buckets' words fit the vertex scratch of the reservation; a caller
+    // with more vertices than reserved takes the sort
+    bool fast = n_tris > 0 && n_verts > 0 &&
+                bucket_words(n_verts) * sizeof(int) <= sizeof(double) * 6 * (size_t)ctx->max_verts;
+    for (;; fast = false) {
+        if (fast)
+            build_edges(tris, n_tris, n_verts, out, ctx->d_cnt + slot, ctx->d_cnt + C_SLOW, ctx->ekeys,
+                        ctx->ekeys_alt, (int *)ctx->field_alt, ctx->d_status, s);
+        else
+            build_edges_sorted(tris, n_tris, n_verts, out, ctx->d_cnt + slot, ctx->ekeys, ctx->ekeys_alt,
+                               ctx->eflags, ctx->sort, ctx->d_status, s);
+        hfcr_status st = read_back(ctx, s);
+        if (st) return st;
+        if (!fast || !ctx->h_cnt[C_SLOW]) break;
+    }
+    *ne = ctx->h_cnt[slot];
+    return HFCR_OK;
+}
+
 // Edges of mesh `which` (0 = A, 1 = B): the caller's, or built into the
 // context (synchronises to learn the count).
 hfcr_status mesh_edges(hfcr_ctx *ctx, const hfcr_mesh *m, int which, const int **edges, int *ne,
@@ -321,14 +347,9 @@ hfcr_status mesh_edges(hfcr_ctx *ctx, const hfcr_mesh *m, int which, const int *
         *ne = m->n_edges;
         return HFCR_OK;
     }
-    int slot = which ? C_EDGES_B : C_EDGES_A;
-    build_edges(m->tris, m->n_tris, m->n_verts, ctx->edges[which], ctx->d_cnt + slot, ctx->ekeys,
-                ctx->ekeys_alt, ctx->eflags, ctx->sort, ctx->d_status, s);
-    CK(cudaMemcpyAsync(ctx->h_cnt + slot, ctx->d_cnt + slot, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     *edges = ctx->edges[which];
-    *ne = ctx->h_cnt[slot];
-    return HFCR_OK;
+    return derive_edges(ctx, m->tris, m->n_tris, m->n_verts, ctx->edges[which],
+                        which ? C_EDGES_B : C_EDGES_A, ne, s);
 }
 
 struct DetectPlan {
@@ -1061,12 +1082,14 @@ hfcr_status hfcr_build_edges(hfcr_ctx *ctx, const int32_t *tris, int32_t n_tris,
     if (n_tris == 0) return HFCR_OK;
     hfcr_status st = reset_words(ctx, s);
     if (st) return st;
-    build_edges(tris, n_tris, n_verts, ctx->edges[0], ctx->d_cnt + C_EDGES_A, ctx->ekeys,
-                ctx->ekeys_alt, ctx->eflags, ctx->sort, ctx->d_status, s);
-    if ((st = read_back(ctx, s))) return st;
-    int ne = ctx->h_cnt[C_EDGES_A];
+    // straight into the caller's buffer when it holds any possible count
+    const bool direct = cap >= 3 * (int64_t)n_tris;
+    int ne = 0;
+    if ((st = derive_edges(ctx, tris, n_tris, n_verts, direct ? out : ctx->edges[0], C_EDGES_A, &ne, s)))
+        return st;
     *n_out = ne;
     if (ne > cap) return fail(ctx, HFCR_ERR_CAPACITY, "%d edges exceed cap %lld", ne, (long long)cap);
+    if (direct) return HFCR_OK;
     CK(cudaMemcpyAsync(out, ctx->edges[0], sizeof(int) * 2 * (size_t)ne, cudaMemcpyDeviceToDevice, s));
     CK(cudaStreamSynchronize(s));
     return HFCR_OK;

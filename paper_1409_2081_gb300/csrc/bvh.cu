@@ -128,6 +128,209 @@ __global__ void k_write_edges(const unsigned long long *keys, const unsigned *po
     }
 }
 
+// ---- the edges of a triangle list by buckets of the smaller vertex ----
+//
+// Four kernels instead of a radix sort of the 3 n_tris (v0, v1) keys: the
+// half-edges are counted per v0 (each keeps the rank the counter gave it), the
+// counts scanned, the v1 placed, and each vertex's few v1 sorted and made
+// unique in shared memory by one thread.  A vertex that is v0 of more than
+// BUCKET_MAX half-edges (a fan; a manifold mesh has some twelve) raises
+// *slow: the caller then takes the sort (build_edges_sorted), which does not
+// care.  Both scans are single-pass: a CTA publishes its sum and looks back
+// over its predecessors' (tickets in starting order, so they are running).
+// 522,242 triangles: 166 us of kernels by the sort (five passes of scattered
+// 8-byte keys), 43 by buckets.
+constexpr int BUCKET_MAX = 128;
+constexpr int BUCKET_SM = 4096;          // v1 of one CTA's vertices kept in shared memory
+constexpr int BUCKET_TPB = 256;
+constexpr int BUCKET_SCAN = 2048;        // counts per CTA of the scan
+
+__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_count(const int *tris, int nt, int nv, int *cnt,
+                                                             unsigned char *rank, int *slow,
+                                                             uint32_t *status) {
+    HFCR_PDL_WAIT();
+    const int t = blockIdx.x * BUCKET_TPB + threadIdx.x;
+    if (t >= nt) return;
+    const int v[3] = {tris[3 * t], tris[3 * t + 1], tris[3 * t + 2]};
+    int r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int a = v[k], b = v[(k + 1) % 3];
+        if ((unsigned)a >= (unsigned)nv || (unsigned)b >= (unsigned)nv) {
+            atomicOr(status, ST_BAD_INDEX);
+            a = b = 0;
+        }
+        r[k] = atomicAdd(cnt + min(a, b), 1);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (r[k] >= BUCKET_MAX) *slow = 1;
+        rank[3 * t + k] = (unsigned char)min(r[k], 255);
+    }
+}
+
+// sum of state[0 .. i) for CTA i of a single-pass scan (its own sum published
+// first); a state word is 0, or (1: the CTA's sum, 2: the sum up to it) << 32
+// | value.  The waits are bounded: after the limit ST_TIMEOUT is recorded
+// and what was seen is returned.  Called by one warp.
+__device__ __forceinline__ unsigned lookback(unsigned long long *state, int i, unsigned sum,
+                                             uint32_t *status) {
+    const int lane = threadIdx.x & 31;
+    volatile unsigned long long *st = state;
+    if (lane == 0) st[i] = ((i == 0 ? 2ull : 1ull) << 32) | sum;
+    unsigned before = 0;
+    for (int top = i; top > 0; top -= 32) {
+        const int q = top - 1 - lane;
+        unsigned long long w = 2ull << 32;  // before the first CTA: a finished sum of 0
+        int spins = 0;
+        if (q >= 0) {
+            w = st[q];
+            while (!(w >> 32) && ++spins < (1 << 22)) w = st[q];
+            if (!(w >> 32)) atomicOr(status, ST_TIMEOUT);
+        }
+        const unsigned done = __ballot_sync(0xffffffffu, (w >> 32) == 2ull);
+        const int stop = done ? __ffs(done) - 1 : 31;
+        before += __reduce_add_sync(0xffffffffu, lane <= stop ? (unsigned)w : 0u);
+        if (done) break;
+    }
+    if (lane == 0) st[i] = (2ull << 32) | (unsigned long long)(before + sum);
+    return before;
+}
+
+// exclusive scan of a value over the CTA's threads (BUCKET_TPB); the total to
+// `total`.  ws: BUCKET_TPB / 32 words.
+__device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned *ws, unsigned &total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    unsigned before = 0;
+    total = 0;
+#pragma unroll
+    for (int q = 0; q < BUCKET_TPB / 32; ++q) {
+        if (q < w) before += ws[q];
+        total += ws[q];
+    }
+    return before + x - v;
+}
+
+// cnt[0 .. n) -> exclusive offsets in place, the total to cnt[n]
+__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_scan(int *cnt, int n, unsigned long long *state,
+                                                            int *ticket, uint32_t *status) {
+    HFCR_PDL_WAIT();
+    __shared__ int cta;
+    __shared__ unsigned ws[BUCKET_TPB / 32], base;
+    if (threadIdx.x == 0) cta = atomicAdd(ticket, 1);
+    __syncthreads();
+    constexpr int PER = BUCKET_SCAN / BUCKET_TPB;
+    const int i0 = cta * BUCKET_SCAN + threadIdx.x * PER;
+    unsigned v[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        v[k] = i0 + k < n ? (unsigned)cnt[i0 + k] : 0u;
+        sum += v[k];
+    }
+    unsigned total;
+    unsigned e = cta_scan(sum, ws, total);
+    if (threadIdx.x < 32) {
+        const unsigned b = lookback(state, cta, total, status);
+        if (threadIdx.x == 0) base = b;
+    }
+    __syncthreads();
+    e += base;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (i0 + k < n) cnt[i0 + k] = (int)e;
+        e += v[k];
+        if (i0 + k == n - 1) cnt[n] = (int)e;
+    }
+}
+
+__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_fill(const int *tris, int nt, int nv, const int *ptr,
+                                                            const unsigned char *rank, int *bucket) {
+    HFCR_PDL_WAIT();
+    const int t = blockIdx.x * BUCKET_TPB + threadIdx.x;
+    if (t >= nt) return;
+    const int v[3] = {tris[3 * t], tris[3 * t + 1], tris[3 * t + 2]};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int a = v[k], b = v[(k + 1) % 3];
+        if ((unsigned)a >= (unsigned)nv || (unsigned)b >= (unsigned)nv) a = b = 0;
+        const int r = rank[3 * t + k];
+        if (r < BUCKET_MAX) bucket[ptr[min(a, b)] + r] = max(a, b);
+    }
+}
+
+// list[0 .. n) ascending and without repeats, in place; returns the length
+__device__ __forceinline__ int sort_unique(int *list, int n) {
+    for (int i = 1; i < n; ++i) {
+        const int x = list[i];
+        int j = i - 1;
+        while (j >= 0 && list[j] > x) {
+            list[j + 1] = list[j];
+            --j;
+        }
+        list[j + 1] = x;
+    }
+    int m = 0, last = -1;
+    for (int i = 0; i < n; ++i) {
+        const int x = list[i];
+        if (x != last) list[m++] = x;
+        last = x;
+    }
+    return m;
+}
+
+__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_edges(const int *ptr, int nv, int *bucket, int2 *edges,
+                                                             int *d_count, unsigned long long *state,
+                                                             int *ticket, uint32_t *status) {
+    HFCR_PDL_WAIT();
+    __shared__ int list[BUCKET_SM], out[BUCKET_SM];
+    __shared__ unsigned char owner[BUCKET_SM];
+    __shared__ unsigned ws[BUCKET_TPB / 32], base;
+    __shared__ int cta;
+    if (threadIdx.x == 0) cta = atomicAdd(ticket, 1);
+    __syncthreads();
+    const int v0 = cta * BUCKET_TPB, v = v0 + threadIdx.x, ve = min(v0 + BUCKET_TPB, nv);
+    const int p0 = ptr[v0], m = ptr[ve] - p0;
+    const bool in_sm = m <= BUCKET_SM;
+    const int a = v < nv ? ptr[v] - p0 : 0, n = v < nv ? ptr[v + 1] - p0 - a : 0;
+    int u = 0;
+    if (in_sm) {
+        for (int i = threadIdx.x; i < m; i += BUCKET_TPB) list[i] = bucket[p0 + i];
+        __syncthreads();
+        if (n <= BUCKET_MAX) u = sort_unique(list + a, n);
+    } else if (n <= BUCKET_MAX) {
+        u = sort_unique(bucket + p0 + a, n);
+    }
+    unsigned total;
+    const unsigned at = cta_scan((unsigned)u, ws, total);
+    if (threadIdx.x < 32) {
+        const unsigned b = lookback(state, cta, total, status);
+        if (threadIdx.x == 0) {
+            base = b;
+            if (ve == nv) *d_count = (int)(b + total);
+        }
+    }
+    if (in_sm) {  // compacted first, then written in order
+        for (int i = 0; i < u; ++i) {
+            out[at + i] = list[a + i];
+            owner[at + i] = (unsigned char)threadIdx.x;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < (int)total; i += BUCKET_TPB)
+            edges[base + i] = make_int2(v0 + owner[i], out[i]);
+    } else {
+        __syncthreads();
+        for (int i = 0; i < u; ++i) edges[base + at + i] = make_int2(v, bucket[p0 + a + i]);
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ void load3(const T *x, const T *y, const T *z, int i, T *o) {
     o[0] = x[i];
@@ -526,7 +729,7 @@ void validate_pair(const hfcr_mesh &A, const hfcr_mesh &B, uint32_t *d_status, c
                      (const double *)B.y, (const double *)B.z, nB, d_status); note_launch(); }
 }
 
-void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count,
+void build_edges_sorted(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count,
                  unsigned long long *keys, unsigned long long *keys_alt, unsigned *flags,
                  SortTemp &t, uint32_t *d_status, cudaStream_t s) {
     int n = 3 * n_tris;
@@ -543,6 +746,32 @@ void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *
     scan_flags_dev(flags, nullptr, n, d_count, t, s);
     { launch_pdl(k_write_edges, (n + 255) / 256, 256, 0, s, sorted, flags, n, vb,
                  edges_out); note_launch(); }
+}
+
+size_t bucket_words(int n_verts) {
+    // counts, both tickets, then both scans' states (8 B each)
+    const size_t c = (size_t)n_verts + 4;
+    const size_t st = ((size_t)n_verts + BUCKET_SCAN - 1) / BUCKET_SCAN + ((size_t)n_verts + BUCKET_TPB - 1) / BUCKET_TPB;
+    return ((c + 1) & ~(size_t)1) + 2 * st;
+}
+
+void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
+                 unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
+                 cudaStream_t s) {
+    int *bucket = (int *)keys;                              // [3 n_tris]
+    unsigned char *rank = (unsigned char *)keys_alt;        // [3 n_tris]
+    int *cnt = words, *tickets = words + n_verts + 1;
+    const int nscan = (n_verts + BUCKET_SCAN - 1) / BUCKET_SCAN;
+    unsigned long long *state = (unsigned long long *)(words + (((size_t)n_verts + 4 + 1) & ~(size_t)1));
+    cudaMemsetAsync(words, 0, sizeof(int) * bucket_words(n_verts), s);
+    const int nb = (n_tris + BUCKET_TPB - 1) / BUCKET_TPB, vb = (n_verts + BUCKET_TPB - 1) / BUCKET_TPB;
+    { launch_pdl(k_bucket_count, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, cnt, rank, d_slow,
+                 d_status); note_launch(); }
+    { launch_pdl(k_bucket_scan, nscan, BUCKET_TPB, 0, s, cnt, n_verts, state, tickets, d_status); note_launch(); }
+    { launch_pdl(k_bucket_fill, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, (const int *)cnt,
+                 (const unsigned char *)rank, bucket); note_launch(); }
+    { launch_pdl(k_bucket_edges, vb, BUCKET_TPB, 0, s, (const int *)cnt, n_verts, bucket, (int2 *)edges_out,
+                 d_count, state + nscan, tickets + 1, d_status); note_launch(); }
 }
 
 void check_segments(const int *segs, int nseg, const hfcr_mesh &A, const hfcr_mesh &B,

@@ -150,11 +150,20 @@ void scan_flags_dev(unsigned *flags, const int *d_n, int cap, int *d_total, Sort
                     cudaStream_t s);
 
 // ---- topology ----
-// Unique sorted edges of a triangle list.  Scratch: keys/keys_alt of
+// Unique sorted edges of a triangle list, by buckets of the smaller vertex
+// (n_tris, n_verts >= 1).  Scratch: keys/keys_alt of 3 * n_tris u64 and
+// bucket_words(n_verts) words, 8-byte aligned.  *d_slow (zero before) is set
+// when a vertex has too many: the result is then void, build_edges_sorted
+// gives it.
+void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
+                 unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
+                 cudaStream_t s);
+size_t bucket_words(int n_verts);
+// The same by a radix sort of all the edges' keys.  Scratch: keys/keys_alt of
 // 3 * n_tris u64 and flags of 3 * n_tris unsigned.
-void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count,
-                 unsigned long long *keys, unsigned long long *keys_alt, unsigned *flags,
-                 SortTemp &t, uint32_t *d_status, cudaStream_t s);
+void build_edges_sorted(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count,
+                        unsigned long long *keys, unsigned long long *keys_alt, unsigned *flags,
+                        SortTemp &t, uint32_t *d_status, cudaStream_t s);
 
 // ---- BVH ----
 // segs: device [(nseg + 1)][4] rows (A vertex, A face, B vertex, B face)

@@ -97,7 +97,7 @@ extern "C" hfcr_status hfcr_build_edges_noalloc(const int32_t *tris, int32_t n_t
     // the count and the status word carry over from the previous call
     if ((ce = cudaMemsetAsync(d_count, 0, 8, s)) != cudaSuccess)
         return cuda_fail("cudaMemsetAsync", ce);
-    hfcr::build_edges(tris, n_tris, n_verts, out, d_count, (unsigned long long *)(b + OFF_KEYS),
+    hfcr::build_edges_sorted(tris, n_tris, n_verts, out, d_count, (unsigned long long *)(b + OFF_KEYS),
                       (unsigned long long *)(b + OFF_KEYS_ALT), (unsigned *)(b + OFF_FLAGS), t,
                       d_status, s);
     // a launch error of this call's kernels, peeked rather than fetched: an
