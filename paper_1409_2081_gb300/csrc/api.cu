@@ -40,7 +40,8 @@ struct GraphEntry {
 // The small device words of one call (status, statistics, counters, solver
 // control words and scalars, the touched-vertex count): one allocation, so
 // that a call clears them with one memset and reads them back with one
-// copy into the pinned mirror of the same layout.
+// copy into the pinned mirror of the same layout.  On the device the words of
+// the stencil list's scan follow (scan_bytes, cleared too, not copied).
 struct DevWords {
     uint32_t status;
     uint32_t pad0;
@@ -52,6 +53,9 @@ struct DevWords {
     int pad1[3];
 };
 
+// the words of stencil_unique for lists of up to `pairs` keys
+static size_t scan_bytes(int64_t pairs) { return sizeof(int) * (2 + 2 * ((size_t)pairs / 1024 + 1)); }
+
 struct hfcr_ctx {
     hfcr_options opt;
     std::string err;
@@ -59,6 +63,7 @@ struct hfcr_ctx {
     int device = 0;
     DevWords *d_words = nullptr;  // the words below point into these two
     DevWords *h_words = nullptr;  // pinned mirror
+    int *scan_words() const { return (int *)(d_words + 1); }
     uint32_t *d_status = nullptr;
     DevStats *d_stats = nullptr;
     int *d_cnt = nullptr;         // [16] device counters
@@ -91,7 +96,6 @@ struct hfcr_ctx {
     unsigned *eflags = nullptr;
     unsigned long long *pkeys = nullptr, *pkeys_alt = nullptr;
     unsigned long long *skeys = nullptr, *skeys_alt = nullptr;
-    unsigned *sflags = nullptr;
     hfcr_stencil *stencils = nullptr;
     SolveBuffers sb;
     // diffusion (Sec. 5): vertex adjacency per mesh, float64 field ping-pong
@@ -153,7 +157,7 @@ cudaError_t dalloc(T **p, size_t n) {
 void free_all(hfcr_ctx *c) {
     void *ptrs[] = {c->d_words, c->sort.hist, c->edges[0], c->edges[1],
                     c->ekeys, c->ekeys_alt, c->eflags, c->pkeys, c->pkeys_alt,
-                    c->skeys, c->skeys_alt, c->sflags, c->stencils,
+                    c->skeys, c->skeys_alt, c->stencils,
                     c->sb.ids_raw, c->sb.n64_raw, c->sb.n32_raw, c->sb.b_raw, c->sb.parent,
                     c->sb.zkey, c->sb.zkey_alt, c->sb.szone, c->sb.zs, c->sb.zv, c->sb.d_nz,
                     c->sb.ck64, c->sb.ck64_alt, c->sb.gst, c->sb.zg, c->sb.d_ng, c->sb.pinv,
@@ -201,7 +205,7 @@ void free_all(hfcr_ctx *c) {
     c->edges[0] = c->edges[1] = nullptr;
     c->ekeys = c->ekeys_alt = nullptr; c->eflags = nullptr;
     c->pkeys = c->pkeys_alt = nullptr;
-    c->skeys = c->skeys_alt = nullptr; c->sflags = nullptr; c->stencils = nullptr;
+    c->skeys = c->skeys_alt = nullptr; c->stencils = nullptr;
     c->sb = SolveBuffers();
     c->h_status = nullptr; c->h_cnt = nullptr; c->h_stats = nullptr; c->h_dw = nullptr; c->h_iw = nullptr;
     c->h_segs = nullptr; c->d_segs = nullptr;
@@ -587,8 +591,8 @@ hfcr_status make_stencils(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B,
     bool flip = radix_sort_u64(ctx->skeys, nullptr, ctx->skeys_alt, nullptr, P, 1 + vb + fb,
                                ctx->sort, s);
     unsigned long long *sorted = flip ? ctx->skeys_alt : ctx->skeys;
-    stencil_unique(sorted, ctx->d_cnt + slot, P, vb, fb, ctx->sflags, out, ctx->d_cnt + C_STENCILS,
-                   ctx->sort, s);
+    stencil_unique(sorted, sorted, ctx->d_cnt + slot, P, vb, fb, out, ctx->d_cnt + C_STENCILS,
+                   ctx->scan_words(), ctx->d_status, s);
     prof_end(ctx, HFCR_STAGE_STENCILS, s);
     hfcr_status st = read_back(ctx, s);
     if (st) return st;
@@ -693,10 +697,11 @@ void enqueue_iteration(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bo
     stencil_keys_from_pair_keys(mp, ctx->pkeys, ctx->d_cnt + C_PAIRS, cap, pl.edges[0], pl.edges[1],
                                 pl.edge_bits, pl.face_bits, vb, fb, ctx->opt.f32_filter,
                                 ctx->skeys, ctx->d_cnt + C_PEFF, ctx->d_stats, ctx->d_status, s);
-    const bool flip = radix_sort_u64_dev(ctx->skeys, ctx->skeys_alt, ctx->d_cnt + C_PEFF, cap,
-                                         (d0 && d1 ? 1 : 0) + vb + fb, ctx->sort, s);
-    stencil_unique(flip ? ctx->skeys_alt : ctx->skeys, ctx->d_cnt + C_PEFF, cap, vb, fb, ctx->sflags,
-                   ctx->stencils, ctx->d_cnt + C_STENCILS, ctx->sort, s);
+    const int where = sort_by_rank_dev(ctx->skeys, ctx->skeys_alt, ctx->d_cnt + C_PEFF, cap,
+                                       (d0 && d1 ? 1 : 0) + vb + fb, ctx->sort, s);
+    stencil_unique(where == 1 ? ctx->skeys_alt : ctx->skeys, where ? ctx->skeys_alt : ctx->skeys,
+                   ctx->d_cnt + C_PEFF, cap, vb, fb, ctx->stencils, ctx->d_cnt + C_STENCILS,
+                   ctx->scan_words(), ctx->d_status, s);
     prof_end(ctx, HFCR_STAGE_STENCILS, s);
     if (!diffusing(ctx)) {
         run_response(ctx, A, B, ctx->stencils, cap, d, 1, nullptr, nullptr, s);
@@ -834,7 +839,7 @@ hfcr_status solve_info(hfcr_ctx *ctx, int k, hfcr_solve_info *info, cudaStream_t
 }
 
 hfcr_status reset_words(hfcr_ctx *ctx, cudaStream_t s) {
-    CK(cudaMemsetAsync(ctx->d_words, 0, sizeof(DevWords), s));
+    CK(cudaMemsetAsync(ctx->d_words, 0, sizeof(DevWords) + scan_bytes(ctx->max_pairs), s));
     return HFCR_OK;
 }
 
@@ -942,8 +947,8 @@ hfcr_status hfcr_reserve(hfcr_ctx *ctx, int64_t max_verts, int64_t max_tris, int
     if (max_tris < 1) max_tris = 1;
     if (max_pairs < 1) max_pairs = 1;
     const size_t T = (size_t)max_tris, P = (size_t)max_pairs, E3 = 3 * T;
-    CK(dalloc(&ctx->d_words, 1));
-    CK(cudaMemset(ctx->d_words, 0, sizeof(DevWords)));
+    CK(cudaMalloc((void **)&ctx->d_words, sizeof(DevWords) + scan_bytes(max_pairs)));
+    CK(cudaMemset(ctx->d_words, 0, sizeof(DevWords) + scan_bytes(max_pairs)));
     CK(cudaMallocHost((void **)&ctx->h_words, sizeof(DevWords)));
     memset(ctx->h_words, 0, sizeof(DevWords));
     ctx->d_status = &ctx->d_words->status;
@@ -984,7 +989,6 @@ hfcr_status hfcr_reserve(hfcr_ctx *ctx, int64_t max_verts, int64_t max_tris, int
     CK(dalloc(&ctx->pkeys_alt, P));
     CK(dalloc(&ctx->skeys, P));
     CK(dalloc(&ctx->skeys_alt, P));
-    CK(dalloc(&ctx->sflags, P));
     CK(dalloc(&ctx->stencils, P));
     {
         const size_t V = (size_t)max_verts;

@@ -13,6 +13,7 @@
 #include <stdint.h>
 
 #include "internal.h"
+#include "sortdev.cuh"
 
 namespace hfcr {
 
@@ -142,7 +143,7 @@ __global__ void k_write_edges(const unsigned long long *keys, const unsigned *po
 // 8-byte keys), 43 by buckets.
 constexpr int BUCKET_MAX = 128;
 constexpr int BUCKET_SM = 4096;          // v1 of one CTA's vertices kept in shared memory
-constexpr int BUCKET_TPB = 256;
+constexpr int BUCKET_TPB = TPB;
 constexpr int BUCKET_SCAN = 2048;        // counts per CTA of the scan
 
 __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_count(const int *tris, int nt, int nv, int *cnt,
@@ -167,56 +168,6 @@ __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_count(const int *tris, in
         if (r[k] >= BUCKET_MAX) *slow = 1;
         rank[3 * t + k] = (unsigned char)min(r[k], 255);
     }
-}
-
-// sum of state[0 .. i) for CTA i of a single-pass scan (its own sum published
-// first); a state word is 0, or (1: the CTA's sum, 2: the sum up to it) << 32
-// | value.  The waits are bounded: after the limit ST_TIMEOUT is recorded
-// and what was seen is returned.  Called by one warp.
-__device__ __forceinline__ unsigned lookback(unsigned long long *state, int i, unsigned sum,
-                                             uint32_t *status) {
-    const int lane = threadIdx.x & 31;
-    volatile unsigned long long *st = state;
-    if (lane == 0) st[i] = ((i == 0 ? 2ull : 1ull) << 32) | sum;
-    unsigned before = 0;
-    for (int top = i; top > 0; top -= 32) {
-        const int q = top - 1 - lane;
-        unsigned long long w = 2ull << 32;  // before the first CTA: a finished sum of 0
-        int spins = 0;
-        if (q >= 0) {
-            w = st[q];
-            while (!(w >> 32) && ++spins < (1 << 22)) w = st[q];
-            if (!(w >> 32)) atomicOr(status, ST_TIMEOUT);
-        }
-        const unsigned done = __ballot_sync(0xffffffffu, (w >> 32) == 2ull);
-        const int stop = done ? __ffs(done) - 1 : 31;
-        before += __reduce_add_sync(0xffffffffu, lane <= stop ? (unsigned)w : 0u);
-        if (done) break;
-    }
-    if (lane == 0) st[i] = (2ull << 32) | (unsigned long long)(before + sum);
-    return before;
-}
-
-// exclusive scan of a value over the CTA's threads (BUCKET_TPB); the total to
-// `total`.  ws: BUCKET_TPB / 32 words.
-__device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned *ws, unsigned &total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[w] = x;
-    __syncthreads();
-    unsigned before = 0;
-    total = 0;
-#pragma unroll
-    for (int q = 0; q < BUCKET_TPB / 32; ++q) {
-        if (q < w) before += ws[q];
-        total += ws[q];
-    }
-    return before + x - v;
 }
 
 // cnt[0 .. n) -> exclusive offsets in place, the total to cnt[n]

@@ -15,6 +15,7 @@
 
 #include "internal.h"
 #include "predicates.cuh"
+#include "sortdev.cuh"
 
 namespace hfcr {
 
@@ -468,29 +469,57 @@ __global__ void k_stencil_keys_from_pair_keys(hfcr_mesh A, hfcr_mesh B,
                                 f32_filter, st, status);
 }
 
-__global__ void k_stencil_flags(const unsigned long long *keys, const int *d_n, int cap,
-                                unsigned *flags) {
-    HFCR_PDL_WAIT();
-    int n = min(*d_n, cap);
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flags[i] = (i == 0 || keys[i] != keys[i - 1]) ? 1u : 0u;
-}
+// sorted keys -> the list of distinct ones, their number to *d_k: one
+// single-pass scan (lookback), UNIQUE_KEYS keys per CTA, in the place of flags,
+// their two-kernel scan and the write
+constexpr int UNIQUE_KEYS = 1024;
 
-__global__ void k_stencil_write(const unsigned long long *keys, const unsigned *pos,
-                                const int *d_n, int cap, int vert_bits, int face_bits,
-                                hfcr_stencil *out) {
+__global__ void __launch_bounds__(TPB) k_stencil_unique(const unsigned long long *many,
+                                                        const unsigned long long *few, const int *d_n, int cap,
+                                                        int vert_bits, int face_bits, hfcr_stencil *out, int *d_k,
+                                                        int *ticket, unsigned long long *state,
+                                                        uint32_t *status) {
     HFCR_PDL_WAIT();
-    int n = min(*d_n, cap);
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (i == 0 || keys[i] != keys[i - 1]) {
-        unsigned long long k = keys[i];
+    const int n = min(*d_n, cap);
+    const unsigned long long *keys = n <= RANK_MAX ? few : many;
+    __shared__ int cta;
+    __shared__ unsigned ws[TPB / 32], base;
+    if ((int)blockIdx.x * UNIQUE_KEYS >= n) {  // nothing for it (the tickets below are the others')
+        if (blockIdx.x == 0 && threadIdx.x == 0) *d_k = 0;
+        return;
+    }
+    if (threadIdx.x == 0) cta = atomicAdd(ticket, 1);
+    __syncthreads();
+    constexpr int PER = UNIQUE_KEYS / TPB;
+    const int i0 = cta * UNIQUE_KEYS + threadIdx.x * PER;
+    unsigned long long k[PER + 1];
+    k[0] = i0 > 0 && i0 <= n ? keys[i0 - 1] : ~0ull;  // no key has every bit set
+#pragma unroll
+    for (int q = 0; q < PER; ++q) k[q + 1] = i0 + q < n ? keys[i0 + q] : k[q];
+    unsigned sum = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) sum += k[q + 1] != k[q];
+    unsigned total;
+    unsigned at = cta_scan(sum, ws, total);
+    if (threadIdx.x < 32) {
+        const unsigned b = lookback(state, cta, total, status);
+        if (threadIdx.x == 0) {
+            base = b;
+            if ((cta + 1) * UNIQUE_KEYS >= n) *d_k = (int)(b + total);
+        }
+    }
+    __syncthreads();
+    at += base;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        if (k[q + 1] == k[q]) continue;
+        const unsigned long long v = k[q + 1];
         hfcr_stencil s;
-        s.dir = (unsigned)(k >> (vert_bits + face_bits));
-        s.x0 = (unsigned)((k >> face_bits) & ((1ull << vert_bits) - 1));
-        s.face = (unsigned)(k & ((1ull << face_bits) - 1));
+        s.dir = (unsigned)(v >> (vert_bits + face_bits));
+        s.x0 = (unsigned)((v >> face_bits) & ((1ull << vert_bits) - 1));
+        s.face = (unsigned)(v & ((1ull << face_bits) - 1));
         s.pad = 0;
-        out[pos[i]] = s;
+        out[at++] = s;
     }
 }
 
@@ -626,15 +655,13 @@ void stencil_keys_from_pair_keys(const MeshPair &mp, const unsigned long long *p
     note_launch();
 }
 
-void stencil_unique(const unsigned long long *keys, const int *d_n, int cap, int vert_bits,
-                    int face_bits, unsigned *flags, hfcr_stencil *out, int *d_k, SortTemp &t,
-                    cudaStream_t s) {
+void stencil_unique(const unsigned long long *keys, const unsigned long long *few, const int *d_n, int cap,
+                    int vert_bits, int face_bits, hfcr_stencil *out, int *d_k, int *words,
+                    uint32_t *d_status, cudaStream_t s) {
     if (cap <= 0) return;
-    int nb = (cap + 255) / 256;
-    { launch_pdl(k_stencil_flags, nb, 256, 0, s, keys, d_n, cap, flags); note_launch(); }
-    scan_flags_dev(flags, d_n, cap, d_k, t, s);
-    { launch_pdl(k_stencil_write, nb, 256, 0, s, keys, flags, d_n, cap, vert_bits, face_bits,
-                 out); note_launch(); }
+    { launch_pdl(k_stencil_unique, (cap + UNIQUE_KEYS - 1) / UNIQUE_KEYS, TPB, 0, s, keys, few, d_n, cap,
+                 vert_bits, face_bits, out, d_k, words, (unsigned long long *)(words + 2), d_status);
+      note_launch(); }
 }
 
 }  // namespace hfcr

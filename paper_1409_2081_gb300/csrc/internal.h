@@ -134,6 +134,12 @@ bool radix_sort_u32_dev(unsigned *k0, int *v0, unsigned *k1, int *v1, const int 
                         int bits, SortTemp &t, cudaStream_t s);
 bool radix_sort_u64v_dev(unsigned long long *k0, int *v0, unsigned long long *k1, int *v1,
                          const int *d_n, int cap, int bits, SortTemp &t, cudaStream_t s);
+// The same for keys that a consumer reads by place: 1 when the result is in
+// k1, 0 when in k0, 2 when it is in k1 for at most RANK_MAX_KEYS keys and in
+// k0 for more.
+int sort_by_rank_dev(unsigned long long *k0, unsigned long long *k1, const int *d_n, int cap, int bits,
+                     SortTemp &t, cudaStream_t s);
+constexpr int RANK_MAX_KEYS = 8192;
 // keys of a batch grouped by segment (segment number in the bits above
 // seg_bits): one CTA sorts each segment over its low seg_bits bits; if a
 // segment is longer than one CTA sorts, *d_rest (scratch) routes the whole
@@ -233,10 +239,12 @@ void stencil_keys_from_pair_keys(const MeshPair &mp, const unsigned long long *p
 void stencil_keys(const MeshPair &mp, const hfcr_pair *pairs, const int *d_n, int cap,
                   int vert_bits, int face_bits, int f32_filter, unsigned long long *keys,
                   DevStats *stats, uint32_t *d_status, cudaStream_t s);
-// sorted keys -> unique stencils, count to d_k
-void stencil_unique(const unsigned long long *keys, const int *d_n, int cap, int vert_bits,
-                    int face_bits, unsigned *flags, hfcr_stencil *out, int *d_k, SortTemp &t,
-                    cudaStream_t s);
+// sorted keys -> unique stencils, count to d_k.  few: where the keys are when
+// there are at most RANK_MAX_KEYS of them.  words: [2 + 2 * (cap / 1024 + 1)],
+// zero before, 8-byte aligned.
+void stencil_unique(const unsigned long long *keys, const unsigned long long *few, const int *d_n, int cap,
+                    int vert_bits, int face_bits, hfcr_stencil *out, int *d_k, int *words,
+                    uint32_t *d_status, cudaStream_t s);
 
 // ---- solver ----
 struct SolveBuffers {

@@ -1,10 +1,12 @@
 // Stable LSD radix sort (8-bit digits) and exclusive scans; the tile
 // ranking, the CTA scan, the single-CTA and grid-wide sort bodies and the
-// grid barrier are in sortdev.cuh.  Inputs of up to SMALL_N keys are
-// sorted by one CTA that walks its tiles in order (one launch for all
-// passes).  A sort whose count only the device knows launches that CTA and
-// one cooperative kernel that runs every multi-CTA pass when the count is
-// larger; the segments of a batch can be sorted one CTA each.
+// grid barrier are in sortdev.cuh.  Inputs of up to RANK_MAX keys whose
+// count the host knows are sorted by ranks.  A sort whose count only the
+// device knows launches one CTA that sorts up to SMALL_N keys, walking its
+// tiles in order, and one cooperative kernel that runs every multi-CTA pass
+// when the count is larger (sort_by_rank_dev: the cooperative kernel alone,
+// by ranks up to RANK_MAX keys); the segments of a batch can be sorted one
+// CTA each.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -224,21 +226,37 @@ __global__ void __launch_bounds__(TPB) k_sort_segments(K *k0, int *v0, K *k1, in
 // (every CTA reads the same count before any barrier, so none waits alone).  Data written by other
 // CTAs in the same launch (keys, histogram rows, digit totals) is read with
 // L2 loads (__ldcg), never through a possibly stale L1 line.
-template <typename K, bool HV>
+// RANKS: up to RANK_MAX keys are sorted here too, by ranks, into k1.
+template <typename K, bool HV, bool RANKS = false>
 __global__ void __launch_bounds__(TPB) k_sort_coop(K *k0, int *v0, K *k1, int *v1, int n,
                                                    const int *d_n, int bits, unsigned *hist,
                                                    unsigned *tot, unsigned *bar, uint32_t *status) {
     HFCR_PDL_WAIT();
     if (d_n) n = min(n, *d_n);
-    if (n <= SMALL_N) return;
+    __shared__ union { SortSmem sort; K tile[RANK_TILE]; } shm;
+    if constexpr (RANKS) {
+        if (n <= RANK_MAX) {
+            rank_sort_body<K, HV>(k0, v0, k1, v1, n, shm.tile);
+            return;
+        }
+    } else if (n <= SMALL_N) {
+        return;
+    }
     unsigned epoch = 0;
-    __shared__ SortSmem sm;
+    SortSmem &sm = shm.sort;
     sort_grid_body<K, HV>(k0, v0, k1, v1, n, bits, hist, tot, bar, epoch, status, sm);
+}
+
+template <typename K, bool HV>
+__global__ void __launch_bounds__(TPB) k_rank(const K *kin, const int *vin, K *kout, int *vout, int n) {
+    HFCR_PDL_WAIT();
+    __shared__ K tile[RANK_TILE];
+    rank_sort_body<K, HV>(kin, vin, kout, vout, n, tile);
 }
 
 // co-resident CTAs of k_sort_coop<K, HV> on this device (0: cooperative
 // launch unavailable)
-template <typename K, bool HV>
+template <typename K, bool HV, bool RANKS = false>
 int coop_grid() {
     static int g[64] = {0};
     static bool done[64] = {false};
@@ -246,7 +264,7 @@ int coop_grid() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     if (!done[dev]) {
         int per_sm = 0, sms = 0, coop = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_coop<K, HV>, TPB, 0) ==
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_coop<K, HV, RANKS>, TPB, 0) ==
                 cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop)
@@ -264,12 +282,17 @@ bool radix_sort_impl(K *k0, int *v0, K *k1, int *v1, int n, const int *d_n, int 
     // n: the element count (d_n == null) or an upper bound of *d_n
     int passes = (bits + 7) / 8;
     if (n <= 0 || passes == 0) return false;
-    if (n <= SMALL_N || d_n) {
+    if (!d_n && n <= RANK_MAX) {
+        { launch_pdl(k_rank<K, HV>, (n + RANK_KEYS - 1) / RANK_KEYS, TPB, 0, s, (const K *)k0,
+                     (const int *)v0, k1, v1, n); note_launch(); }
+        return true;
+    }
+    if (d_n) {
         // with a device count the single CTA sorts whenever *d_n <= SMALL_N
         // and the multi-CTA kernels below return at once; otherwise the reverse
         { launch_pdl(k_sort_small<K, HV>, 1, TPB, 0, s, k0, v0, k1, v1, n, d_n,
                      passes * 8); note_launch(); }
-        if (n <= SMALL_N) return passes & 1;
+        if (n <= SMALL_N) return passes & 1;  // the bound already fits
     }
     int nb = (n + TILE - 1) / TILE;
     // the digit totals sit in the spare row after the largest histogram
@@ -349,6 +372,32 @@ bool radix_sort_u64v_dev(unsigned long long *k0, int *v0, unsigned long long *k1
 bool radix_sort_u32_dev(unsigned *k0, int *v0, unsigned *k1, int *v1, const int *d_n, int cap,
                         int bits, SortTemp &t, cudaStream_t s) {
     return radix_sort_impl<unsigned, true>(k0, v0, k1, v1, cap, d_n, bits, t, s);
+}
+
+int sort_by_rank_dev(unsigned long long *k0, unsigned long long *k1, const int *d_n, int cap, int bits,
+                     SortTemp &t, cudaStream_t s) {
+    typedef unsigned long long K;
+    const int passes = (bits + 7) / 8;
+    int grid = coop_grid<K, false, true>();
+    const int nb = (cap + TILE - 1) / TILE, nr = ((cap < RANK_MAX ? cap : RANK_MAX) + RANK_KEYS - 1) / RANK_KEYS;
+    const int want = nb > nr ? nb : nr;
+    if (grid > want) grid = want;
+    if (cap > 0 && passes > 0 && grid > 0 && t.status) {
+        K *a = k0, *b = k1;
+        int *none = nullptr, n = cap, bits8 = passes * 8;
+        unsigned *tot = t.hist + 256 * (size_t)(t.max_blocks - 1);
+        unsigned *bar = t.hist + 256 * (size_t)(t.max_blocks - 2);
+        uint32_t *status = t.status;
+        cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
+        void *args[] = {&a, &none, &b, &none, &n, (void *)&d_n, &bits8, &t.hist, &tot, &bar, &status};
+        if (cudaLaunchCooperativeKernel((const void *)k_sort_coop<K, false, true>, grid, TPB, args, 0, s) ==
+            cudaSuccess) {
+            note_launch();
+            return (passes & 1) ? 1 : 2;
+        }
+        cudaGetLastError();
+    }
+    return radix_sort_u64_dev(k0, k1, d_n, cap, bits, t, s) ? 1 : 0;
 }
 
 void scan_flags_dev(unsigned *flags, const int *d_n, int cap, int *d_total, SortTemp &t,

@@ -202,6 +202,109 @@ __device__ __forceinline__ void sort_small_body(K *k0, int *v0, K *k1, int *v1, 
     }
 }
 
+// sum of state[0 .. i) for CTA i of a single-pass scan (its own sum published
+// first); a state word is 0, or (1: the CTA's sum, 2: the sum up to it) << 32
+// | value.  The waits are bounded: after the limit ST_TIMEOUT is recorded
+// and what was seen is returned.  Called by one warp.
+__device__ __forceinline__ unsigned lookback(unsigned long long *state, int i, unsigned sum,
+                                             uint32_t *status) {
+    const int lane = threadIdx.x & 31;
+    volatile unsigned long long *st = state;
+    if (lane == 0) st[i] = ((i == 0 ? 2ull : 1ull) << 32) | sum;
+    unsigned before = 0;
+    for (int top = i; top > 0; top -= 32) {
+        const int q = top - 1 - lane;
+        unsigned long long w = 2ull << 32;  // before the first CTA: a finished sum of 0
+        int spins = 0;
+        if (q >= 0) {
+            w = st[q];
+            while (!(w >> 32) && ++spins < (1 << 22)) w = st[q];
+            if (!(w >> 32)) atomicOr(status, ST_TIMEOUT);
+        }
+        const unsigned done = __ballot_sync(0xffffffffu, (w >> 32) == 2ull);
+        const int stop = done ? __ffs(done) - 1 : 31;
+        before += __reduce_add_sync(0xffffffffu, lane <= stop ? (unsigned)w : 0u);
+        if (done) break;
+    }
+    if (lane == 0) st[i] = (2ull << 32) | (unsigned long long)(before + sum);
+    return before;
+}
+
+// exclusive scan of a value over the CTA's threads (TPB); the total to
+// `total`.  ws: TPB / 32 words.
+__device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned *ws, unsigned &total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    unsigned before = 0;
+    total = 0;
+#pragma unroll
+    for (int q = 0; q < TPB / 32; ++q) {
+        if (q < w) before += ws[q];
+        total += ws[q];
+    }
+    return before + x - v;
+}
+
+// Stable sort by ranks, for n of at most RANK_MAX keys: a key's place is the
+// number of smaller ones, and of equal ones before it.  n^2 comparisons from
+// shared memory by every CTA of the grid, two keys per 16 threads, instead of
+// one CTA's passes over the digits (2,732 keys: 32 us by the single CTA, 7
+// by ranks); past RANK_MAX the multi-CTA passes win.  From kin to kout.
+constexpr int RANK_MAX = RANK_MAX_KEYS;
+constexpr int RANK_TILE = 1024;
+constexpr int RANK_KEYS = TPB / 16 * 2;  // keys of a CTA at a time
+
+template <typename K, bool HV>
+__device__ __forceinline__ void rank_sort_body(const K *kin, const int *vin, K *kout, int *vout, int n,
+                                               K *tile) {
+    const int sub = threadIdx.x & 15;
+    for (int kb = blockIdx.x * RANK_KEYS; kb < n; kb += gridDim.x * RANK_KEYS) {
+        const int i = kb + (threadIdx.x >> 4) * 2;
+        const K a = i < n ? kin[i] : (K)0, b = i + 1 < n ? kin[i + 1] : (K)0;
+        unsigned ra = 0, rb = a == b ? (sub == 0) : 0;  // key i counts before an equal key i + 1
+        for (int tb = 0; tb < n; tb += RANK_TILE) {
+            const int len = min(RANK_TILE, n - tb);
+            __syncthreads();  // the last tile is read
+            for (int q = threadIdx.x; q < len; q += TPB) tile[q] = kin[tb + q];
+            __syncthreads();
+            const int mid = min(max(i - tb, 0), len);  // keys before i: equal ones count too
+            int q = sub;
+            for (; q < mid; q += 16) {
+                const K x = tile[q];
+                ra += x <= a;
+                rb += x <= b;
+            }
+            for (; q < len; q += 16) {
+                const K x = tile[q];
+                ra += x < a;
+                rb += x < b;
+            }
+        }
+#pragma unroll
+        for (int o = 8; o; o >>= 1) {
+            ra += __shfl_xor_sync(0xffffffffu, ra, o);
+            rb += __shfl_xor_sync(0xffffffffu, rb, o);
+        }
+        if (sub == 0) {
+            if (i < n) {
+                kout[ra] = a;
+                if (HV) vout[ra] = vin[i];
+            }
+            if (i + 1 < n) {
+                kout[rb] = b;
+                if (HV) vout[rb] = vin[i + 1];
+            }
+        }
+    }
+}
+
 // Grid-wide barrier: a monotone arrival counter (zeroed before the launch);
 // barrier number e is passed when it reaches e * parts, parts = the CTAs
 // taking part (gridDim.x unless given; CTAs beyond it must not call).  The

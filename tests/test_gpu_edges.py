@@ -2,7 +2,7 @@
 over: valences around the bucket limit of 128, a block of 256 vertices around
 what its shared memory holds (4,096 half-edges), fans, repeated and degenerate
 triangles, isolated vertices, more vertices than reserved, short output
-buffers.  Against numpy's sorted unique pairs."""
+buffers, and the sort's own change from ranks to passes at 8,192 keys.  Against numpy's sorted unique pairs."""
 import numpy as np
 import pytest
 
@@ -41,6 +41,8 @@ LISTS = {
     "one": np.array([[2, 0, 1]]),
     "degenerate": np.array([[0, 0, 0], [1, 1, 2], [2, 1, 1], [3, 4, 5], [5, 4, 3]]),
     "fan_64": fan(64), "fan_65": fan(65), "fan_5000": fan(5000),
+    # three keys a triangle into the sort: 8,190 by ranks, 8,193 by passes
+    "fan_2730": fan(2730), "fan_2731": fan(2731),
     "random": RNG.integers(0, 900, (3000, 3)),
     "dense_7": dense(RNG, 300, 7), "dense_8": dense(RNG, 256, 8), "dense_9": dense(RNG, 600, 9),
     "dense_60": dense(RNG, 300, 60),
