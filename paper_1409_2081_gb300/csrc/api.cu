@@ -124,7 +124,7 @@ struct hfcr_ctx {
 // device counter slots
 enum { C_PAIRS = 0, C_STENCILS = 1, C_EDGES_A = 2, C_EDGES_B = 3, C_N4 = 4, C_NPAIRS_IN = 5, C_PEFF = 6,
        C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 /* to 13: two words per direction */,
-       C_SLOW = 14 };
+       C_SLOW = 14, C_BAND_DONE = C_DIFF_ITERS + 8 /* the diffusion's ctl word 8 */ };
 
 namespace {
 

@@ -10,9 +10,9 @@
 //     deg(v) u_v - sum of u_w over band neighbours w
 //         = sum of the Dirichlet values of v's other neighbours
 // is solved for each coordinate, by Jacobi-preconditioned conjugate
-// gradients to a relative residual `tol` (k_band_cl on one thread-block
-// cluster for bands of up to some 27,000 vertices, k_band_cg over the whole
-// grid beyond).  The older fixed-sweep form (S Jacobi sweeps of
+// gradients to a relative residual `tol` (k_band_pipe and k_band_cl on one
+// thread-block cluster for bands of up to 15,360 and 22,528 vertices,
+// k_band_cg over the whole grid beyond).  The older fixed-sweep form (S Jacobi sweeps of
 // the neighbour mean from zero, whose limit is that field) stays available
 // as a named approximation.
 //
@@ -334,7 +334,8 @@ struct BandArgs {
     int eoffB;           //   mesh B from eoffB on
     double *part;        // [2][grid][9] per-CTA partial sums (doubles, or floats in the same space)
     unsigned *bar;       // grid barrier counter, zeroed before the launch
-    int *ctl;            // [0] CG iterations run, [1] set when a coordinate stopped unconverged
+    int *ctl;            // [0] CG iterations run, [1] set when a coordinate stopped unconverged,
+                         // [BAND_DONE] set when the pipelined kernel solved the band
     uint32_t *status;
     double tol;
     int max_iters;
@@ -771,7 +772,15 @@ __global__ void __launch_bounds__(BAND_TPB) k_band_cg(BandArgs a, int limit) {
 // barriers: nothing here spins.
 namespace cgx = cooperative_groups;
 
+// Of the cluster's CTAs only as many work as the band needs at BCL_PER vertices
+// each; the others leave at once (a cluster barrier waits for the threads
+// that have not exited), and a band of one CTA needs no cluster barrier.
 constexpr int BCL_THREADS = 1024;
+constexpr int BCL_PER = 256;                 // vertices of a CTA when fewer CTAs do
+constexpr int BAND_DONE = 8;                 // word of ctl set when the pipelined kernel solved the band
+constexpr int PIPE_RINGS = 8;
+constexpr float PIPE_TOL = 6e-6f;            // reduction of one pipelined round
+constexpr int PIPE_ITERS = 200;              // its iterations at most
 constexpr int BCL_MAX = 16;                  // CTAs per cluster at most
 constexpr int BCL_SMEM = 220 * 1024;  // dynamic shared memory per CTA
 constexpr int BCL_NB = 8;             // neighbour codes kept in shared memory per vertex
@@ -790,12 +799,90 @@ struct BclState {
     // set by thread 0, rather than in every thread's registers)
     float gam[3], alp[3], bet[3], stop[3];
     double target[3];
+    double before[3];  // |r|^2 at the start of a pipelined round
     int in;  // coordinates whose float32 run goes on (bit c)
     float scr[32 * 9];
     double scrd[32 * 3];
+    float cta[9];   // this CTA's sums, on their way
     float *recv_of[BCL_MAX];
     double *recvd_of[BCL_MAX];
 };
+
+// Nine sums over the warp by halving: a lane gives half of its eight values
+// away at each of three steps (4 + 2 + 1 shuffles), then two steps finish, and
+// the ninth takes five: 14 shuffles where nine butterflies and their
+// broadcast take 54 (an SM shuffles one warp per cycle, so 32 warps paid
+// 0.9 us an iteration).  Lane 4 k ends with sum k, lane 0 with sum 8 too; to
+// scr[9].
+__device__ __forceinline__ void warp_sums9(const float (&v)[9], float *scr) {
+    const int lane = threadIdx.x & 31;
+    float t[4], n8 = v[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float give = (lane & 16) ? v[k] : v[k + 4], keep = (lane & 16) ? v[k + 4] : v[k];
+        t[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float give = (lane & 8) ? t[k] : t[k + 2], keep = (lane & 8) ? t[k + 2] : t[k];
+        t[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+    {
+        const float give = (lane & 4) ? t[0] : t[1], keep = (lane & 4) ? t[1] : t[0];
+        t[0] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+#pragma unroll
+    for (int o = 2; o; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) n8 += __shfl_xor_sync(0xffffffffu, n8, o);
+    if ((lane & 3) == 0) scr[((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = t[0];
+    if (lane == 0) scr[8] = n8;
+}
+
+// Three float64 sums over the warp by halving (six additions instead of
+// fifteen: an SM adds two float64 lanes per cycle); to scr[3].
+__device__ __forceinline__ void warp_sums3(const double (&v)[3], double *scr) {
+    const int lane = threadIdx.x & 31;
+    double t[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {  // lanes with bit 16 keep v[2] (and nothing)
+        const double hi = k == 0 ? v[2] : 0.0;
+        const double give = (lane & 16) ? v[k] : hi, keep = (lane & 16) ? hi : v[k];
+        t[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+    const double give = (lane & 8) ? t[0] : t[1], keep = (lane & 8) ? t[1] : t[0];
+    double x = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const int k = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+    if ((lane & 7) == 0 && k < 3) scr[k] = x;
+}
+
+// One warp: the three sums over `rows` <= 20 rows of three; lane k < 3 ends
+// with sum k
+__device__ __forceinline__ double fold3(const double *rows3, int rows) {
+    const int lane = threadIdx.x & 31, q = lane / 3, k = lane % 3;
+    double t = lane < 30 && q < rows ? rows3[3 * q + k] : 0.0;
+    t += lane < 30 && q + 10 < rows ? rows3[3 * (q + 10) + k] : 0.0;
+    const double h = __shfl_down_sync(0xffffffffu, t, 15);
+    t += h;
+    const double a = __shfl_down_sync(0xffffffffu, t, 3), b = __shfl_down_sync(0xffffffffu, t, 6),
+                 c = __shfl_down_sync(0xffffffffu, t, 9), d = __shfl_down_sync(0xffffffffu, t, 12);
+    return ((t + a) + (b + c)) + d;
+}
+
+// One warp: the nine sums over `rows` <= 18 rows of nine; lane k < 9 ends with sum
+// k (lanes k, k + 9 and k + 18 add every third row)
+__device__ __forceinline__ float fold9(const float *rows9, int rows) {
+    const int lane = threadIdx.x & 31;
+    const int q0 = lane / 9;
+    float x[6];  // at most 18 rows: every load in flight
+#pragma unroll
+    for (int i = 0; i < 6; ++i) x[i] = lane < 27 && q0 + 3 * i < rows ? rows9[9 * (q0 + 3 * i) + lane % 9] : 0.f;
+    const float t = ((x[0] + x[1]) + (x[2] + x[3])) + (x[4] + x[5]);
+    const float a = __shfl_down_sync(0xffffffffu, t, 9), b = __shfl_down_sync(0xffffffffu, t, 18);
+    return t + a + b;
+}
 
 // K warp butterflies side by side (level by level, so the shuffles of the
 // K values overlap); every lane ends with lane 0's sums
@@ -817,7 +904,13 @@ __device__ __forceinline__ void warp_sums(T (&t)[K]) {
 // received sums in rank order (lane q holds CTA q's).  A parity's slots are
 // rewritten two calls later, after every CTA has passed the barrier that
 // follows its reads.
-template <typename T, int K, bool SYNC_END = true>
+// barrier of the CTAs that work
+__device__ __forceinline__ void bcl_sync(cgx::cluster_group &cl, int ncta) {
+    if (ncta > 1) cl.sync();
+    else __syncthreads();
+}
+
+template <typename T, int K, bool SYNC_END = true, int THREADS = BCL_THREADS>
 __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K], T *scr, T *recv,
                                          T *const *recv_of, int par, int rank, int ncta, T *out) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -832,7 +925,7 @@ __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K]
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) t[k] = lane < BCL_THREADS / 32 ? scr[lane * K + k] : (T)0;
+        for (int k = 0; k < K; ++k) t[k] = lane < THREADS / 32 ? scr[lane * K + k] : (T)0;
         warp_sums<T, K>(t);
         if (lane < ncta) {
             T *dst = recv_of[lane] + (par * BCL_MAX + rank) * K;
@@ -840,7 +933,7 @@ __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K]
             for (int k = 0; k < K; ++k) dst[k] = t[k];
         }
     }
-    cl.sync();  // every CTA's sums received
+    bcl_sync(cl, ncta);  // every CTA's sums received
     if (w == 0) {
 #pragma unroll
         for (int k = 0; k < K; ++k) t[k] = lane < ncta ? recv[(par * BCL_MAX + lane) * K + k] : (T)0;
@@ -867,35 +960,15 @@ __device__ __forceinline__ void bcl_codes(const int4 *cq, const int *cnbr, int l
     }
 }
 
-__global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limit) {
-    constexpr int vcap = BCL_VCAP;
-    HFCR_PDL_WAIT();
-    cgx::cluster_group cl = cgx::this_cluster();
-    const int n = *a.d_nfree;
-    if (n > limit) return;  // the grid kernel's band (the same n in every CTA)
-    extern __shared__ float4 bsm[];
-    __shared__ BclState st;
-    const int ncta = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    const int chunk = n > 0 ? (n + ncta - 1) / ncta : 1;
-    const int lo = rank * chunk;
-    const int cnt = n - lo < chunk ? (n - lo > 0 ? n - lo : 0) : chunk;
-    float4 *rq = bsm;  // r (x, y, z) and 1 / deg
-    float4 *gz = (float4 *)a.rec;  // z of every band vertex, for the other CTAs
-    double *gu = a.u64;            // u of every band vertex
-    float4 *pq = rq + vcap, *sq = pq + vcap, *xq = sq + vcap, *wq = xq + vcap;
-    float4 *zq = wq + vcap;
-    int4 *cq = (int4 *)(zq + vcap);  // two int4 (BCL_NB codes) per vertex
-    double *uq = (double *)(cq + 2 * (size_t)vcap);  // u (x, y, z) of the rounds
-    int2 *ed = (int2 *)(uq + 3 * (size_t)vcap);
-    if ((int)threadIdx.x < ncta) {
-        st.recv_of[threadIdx.x] = cl.map_shared_rank(&st.recv[0][0][0], threadIdx.x);
-        st.recvd_of[threadIdx.x] = cl.map_shared_rank(&st.recvd[0][0][0], threadIdx.x);
-    }
-    // the right-hand side (Dirichlet values of the neighbours outside the
-    // band), the neighbours' record addresses, the first round's state
-    // (r = b, u = 0)
-    double dl[3] = {0.0, 0.0, 0.0};
-    for (int li = threadIdx.x; li < cnt; li += BCL_THREADS) {
+// the band vertices lo .. lo + cnt of one CTA: the right-hand side (Dirichlet
+// values of the neighbours outside the band) to b64, and in shared memory
+// r = b with 1 / deg, the neighbour codes, the slot range and u = 0; adds |b|^2
+// to dl
+template <int THREADS>
+__device__ __forceinline__ void bcl_setup(const BandArgs &a, int lo, int cnt, int chunk, int rank, float4 *rq,
+                                          int4 *cq, double *uq, int2 *ed, double *dl) {
+    if ((int)threadIdx.x >= THREADS) return;  // not a thread with vertices
+    for (int li = threadIdx.x; li < cnt; li += THREADS) {
         const int i = lo + li;
         const int g = a.fv[i];
         const bool inB = g >= a.P.m[1].off;
@@ -929,17 +1002,416 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
         // a band vertex has a neighbour one ring closer, so e1 > e0
         ed[li] = make_int2(s0, e1 - e0);
         rq[li] = make_float4((float)b[0], (float)b[1], (float)b[2], 1.0f / (float)(e1 - e0));
-        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        pq[li] = z4;
-        sq[li] = z4;
-        xq[li] = z4;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             a.b64[3 * (size_t)i + c] = b[c];
             uq[3 * li + c] = 0.0;
-            gu[3 * (size_t)i + c] = 0.0;
             dl[c] += b[c] * b[c];
         }
+    }
+}
+
+// ---- the pipelined form on the cluster ----
+//
+// Bands of up to PIPE_MAX vertices of up to PIPE_RINGS rings, by the same rounds
+// with pipelined iterations (Ghysels and Vanroose 2014): the recurrences carry
+// u = M^-1 r, w = L u and their images under M^-1 and L M^-1, so that an
+// iteration publishes m = M^-1 w and its sums together and has one cluster
+// barrier instead of two; a warp of its own folds the sums beside the gather
+// of L m.  512 threads a CTA, up to two vertices each: a vertex's recurrences and
+// packed neighbour codes live in registers (1,024 threads have 64 each and
+// spill, and with this much shared memory the spills go to L2).
+// In float32 the recurrences are good to a reduction of a few 1e-6 on narrow
+// bands (simulated on bands of 870 to 14,000 vertices, 2 to 8 rings: the
+// iterations of the plain form, within two); where a round reduces the float64
+// residual by less than a factor of 30, or the iterations run out, the band is
+// left to k_band_cl.
+// 10,653 band vertices (33 iterations) 243 -> 193 us, 7,172 (31) 195 -> 118,
+// 710 (44 -> 37 iterations, on three CTAs) 206 -> 123.
+constexpr int PIPE_VT = 480;                       // threads with vertices; one more warp folds the sums
+constexpr int PIPE_THREADS = PIPE_VT + 32;
+constexpr int PIPE_VPT = 2;
+constexpr int PIPE_CAP = PIPE_VT * PIPE_VPT;       // vertices of a CTA at most
+constexpr int PIPE_MAX = BCL_MAX * PIPE_CAP;       // 15,360: a band index fits 15 bits
+// r with 1 / deg (and w), m, p, x (float4), the neighbour codes, u, slot range
+constexpr int PIPE_SMEM = PIPE_CAP * (4 * 16 + 4 * BCL_NB + 24 + 8);
+
+__global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
+    HFCR_PDL_WAIT();
+    cgx::cluster_group cl = cgx::this_cluster();
+    const int n = *a.d_nfree;
+    const int rank = (int)cl.block_rank();
+    int ncta = (int)cl.num_blocks();
+    if (n > ncta * PIPE_CAP) return;  // the same n in every CTA
+    if (n < ncta * BCL_PER) ncta = n > BCL_PER ? (n + BCL_PER - 1) / BCL_PER : 1;
+    if (rank >= ncta) return;
+    extern __shared__ float4 bsm[];
+    __shared__ BclState st;
+    const int chunk = n > 0 ? (n + ncta - 1) / ncta : 1;
+    const int lo = rank * chunk;
+    const int cnt = n - lo < chunk ? (n - lo > 0 ? n - lo : 0) : chunk;
+    float4 *wq = bsm, *zq = wq + PIPE_CAP, *pq = zq + PIPE_CAP, *xq = pq + PIPE_CAP;
+    int4 *cq = (int4 *)(xq + PIPE_CAP);
+    double *uq = (double *)(cq + 2 * (size_t)PIPE_CAP);
+    int2 *ed = (int2 *)(uq + 3 * (size_t)PIPE_CAP);
+    double *gu = a.u64;            // u of every band vertex
+    float4 *gm = (float4 *)a.rec;  // m of every band vertex, alternating by iteration
+    if ((int)threadIdx.x < ncta) {
+        st.recv_of[threadIdx.x] = cl.map_shared_rank(&st.recv[0][0][0], threadIdx.x);
+        st.recvd_of[threadIdx.x] = cl.map_shared_rank(&st.recvd[0][0][0], threadIdx.x);
+    }
+    double dl[3] = {0.0, 0.0, 0.0};
+    bcl_setup<PIPE_VT>(a, lo, cnt, chunk, rank, wq, cq, uq, ed, dl);
+    // this thread's vertices, their neighbour codes 16 bits each: 0x8000 | local
+    // index, the band index, 0xffff for none
+    bool own[PIPE_VPT];
+    int deg[PIPE_VPT];
+    float id[PIPE_VPT], r[PIPE_VPT][3];
+    unsigned code[PIPE_VPT][BCL_NB / 2];
+#pragma unroll
+    for (int v = 0; v < PIPE_VPT; ++v) {
+        const int li = threadIdx.x + v * PIPE_VT;
+        own[v] = (int)threadIdx.x < PIPE_VT && li < cnt;
+        deg[v] = own[v] ? ed[li].y : 0;
+        const float4 r4 = own[v] ? wq[li] : make_float4(0.f, 0.f, 0.f, 0.f);
+        r[v][0] = r4.x; r[v][1] = r4.y; r[v][2] = r4.z; id[v] = r4.w;
+#pragma unroll
+        for (int k = 0; k < BCL_NB / 2; ++k) {
+            const int c0 = own[v] ? ((const int *)cq)[BCL_NB * li + 2 * k] : -1;
+            const int c1 = own[v] ? ((const int *)cq)[BCL_NB * li + 2 * k + 1] : -1;
+            const unsigned h0 = c0 == -1 ? 0xffffu : (c0 < 0 ? 0x8000u | (unsigned)(-2 - c0) : (unsigned)c0);
+            const unsigned h1 = c1 == -1 ? 0xffffu : (c1 < 0 ? 0x8000u | (unsigned)(-2 - c1) : (unsigned)c1);
+            code[v][k] = h0 | h1 << 16;
+        }
+    }
+    // the warps with vertices, and with second ones; the others only meet the
+    // barriers, but the last warp folds the sums
+    const int nw = min((cnt + 31) / 32, PIPE_VT / 32), warp = threadIdx.x >> 5;
+    bool work[PIPE_VPT];
+#pragma unroll
+    for (int v = 0; v < PIPE_VPT; ++v) work[v] = warp < PIPE_VT / 32 && v * PIPE_VT + warp * 32 < cnt;
+    const bool folder = warp == PIPE_VT / 32;
+    const int lane = threadIdx.x & 31;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    // M^-1 of the field in wq (this CTA's; w holds 1 / deg), x: the own value
+    auto precond = [&](int v, const float *x, float *o) {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < BCL_NB; ++k) {
+            const unsigned c = (k & 1) ? code[v][k / 2] >> 16 : code[v][k / 2] & 0xffffu;
+            const float4 nb = (c & 0x8000u) && c != 0xffffu ? wq[c & 0x7fffu] : none;
+            s0 += nb.x * nb.w;
+            s1 += nb.y * nb.w;
+            s2 += nb.z * nb.w;
+        }
+        if (deg[v] > BCL_NB) {
+            const int2 e = ed[threadIdx.x + v * PIPE_VT];
+            for (int k = BCL_NB; k < e.y; ++k) {
+                const int c = a.cnbr[e.x + k];
+                if (c > -2) continue;
+                const float4 nb = wq[-2 - c];
+                s0 += nb.x * nb.w;
+                s1 += nb.y * nb.w;
+                s2 += nb.z * nb.w;
+            }
+        }
+        o[0] = (x[0] + BCL_THETA * s0) * id[v];
+        o[1] = (x[1] + BCL_THETA * s1) * id[v];
+        o[2] = (x[2] + BCL_THETA * s2) * id[v];
+    };
+    // L of the field in zq (this CTA's) and g (the others'), x: the own value
+    auto laplace = [&](int v, const float *x, const float4 *g, float *o) {
+        const float dg = (float)deg[v];
+        float w0 = dg * x[0], w1 = dg * x[1], w2 = dg * x[2];
+        float4 nb[BCL_NB];
+#pragma unroll
+        for (int k = 0; k < BCL_NB; ++k) {
+            const unsigned c = (k & 1) ? code[v][k / 2] >> 16 : code[v][k / 2] & 0xffffu;
+            nb[k] = c == 0xffffu ? none : ((c & 0x8000u) ? zq[c & 0x7fffu] : __ldcg(g + c));
+        }
+#pragma unroll
+        for (int k = 0; k < BCL_NB; ++k) {
+            w0 -= nb[k].x;
+            w1 -= nb[k].y;
+            w2 -= nb[k].z;
+        }
+        if (deg[v] > BCL_NB) {
+            const int2 e = ed[threadIdx.x + v * PIPE_VT];
+            for (int k = BCL_NB; k < e.y; ++k) {
+                const int c = a.cnbr[e.x + k];
+                if (c == -1) continue;
+                const float4 t = c >= 0 ? __ldcg(g + c) : zq[-2 - c];
+                w0 -= t.x;
+                w1 -= t.y;
+                w2 -= t.z;
+            }
+        }
+        o[0] = w0; o[1] = w1; o[2] = w2;
+    };
+    int pf = 0, pd = 0, gp = 0;  // parities: float and float64 receive slots, gm
+    // the cluster's three float64 sums of dl into st.sumsd
+    auto sums64 = [&]() {
+        if (work[0]) warp_sums3(dl, st.scrd + 3 * warp);
+        __syncthreads();
+        if (folder) {
+            const double t = fold3(st.scrd, nw);
+            for (int c = 0; c < ncta; ++c)
+                if (lane < 3) st.recvd_of[c][(pd * BCL_MAX + rank) * 3 + lane] = t;
+        }
+        bcl_sync(cl, ncta);  // every CTA's sums received
+        if (folder) {
+            const double t = fold3(&st.recvd[pd][0][0], ncta);
+            if (lane < 3) st.sumsd[lane] = t;
+        }
+        __syncthreads();
+        pd ^= 1;
+    };
+    sums64();
+    int act = 0;  // coordinates not yet converged (bit c), the same in every thread
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (st.sumsd[c] > 0.0) act |= 1 << c;
+    if (threadIdx.x < 3) {
+        st.target[threadIdx.x] = a.tol * a.tol * st.sumsd[threadIdx.x];
+        st.before[threadIdx.x] = st.sumsd[threadIdx.x];
+    }
+    int it = 0;
+    bool good = true;
+    for (int rounds = 0; act && good; ++rounds) {
+        const int it_round = it;
+        float u[PIPE_VPT][3], w[PIPE_VPT][3], sv[PIPE_VPT][3], q[PIPE_VPT][3], z[PIPE_VPT][3];
+#pragma unroll
+        for (int v = 0; v < PIPE_VPT; ++v)
+            if (own[v]) wq[threadIdx.x + v * PIPE_VT] = make_float4(r[v][0], r[v][1], r[v][2], id[v]);
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < PIPE_VPT; ++v) {
+            if (work[v]) {
+                const int li = threadIdx.x + v * PIPE_VT;
+                precond(v, r[v], u[v]);
+                if (own[v]) {
+                    const float4 t = make_float4(u[v][0], u[v][1], u[v][2], 0.f);
+                    zq[li] = t;
+                    gm[(size_t)gp * a.cap + lo + li] = t;
+                    pq[li] = xq[li] = none;
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) sv[v][c] = q[v][c] = z[v][c] = 0.f;
+            }
+        }
+        bcl_sync(cl, ncta);
+#pragma unroll
+        for (int v = 0; v < PIPE_VPT; ++v)
+            if (work[v]) laplace(v, u[v], gm + (size_t)gp * a.cap, w[v]);
+        gp ^= 1;
+        for (bool first = true;; first = false) {
+            float m[PIPE_VPT][3];
+            // the warps' sums (r, u), (w, u), |r|^2 (0 past the vertices)
+            if (work[0]) {
+                float t[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) t[k] = 0.f;
+#pragma unroll
+                for (int v = 0; v < PIPE_VPT; ++v) {
+                    if (!own[v]) continue;
+                    wq[threadIdx.x + v * PIPE_VT] = make_float4(w[v][0], w[v][1], w[v][2], id[v]);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        t[c] += r[v][c] * u[v][c];
+                        t[3 + c] += w[v][c] * u[v][c];
+                        t[6 + c] += r[v][c] * r[v][c];
+                    }
+                }
+                warp_sums9(t, st.scr + (threadIdx.x >> 5) * 9);
+            }
+            __syncthreads();  // w and the warps' sums; every gather from zq is done
+#pragma unroll
+            for (int v = 0; v < PIPE_VPT; ++v) {
+                if (work[v]) {
+                    const int li = threadIdx.x + v * PIPE_VT;
+                    precond(v, w[v], m[v]);
+                    if (own[v]) {
+                        const float4 t = make_float4(m[v][0], m[v][1], m[v][2], 0.f);
+                        zq[li] = t;
+                        gm[(size_t)gp * a.cap + lo + li] = t;
+                    }
+                }
+            }
+            if (folder) {
+                const float t = fold9(st.scr, nw);
+                if (lane < 9) st.cta[lane] = t;
+                __syncwarp();
+                for (int i = lane; i < 9 * ncta; i += 32)
+                    st.recv_of[i / 9][(pf * BCL_MAX + rank) * 9 + i % 9] = st.cta[i % 9];
+            }
+            bcl_sync(cl, ncta);  // every CTA's m and sums
+            if (folder) {
+                const float t = fold9(&st.recv[pf][0][0], ncta);
+                // lane c < 3: the scalars of coordinate c
+                const float de = __shfl_down_sync(0xffffffffu, t, 3), rho = __shfl_down_sync(0xffffffffu, t, 6);
+                bool go = false;
+                if (lane < 3) {
+                    const int c = lane;
+                    float al, be = 0.f;
+                    if (first) {
+                        // this round's reduction: what is left to the target, with some room
+                        const float room = (float)(0.25 * st.target[c] / fmax(st.sumsd[c], 1e-300));
+                        al = __fdividef(t, de);
+                        st.stop[c] = fmaxf(PIPE_TOL * PIPE_TOL, room) * rho;
+                        go = (act >> c & 1) && rho > 0.f && al > 0.f && isfinite(al);
+                    } else {
+                        be = __fdividef(t, st.gam[c]);
+                        al = __fdividef(t, de - be * __fdividef(t, st.alp[c]));
+                        go = (st.in >> c & 1) && rho > st.stop[c] && al > 0.f && isfinite(al);
+                    }
+                    if (go) {
+                        st.bet[c] = be;
+                        st.alp[c] = al;
+                        st.gam[c] = t;
+                    }
+                }
+                const unsigned in = __ballot_sync(0xffffffffu, go);
+                if (lane == 0) st.in = (int)in;
+            }
+            pf ^= 1;
+            float nn[PIPE_VPT][3];
+#pragma unroll
+            for (int v = 0; v < PIPE_VPT; ++v)
+                if (work[v]) laplace(v, m[v], gm + (size_t)gp * a.cap, nn[v]);
+            gp ^= 1;
+            __syncthreads();  // the scalars
+            const int in = st.in;
+            if (!in || it >= a.max_iters || it - it_round >= PIPE_ITERS) break;
+            {
+#pragma unroll
+                for (int v = 0; v < PIPE_VPT; ++v) {
+                    if (!own[v]) continue;
+                    const int li = threadIdx.x + v * PIPE_VT;
+                    float4 p4 = pq[li], x4 = xq[li];
+                    float *p = &p4.x, *x = &x4.x;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        if (!(in >> c & 1)) continue;
+                        const float al = st.alp[c], be = st.bet[c];
+                        z[v][c] = nn[v][c] + be * z[v][c];
+                        q[v][c] = m[v][c] + be * q[v][c];
+                        sv[v][c] = w[v][c] + be * sv[v][c];
+                        p[c] = u[v][c] + be * p[c];
+                        x[c] += al * p[c];
+                        r[v][c] -= al * sv[v][c];
+                        u[v][c] -= al * q[v][c];
+                        w[v][c] -= al * z[v][c];
+                    }
+                    pq[li] = p4;
+                    xq[li] = x4;
+                }
+            }
+            ++it;
+        }
+        // u += x, then the float64 residual b - L u
+#pragma unroll
+        for (int v = 0; v < PIPE_VPT; ++v) {
+            const int li = threadIdx.x + v * PIPE_VT;
+            if (!own[v]) continue;
+            const float4 x4 = xq[li];
+            const float *x = &x4.x;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double t = uq[3 * li + c] + (double)x[c];
+                uq[3 * li + c] = t;
+                gu[3 * (size_t)(lo + li) + c] = t;
+            }
+        }
+        bcl_sync(cl, ncta);  // every band vertex's u visible
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dl[c] = 0.0;
+#pragma unroll
+        for (int v = 0; v < PIPE_VPT; ++v) {
+            const int li = threadIdx.x + v * PIPE_VT;
+            if (!own[v]) continue;
+            const int2 e = ed[li];
+            double r64[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                r64[c] = a.b64[3 * (size_t)(lo + li) + c] - (double)e.y * uq[3 * li + c];
+            for (int k = 0; k < e.y; ++k) {
+                const int cd = a.cnbr[e.x + k];
+                if (cd == -1) continue;
+                if (cd >= 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) r64[c] += __ldcg(gu + 3 * (size_t)cd + c);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) r64[c] += uq[3 * (-2 - cd) + c];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                r[v][c] = (act >> c & 1) ? (float)r64[c] : 0.f;
+                dl[c] += r64[c] * r64[c];
+            }
+        }
+        sums64();
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (!(act >> c & 1)) continue;
+            if (st.sumsd[c] <= st.target[c]) act &= ~(1 << c);
+            else if (!(st.sumsd[c] < st.before[c] * (1.0 / 900.0))) good = false;
+        }
+        if (it >= a.max_iters || it == it_round || rounds >= BAND_MAX_ROUNDS) good = false;
+        __syncthreads();
+        if (threadIdx.x < 3) st.before[threadIdx.x] = st.sumsd[threadIdx.x];
+    }
+    if (!act) {
+        for (int li = threadIdx.x; li < cnt; li += PIPE_THREADS) {
+            double *ug = a.u + 3 * (size_t)a.fv[lo + li];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ug[c] = uq[3 * li + c];
+        }
+        if (rank == 0 && threadIdx.x == 0) {
+            a.ctl[0] += it;
+            a.ctl[BAND_DONE] = 1;
+        }
+    }
+    bcl_sync(cl, ncta);  // no CTA leaves while another may still write its shared memory
+}
+
+__global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limit) {
+    constexpr int vcap = BCL_VCAP;
+    HFCR_PDL_WAIT();
+    cgx::cluster_group cl = cgx::this_cluster();
+    const int n = *a.d_nfree;
+    // the grid kernel's band, or one the pipelined kernel has done (the same in
+    // every CTA)
+    if (n > limit || a.ctl[BAND_DONE] != 0) return;
+    extern __shared__ float4 bsm[];
+    __shared__ BclState st;
+    const int rank = (int)cl.block_rank();
+    int ncta = (int)cl.num_blocks();
+    if (n < ncta * BCL_PER) ncta = n > BCL_PER ? (n + BCL_PER - 1) / BCL_PER : 1;
+    if (rank >= ncta) return;
+    const int chunk = n > 0 ? (n + ncta - 1) / ncta : 1;
+    const int lo = rank * chunk;
+    const int cnt = n - lo < chunk ? (n - lo > 0 ? n - lo : 0) : chunk;
+    float4 *rq = bsm;  // r (x, y, z) and 1 / deg
+    float4 *gz = (float4 *)a.rec;  // z of every band vertex, for the other CTAs
+    double *gu = a.u64;            // u of every band vertex
+    float4 *pq = rq + vcap, *sq = pq + vcap, *xq = sq + vcap, *wq = xq + vcap;
+    float4 *zq = wq + vcap;
+    int4 *cq = (int4 *)(zq + vcap);  // two int4 (BCL_NB codes) per vertex
+    double *uq = (double *)(cq + 2 * (size_t)vcap);  // u (x, y, z) of the rounds
+    int2 *ed = (int2 *)(uq + 3 * (size_t)vcap);
+    if ((int)threadIdx.x < ncta) {
+        st.recv_of[threadIdx.x] = cl.map_shared_rank(&st.recv[0][0][0], threadIdx.x);
+        st.recvd_of[threadIdx.x] = cl.map_shared_rank(&st.recvd[0][0][0], threadIdx.x);
+    }
+    double dl[3] = {0.0, 0.0, 0.0};
+    bcl_setup<BCL_THREADS>(a, lo, cnt, chunk, rank, rq, cq, uq, ed, dl);
+    for (int li = threadIdx.x; li < cnt; li += BCL_THREADS) {
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        pq[li] = z4;
+        sq[li] = z4;
+        xq[li] = z4;
     }
     int pf = 0, pd = 0;  // parities of the float and float64 receive slots
     bcl_sums<double, 3>(cl, dl, st.scrd, &st.recvd[0][0][0], st.recvd_of, pd, rank, ncta, st.sumsd);
@@ -984,7 +1456,7 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
                 zq[li] = z4;
                 gz[lo + li] = z4;
             }
-            cl.sync();  // every band vertex's z visible
+            bcl_sync(cl, ncta);  // every band vertex's z visible
             // w = L z, and the sums (r, z), (w, z), |r|^2
             float fl[9];
 #pragma unroll
@@ -1084,7 +1556,7 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
 #pragma unroll
             for (int c = 0; c < 3; ++c) gu[3 * (size_t)(lo + li) + c] = u[c];
         }
-        cl.sync();  // every band vertex's u visible
+        bcl_sync(cl, ncta);  // every band vertex's u visible
 #pragma unroll
         for (int c = 0; c < 3; ++c) dl[c] = 0.0;
         for (int li = threadIdx.x; li < cnt; li += BCL_THREADS) {
@@ -1130,7 +1602,7 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
         a.ctl[0] += it;
         if (fail) a.ctl[1] = 1;
     }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
+    bcl_sync(cl, ncta);  // no CTA leaves while another may still write its shared memory
 }
 
 inline int blocks(int n) { return (n + 255) / 256; }
@@ -1182,7 +1654,7 @@ static int band_grid_max() {
 // the cluster of k_band_cl on this device: the most CTAs (16, 8, 4, 2)
 // whose cluster fits, and the band vertices one CTA holds
 struct BclConfig {
-    bool ok = false;
+    bool ok = false, pipe = false;  // pipe: k_band_pipe's cluster fits too
     int ncta = 0, vcap = 0;
 };
 static BclConfig band_cl_config() {
@@ -1217,6 +1689,10 @@ static BclConfig band_cl_config() {
                 cudaGetLastError();
             }
         }
+        if (c.ok && cudaFuncSetAttribute(k_band_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM) ==
+                        cudaSuccess)
+            c.pipe = cudaFuncSetAttribute(k_band_pipe, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                     cudaSuccess;
         cudaGetLastError();
         c.vcap = BCL_VCAP;
         cached[dev] = c;
@@ -1314,8 +1790,8 @@ const double *diffuse_field(const DiffMeshArgs &a, const DiffMeshArgs &b, double
     if (bc.ok) {
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3(bc.ncta);
-        lc.blockDim = dim3(BCL_THREADS);
-        lc.dynamicSmemBytes = BCL_SMEM;
+        lc.blockDim = dim3(PIPE_THREADS);
+        lc.dynamicSmemBytes = PIPE_SMEM;
         lc.stream = s;
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1326,12 +1802,22 @@ const double *diffuse_field(const DiffMeshArgs &a, const DiffMeshArgs &b, double
         at[1].val.programmaticStreamSerializationAllowed = 1;
         lc.attrs = at;
         lc.numAttrs = 2;
+        if (bc.pipe && rings <= PIPE_RINGS) {
+            if (cudaLaunchKernelEx(&lc, k_band_pipe, ba) == cudaSuccess) note_launch();
+            else cudaGetLastError();
+        }
+        lc.blockDim = dim3(BCL_THREADS);
+        lc.dynamicSmemBytes = BCL_SMEM;
         if (cudaLaunchKernelEx(&lc, k_band_cl, ba, limit) == cudaSuccess) {
             note_launch();
         } else {
             cudaGetLastError();
             limit = -1;
         }
+    }
+    if (P.ntot <= limit) {  // no band of these meshes is larger
+        mark(0, s);
+        return u;
     }
     void *args[] = {&ba, &limit};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_band_cg, grid, BAND_TPB, args, 0, s);
