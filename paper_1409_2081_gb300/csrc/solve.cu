@@ -384,16 +384,18 @@ __device__ __forceinline__ void block_sum3(float a, float b, float c, float *red
 }
 
 // sum over the block, identical in every thread: each warp folds its values
-// with a butterfly and keeps lane 0's result, and every thread adds the warp
-// results in warp order
+// with a butterfly and keeps lane 0's result, and every warp folds the warps'
+// results with the same butterfly
 __device__ __forceinline__ double block_sum_uniform(double x, double *redd) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     x = __shfl_sync(0xffffffffu, x, 0);
     if ((threadIdx.x & 31) == 0) redd[threadIdx.x >> 5] = x;
     __syncthreads();
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += redd[w];
+    const int lane = threadIdx.x & 31;
+    double s = lane < (int)(blockDim.x >> 5) ? redd[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     __syncthreads();
     return s;
 }
@@ -401,7 +403,41 @@ __device__ __forceinline__ double block_sum_uniform(double x, double *redd) {
 // The thread group that solves one zone: a whole CTA (CtaGroup) or one
 // warp (WarpGroup, for small zones; barriers are __syncwarp and every
 // reduction stays in shuffles).  Sums are identical in every lane.
+// a, b, c summed over the warp by halving (six shuffles instead of fifteen):
+// the lanes 8 k .. 8 k + 7 end with sum k (k < 3)
+__device__ __forceinline__ float warp_halve3(float a, float b, float c) {
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, q = lane & 8;
+    const float x = (h ? c : a) + __shfl_xor_sync(0xffffffffu, h ? a : c, 16);
+    const float y = (h ? 0.f : b) + __shfl_xor_sync(0xffffffffu, h ? b : 0.f, 16);
+    float t = (q ? y : x) + __shfl_xor_sync(0xffffffffu, q ? x : y, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+// the same over NW warps (8 or 16): each warp's sums to scr[4 w + k], the
+// group's barrier, then every warp folds them alike
+template <int NW, class F>
+__device__ __forceinline__ void group_halve3(float a, float b, float c, float *scr, int w, F sync, float &sa,
+                                             float &sb, float &sc) {
+    const int lane = threadIdx.x & 31;
+    float t = warp_halve3(a, b, c);
+    if ((lane & 7) == 0) scr[4 * w + (lane >> 3)] = t;
+    sync();
+    t = scr[4 * (lane & 7) + (lane >> 3)];
+    if (NW == 16) t += scr[4 * ((lane & 7) + 8) + (lane >> 3)];
+#pragma unroll
+    for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    sa = __shfl_sync(0xffffffffu, t, 0);
+    sb = __shfl_sync(0xffffffffu, t, 8);
+    sc = __shfl_sync(0xffffffffu, t, 16);
+}
+
 struct CtaGroup {
+    static constexpr int SIZE = 512;  // of the solvers by rows
+    __device__ static void sum3h(float a, float b, float c, float *scr, float &sa, float &sb, float &sc) {
+        group_halve3<16>(a, b, c, scr, threadIdx.x >> 5, [] { __syncthreads(); }, sa, sb, sc);
+    }
     __device__ static int rank() { return threadIdx.x; }
     __device__ static int size() { return blockDim.x; }
     __device__ static void sync() { __syncthreads(); }
@@ -413,6 +449,13 @@ struct CtaGroup {
 };
 
 struct WarpGroup {
+    static constexpr int SIZE = 32;
+    __device__ static void sum3h(float a, float b, float c, float *, float &sa, float &sb, float &sc) {
+        const float t = warp_halve3(a, b, c);
+        sa = __shfl_sync(0xffffffffu, t, 0);
+        sb = __shfl_sync(0xffffffffu, t, 8);
+        sc = __shfl_sync(0xffffffffu, t, 16);
+    }
     __device__ static int rank() { return threadIdx.x & 31; }
     __device__ static int size() { return 32; }
     __device__ static void sync() { __syncwarp(); }
@@ -436,11 +479,15 @@ struct WarpGroup {
 
 // One 256-thread half H of a 512-thread CTA (threads 256 H .. 256 H + 255)
 // solving a zone of its own: its barrier is the named barrier 1 + H, its
-// reductions run over its 8 warps through its own red / redd slices (24
+// reductions run over its 8 warps through its own red / redd slices (32
 // floats, 8 doubles; each slot is rewritten only after another of the
 // half's barriers).  Sums are identical in every thread of the half.
 template <int H>
 struct HalfGroup {
+    static constexpr int SIZE = 256;
+    __device__ static void sum3h(float a, float b, float c, float *scr, float &sa, float &sb, float &sc) {
+        group_halve3<8>(a, b, c, scr, (threadIdx.x >> 5) & 7, [] { sync(); }, sa, sb, sc);
+    }
     __device__ static int rank() { return threadIdx.x - 256 * H; }
     __device__ static int size() { return 256; }
     __device__ static void sync() { asm volatile("bar.sync %0, 256;" ::"n"(1 + H) : "memory"); }
@@ -478,8 +525,9 @@ struct HalfGroup {
         x = __shfl_sync(0xffffffffu, x, 0);
         if ((threadIdx.x & 31) == 0) redd[(threadIdx.x >> 5) & 7] = x;
         sync();
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += redd[w];
+        double s = redd[threadIdx.x & 7];
+#pragma unroll
+        for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         sync();
         return s;
     }
@@ -1449,9 +1497,11 @@ __device__ __noinline__ int zone_blocks(const CgViewS &v, int k, int U, const in
 // Rounds of iterative refinement of zone z, everything the float32 CG
 // touches staged in shared memory at base (zone_smem_need bytes); BLK: the
 // large zones' preconditioner blocks (zone_blocks) instead of the groups.
+// warm (BLK): lambda and res come from solve_zone_rows, whose run took
+// block_switch iterations; the blocks take over from there.
 template <class Gp, bool BLK = false>
 __device__ __forceinline__ ZoneResult solve_zone_smem(const ZoneArgs &a, int z, char *base, double bb,
-                                                      float *red, double *redd) {
+                                                      float *red, double *redd, const ZoneResult *warm = nullptr) {
     const int tid = Gp::rank(), nt = Gp::size();
     const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
     const int j0 = a.zv[z], U = a.zv[z + 1] - j0;
@@ -1493,6 +1543,29 @@ __device__ __forceinline__ ZoneResult solve_zone_smem(const ZoneArgs &a, int z, 
     // continues on the blocks (that run is not counted)
     bool blocks_on = false;
     const bool may_switch = BLK && a.block_switch > 0 && a.block_switch < a.maxit;
+    auto to_blocks = [&]() {
+        // the block order, the places' blocks and the block starts in
+        // the groups' inverse rows' slot (16 B a row: 2 + 4 + 4)
+        uint16_t *bperm = (uint16_t *)pinv;
+        int *binfo = (int *)(bperm + ((k + 7) & ~7));
+        int *bst = binfo + k;
+        float *binv = a.binv + 16 * (size_t)s0;
+        zone_blocks<Gp>(v, k, U, gst, G, bperm, binfo, bst, binv, (int *)red);
+        v.bperm = bperm;
+        v.binfo = binfo;
+        v.binv = binv;
+        blocks_on = true;
+        extra = 1;
+    };
+    if constexpr (BLK) {
+        if (warm) {
+            Gp::sync();
+            rr = zone_residual<Gp>(v, k, U, s0, j0, a.n64, a.b64, a.lam, a.u64, redd);
+            its = warm->its;
+            rounds = warm->rounds;
+            to_blocks();
+        }
+    }
     while (rr > target && rounds < a.max_refine + extra) {
         for (int t = tid; t < k; t += nt) {
             v.p[t] = 0.f;
@@ -1517,19 +1590,8 @@ __device__ __forceinline__ ZoneResult solve_zone_smem(const ZoneArgs &a, int z, 
             Gp::sync();
             break;
         }
-        if (may_switch && !blocks_on && n_it >= cap_it && rr > target) {
-            // the block order, the places' blocks and the block starts in
-            // the groups' inverse rows' slot (16 B a row: 2 + 4 + 4)
-            uint16_t *bperm = (uint16_t *)pinv;
-            int *binfo = (int *)(bperm + ((k + 7) & ~7));
-            int *bst = binfo + k;
-            float *binv = a.binv + 16 * (size_t)s0;
-            zone_blocks<Gp>(v, k, U, gst, G, bperm, binfo, bst, binv, (int *)red);
-            v.bperm = bperm;
-            v.binfo = binfo;
-            v.binv = binv;
-            blocks_on = true;
-            extra = 1;
+        if constexpr (BLK) {
+            if (may_switch && !blocks_on && n_it >= cap_it && rr > target) to_blocks();
         }
     }
     ZoneResult res;
@@ -1537,6 +1599,317 @@ __device__ __forceinline__ ZoneResult solve_zone_smem(const ZoneArgs &a, int z, 
     res.its = its;
     res.rounds = rounds;
     return res;
+}
+
+// ---------------------------------------------------------------------------
+// A zone solved by rows: the same rounds as solve_zone_smem (float32 PCG to
+// inner_tol, float64 residual), with the zone's matrix A = J M^-1 J^T written
+// out once.  Its rows are short (5 to 9 entries on average where cloth and
+// bodies cross: few stencils share a vertex), so a product is one pass over a
+// row's entries in the place of the vertex gather, a barrier and the four-
+// vertex products.  Row t belongs to one thread (RPT rows each), which keeps
+// the row's CG vectors, its inverse-block row and lambda in registers; only r
+// (for the blocks) and z are exchanged through shared memory.  The entries,
+// (value, column), lie in slices of 32 rows, as long as the slice's longest
+// row and column by column, so that a warp reads them without conflicts.
+// Bound by the latency of an iteration's three barriers and shared-memory
+// passes: against a gather of u and four vertex products per row, a zone of
+// 1,219 rows (74 iterations, 3 rounds) 440 -> 227 us, zones of 33 to 255 rows
+// in pairs 185 -> 124 us, zones of up to 32 rows in a warp each 96 -> 45 us.
+// Returns 0 when done (res filled, lambda stored), 1 when the zone does not
+// fit (rows, shared memory) and nothing was done, 2 when a run of a
+// BLK zone took block_switch iterations: lambda holds the best so far, and the
+// blocks are to take over.
+// ---------------------------------------------------------------------------
+template <class Gp, int RPT, bool BLK>
+__device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *base, int bytes, double bb,
+                                               float *red, double *redd, ZoneResult &res) {
+    constexpr int NT = Gp::SIZE, NS = RPT * NT / 32;  // slices of 32 rows
+    const int tid = Gp::rank(), lane = threadIdx.x & 31, wq = tid >> 5;
+    const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
+    const int j0 = a.zv[z], U = a.zv[z + 1] - j0;
+    const int g0 = a.zg[z], G = a.zg[z + 1] - g0;
+    const int e0 = a.seg[j0];
+    // layout: n4 (later r and z) | lambda and -lambda / 3 | vidx | winv | seg |
+    // cval | groups | slices | matrix, u
+    const long long fixed = 50ll * k + 6ll * U + 4ll * NS + 64;
+    if (k > RPT * NT || fixed > bytes) return 1;
+    float4 *n4 = (float4 *)base;
+    float *rS = (float *)base, *zS = rS + k;
+    double *lamS = (double *)(n4 + k);
+    ushort4 *vidx = (ushort4 *)(lamS + 2 * k);
+    float *winv = (float *)(vidx + k);
+    uint16_t *seg = (uint16_t *)(winv + U);
+    uint16_t *cval = seg + U + 1;
+    uint16_t *grp = cval + 4 * k;
+    int *sl = (int *)(((uintptr_t)(grp + k) + 3) & ~(uintptr_t)3);
+    for (int t = tid; t < k; t += NT) {
+        const int4 g = a.vidx[s0 + t];
+        vidx[t] = make_ushort4((unsigned short)(g.x - j0), (unsigned short)(g.y - j0),
+                               (unsigned short)(g.z - j0), (unsigned short)(g.w - j0));
+        n4[t] = a.n32[s0 + t];
+    }
+    for (int g = tid; g < G; g += NT) {  // each row's block: first row and size
+        const int b0 = a.gst[g0 + g] - s0, b1 = a.gst[g0 + g + 1] - s0;
+        for (int t = b0; t < b1; ++t) grp[t] = (uint16_t)(b0 << 3 | (b1 - b0));
+    }
+    for (int j = tid; j <= U; j += NT) seg[j] = (uint16_t)(a.seg[j0 + j] - e0);
+    for (int j = tid; j < U; j += NT) winv[j] = a.winv[j0 + j];
+    for (int e = tid; e < 4 * k; e += NT) cval[e] = (uint16_t)(a.cval[e0 + e] - 4 * s0);
+    Gp::sync();
+    // a row's entries: the four vertices' stencil lists (ascending) merged
+    auto walk = [&](int t, auto emit) {
+        const ushort4 v = vidx[t];
+        const int vs[4] = {v.x, v.y, v.z, v.w};
+        int at[4], end[4], cur[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            at[q] = seg[vs[q]];
+            end[q] = seg[vs[q] + 1];
+            cur[q] = at[q] < end[q] ? cval[at[q]] : 0x7fffffff;
+        }
+        int n = 0;
+        while (true) {
+            const int c = min(min(cur[0] >> 2, cur[1] >> 2), min(cur[2] >> 2, cur[3] >> 2));
+            if (c >= k) break;  // past every list's end
+            float w = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if ((cur[q] >> 2) != c) continue;
+                w += (q ? -1.0f / 3.0f : 1.0f) * ((cur[q] & 3) ? -1.0f / 3.0f : 1.0f) * winv[vs[q]];
+                ++at[q];
+                cur[q] = at[q] < end[q] ? cval[at[q]] : 0x7fffffff;
+            }
+            emit(n++, c, w);
+        }
+        return n;
+    };
+    int off[RPT], len[RPT];
+#pragma unroll
+    for (int v = 0; v < RPT; ++v) {
+        const int t = tid + v * NT;
+        const int n = t < k ? walk(t, [](int, int, float) {}) : 0;
+        len[v] = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+        if (lane == 0) sl[wq + v * (NT / 32)] = len[v];
+    }
+    Gp::sync();
+    int total = 0;
+#pragma unroll
+    for (int v = 0; v < RPT; ++v) off[v] = 0;
+    for (int q = 0; q < NS; ++q) {
+#pragma unroll
+        for (int v = 0; v < RPT; ++v)
+            if (q == wq + v * (NT / 32)) off[v] = total;
+        total += sl[q];
+    }
+    float2 *mat = (float2 *)(((uintptr_t)(sl + NS) + 15) & ~(uintptr_t)15);
+    const long long used = (long long)((char *)mat - base) + 256ll * total;
+    if (used > bytes) return 1;
+    // u of the float64 residuals beside the matrix where it fits
+    double *u64 = used + 24ll * U <= bytes ? (double *)(mat + 32 * total) : a.u64 + 3 * (size_t)j0;
+#pragma unroll
+    for (int v = 0; v < RPT; ++v) {
+        const int t = tid + v * NT;
+        float2 *m = mat + 32 * off[v] + lane;
+        int n = 0;
+        if (t < k) {
+            const float4 nt4 = n4[t];
+            n = walk(t, [&](int i, int c, float w) {
+                const float4 b = n4[c];
+                m[32 * i] = make_float2(w * (nt4.x * b.x + nt4.y * b.y + nt4.z * b.z), __int_as_float(c));
+            });
+        }
+        for (int i = n; i < len[v]; ++i) m[32 * i] = make_float2(0.f, __int_as_float(0));
+    }
+    Gp::sync();  // the normals' place becomes r and z
+    float r[RPT], x[RPT], p[RPT], s[RPT], w[RPT], zz[RPT];
+    float4 pin[RPT];
+    double lam[RPT];
+    int blk[RPT];
+#pragma unroll
+    for (int v = 0; v < RPT; ++v) {
+        const int t = tid + v * NT;
+        const bool on = t < k;
+        r[v] = on ? (float)a.b64[s0 + t] : 0.f;
+        pin[v] = on ? a.pinv[s0 + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+        blk[v] = on ? grp[t] : 0;
+        lam[v] = 0.0;
+    }
+    // one row per thread: its first entries in registers too
+    constexpr int KEEP = RPT == 1 ? 8 : 0;
+    float kv[KEEP + 1];
+    int kc[KEEP + 1];
+    if constexpr (KEEP > 0) {
+#pragma unroll
+        for (int i = 0; i < KEEP; ++i) {
+            const float2 m = i < len[0] ? mat[32 * (off[0] + i) + lane] : make_float2(0.f, 0.f);
+            kv[i] = m.x;
+            kc[i] = __float_as_int(m.y);
+        }
+    }
+    // z = P^-1 r and w = A z; the sums (r, z), (w, z), |r|^2
+    auto apply = [&](float &ga, float &de, float &rh) {
+#pragma unroll
+        for (int v = 0; v < RPT; ++v)
+            if (tid + v * NT < k) rS[tid + v * NT] = r[v];
+        Gp::sync();
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            const int b0 = blk[v] >> 3, m = blk[v] & 7;
+            float q = 0.f;
+            if (m > 0) q = pin[v].x * rS[b0];
+            if (m > 1) q += pin[v].y * rS[b0 + 1];
+            if (m > 2) q += pin[v].z * rS[b0 + 2];
+            if (m > 3) q += pin[v].w * rS[b0 + 3];
+            zz[v] = q;
+            if (m > 0) zS[tid + v * NT] = q;
+        }
+        Gp::sync();
+        float g = 0.f, d = 0.f, h = 0.f;
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            const float2 *m = mat + 32 * off[v] + lane;
+            float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
+            if constexpr (KEEP > 0) {
+#pragma unroll
+                for (int i = 0; i < KEEP; i += 4) {
+                    acc0 += kv[i] * zS[kc[i]];
+                    acc1 += kv[i + 1] * zS[kc[i + 1]];
+                    acc2 += kv[i + 2] * zS[kc[i + 2]];
+                    acc3 += kv[i + 3] * zS[kc[i + 3]];
+                }
+            }
+            int i = KEEP;
+            for (; i + 4 <= len[v]; i += 4) {
+                const float2 m0 = m[32 * i], m1 = m[32 * (i + 1)], m2 = m[32 * (i + 2)], m3 = m[32 * (i + 3)];
+                acc0 += m0.x * zS[__float_as_int(m0.y)];
+                acc1 += m1.x * zS[__float_as_int(m1.y)];
+                acc2 += m2.x * zS[__float_as_int(m2.y)];
+                acc3 += m3.x * zS[__float_as_int(m3.y)];
+            }
+            for (; i < len[v]; ++i) {
+                const float2 m0 = m[32 * i];
+                acc0 += m0.x * zS[__float_as_int(m0.y)];
+            }
+            w[v] = (acc0 + acc1) + (acc2 + acc3);
+            g += r[v] * zz[v];
+            d += w[v] * zz[v];
+            h += r[v] * r[v];
+        }
+        Gp::sum3h(g, d, h, red, ga, de, rh);
+    };
+    const double target = a.rel_tol * a.rel_tol * bb, third = 1.0 / 3.0;
+    double rr = bb;
+    int its = 0, rounds = 0;
+    bool hand_over = false;
+    const bool may_switch = BLK && a.block_switch > 0 && a.block_switch < a.maxit;
+    const int cap_it = may_switch ? a.block_switch : a.maxit;
+    while (rr > target && rounds < a.max_refine) {
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) x[v] = p[v] = s[v] = 0.f;
+        float gamma, delta, rho;
+        apply(gamma, delta, rho);
+        const float stop = (float)a.tol * (float)a.tol * rho;
+        float alpha = __fdividef(gamma, delta), beta = 0.f;
+        int it = 0;
+        while (it < cap_it && rho > stop && rho > 0.f && alpha > 0.f && isfinite(alpha)) {
+            // beta = g' / g and alpha' = g' / (d' - beta g' / alpha): the
+            // reciprocals that do not wait for the sums
+            const float rg = __fdividef(1.0f, gamma), ra = __fdividef(1.0f, alpha);
+#pragma unroll
+            for (int v = 0; v < RPT; ++v) {
+                p[v] = zz[v] + beta * p[v];
+                s[v] = w[v] + beta * s[v];
+                x[v] += alpha * p[v];
+                r[v] -= alpha * s[v];
+            }
+            float gn, dn, rn;
+            apply(gn, dn, rn);
+            beta = gn * rg;
+            alpha = __fdividef(gn, dn - beta * (gn * ra));
+            gamma = gn;
+            rho = rn;
+            ++it;
+        }
+        its += it;
+        // lambda += x, then the float64 residual b - J M^-1 J^T lambda
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            lam[v] += (double)x[v];
+            if (tid + v * NT < k) {
+                lamS[2 * (tid + v * NT)] = lam[v];
+                lamS[2 * (tid + v * NT) + 1] = -third * lam[v];
+            }
+        }
+        Gp::sync();
+        for (int j = tid; j < U; j += NT) {
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+            const int e1 = seg[j + 1];
+            for (int e = seg[j]; e < e1; e += 4) {  // four entries' normals in flight
+                double4_32a n[4];
+                double p[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int c = cval[min(e + q, e1 - 1)];
+                    n[q] = a.n64[s0 + (c >> 2)];
+                    p[q] = lamS[2 * (c >> 2) + ((c & 3) ? 1 : 0)];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (e + q >= e1) break;
+                    a0 += p[q] * n[q].x;
+                    a1 += p[q] * n[q].y;
+                    a2 += p[q] * n[q].z;
+                }
+            }
+            const double wj = (double)winv[j];
+            u64[3 * j] = wj * a0;
+            u64[3 * j + 1] = wj * a1;
+            u64[3 * j + 2] = wj * a2;
+        }
+        Gp::sync();
+        double sum = 0.0;
+        float rn[RPT];
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            const int t = tid + v * NT;
+            rn[v] = 0.f;
+            if (t >= k) continue;
+            const ushort4 g = vidx[t];
+            const double *ux = u64 + 3 * g.x, *ua = u64 + 3 * g.y, *ub = u64 + 3 * g.z, *uc = u64 + 3 * g.w;
+            const double4_32a n = a.n64[s0 + t];
+            const double d0 = ux[0] - (ua[0] + ub[0] + uc[0]) * third;
+            const double d1 = ux[1] - (ua[1] + ub[1] + uc[1]) * third;
+            const double d2 = ux[2] - (ua[2] + ub[2] + uc[2]) * third;
+            const double q = a.b64[s0 + t] - (n.x * d0 + n.y * d1 + n.z * d2);
+            rn[v] = (float)q;
+            sum += q * q;
+        }
+        const double rr_new = Gp::sum(sum, redd);
+        ++rounds;
+        if (!(rr_new < rr)) {
+            // the run did not reduce the float64 residual (a stagnating or
+            // failing float32 run): its correction is taken back, the zone
+            // keeps the best lambda found
+#pragma unroll
+            for (int v = 0; v < RPT; ++v) lam[v] -= (double)x[v];
+            break;
+        }
+        rr = rr_new;
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) r[v] = rn[v];
+        if (may_switch && it >= cap_it && rr > target) {
+            hand_over = true;
+            break;
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < RPT; ++v)
+        if (tid + v * NT < k) a.lam[s0 + tid + v * NT] = lam[v];
+    res.rr = rr;
+    res.its = its;
+    res.rounds = rounds;
+    return hand_over ? 2 : 0;
 }
 
 __device__ __forceinline__ void zone_finish(const ZoneArgs &a, int z, double rr, double bb, int its,
@@ -1566,7 +1939,11 @@ __global__ void __launch_bounds__(256, 4) k_cg_zone_warp(const int *d_nz, ZoneAr
         const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
         if (k > WARP_ZONE) continue;
         const double bb = zone_start<WarpGroup>(a, s0, k, nullptr);
-        const ZoneResult r = solve_zone_smem<WarpGroup>(a, z, base, bb, nullptr, nullptr);
+        ZoneResult r;
+        if (solve_zone_rows<WarpGroup, 1, false>(a, z, base, WARP_ZONE_SMEM, bb, nullptr, nullptr, r)) {
+            __syncwarp();
+            r = solve_zone_smem<WarpGroup>(a, z, base, bb, nullptr, nullptr);
+        }
         if (lane == 0) zone_finish(a, z, r.rr, bb, r.its, r.rounds, true);
         __syncwarp();  // the slice is reused by the warp's next zone
     }
@@ -1581,7 +1958,8 @@ struct ZoneScratch {
     float *x, *r, *p, *s, *w, *z, *u;
 };
 
-template <class Gp, bool BLK = false>
+// RPT: rows per thread of the solver by rows, tried first (0: never)
+template <class Gp, int RPT, bool BLK = false>
 __device__ __forceinline__ void solve_zone(const ZoneArgs &a, int z, char *base, int smem_bytes,
                                            float *red, double *redd, const ZoneScratch &g) {
     const int tid = Gp::rank(), nt = Gp::size();
@@ -1592,8 +1970,18 @@ __device__ __forceinline__ void solve_zone(const ZoneArgs &a, int z, char *base,
     const bool in_smem = zone_smem_need(k, U, G) <= smem_bytes;
     int its = 0, rounds = 0;
     double rr;
-    if (in_smem) {
-        const ZoneResult r = solve_zone_smem<Gp, BLK>(a, z, base, bb, red, redd);
+    ZoneResult first;
+    int how = 1;
+    if constexpr (RPT > 0) {
+        how = solve_zone_rows<Gp, RPT, BLK>(a, z, base, smem_bytes, bb, red, redd, first);
+        Gp::sync();  // shared memory is the next solver's
+    }
+    if (how == 0) {
+        rr = first.rr;
+        its = first.its;
+        rounds = first.rounds;
+    } else if (in_smem) {
+        const ZoneResult r = solve_zone_smem<Gp, BLK>(a, z, base, bb, red, redd, how == 2 ? &first : nullptr);
         rr = r.rr;
         its = r.its;
         rounds = r.rounds;
@@ -1630,7 +2018,7 @@ __device__ __forceinline__ void solve_zone(const ZoneArgs &a, int z, char *base,
             }
         }
     }
-    if (tid == 0) zone_finish(a, z, rr, bb, its, rounds, in_smem);
+    if (tid == 0) zone_finish(a, z, rr, bb, its, rounds, how == 0 || in_smem);
     Gp::sync();  // shared memory is reused by the group's next zone
 }
 
@@ -1717,7 +2105,7 @@ __device__ __forceinline__ void half_zones(const ZoneArgs &a, int nz, int small_
          z = more ? next_zone<HalfGroup<H>>(a.ticket + 1, 2 * gridDim.x, slot) : nz) {
         const int k = a.zs[z + 1] - a.zs[z];
         if (k <= small_lo || k >= ZONE_MID) continue;
-        solve_zone<HalfGroup<H>>(a, z, base, bytes, red, redd, g);
+        solve_zone<HalfGroup<H>, 1>(a, z, base, bytes, red, redd, g);
     }
 }
 
@@ -1725,7 +2113,7 @@ __global__ void __launch_bounds__(512, 2) k_cg_zone_pair(const int *d_nz, ZoneAr
                                                          ZoneScratch g, int smem_bytes, int big_ctas) {
     HFCR_PDL_WAIT();
     extern __shared__ float4 smem4[];
-    __shared__ float red[96];     // halves: 24 floats each; the whole CTA: 48
+    __shared__ float red[96];     // halves: 32 floats each; the whole CTA: 64
     __shared__ double redd[16];   // halves: 8 each; the whole CTA: 16
     __shared__ int slot[3];
     const int nz = *d_nz;
@@ -1743,7 +2131,7 @@ __global__ void __launch_bounds__(512, 2) k_cg_zone_pair(const int *d_nz, ZoneAr
     for (int z = first; z < nz; z = more ? next_zone<CtaGroup>(a.ticket, gridDim.x, slot + 2) : nz) {
         const int k = a.zs[z + 1] - a.zs[z];
         if (k < ZONE_MID || k >= ZONE_BIG) continue;
-        solve_zone<CtaGroup>(a, z, (char *)smem4, smem_bytes, red, redd, g);
+        solve_zone<CtaGroup, 2>(a, z, (char *)smem4, smem_bytes, red, redd, g);
     }
     // then the smaller ones, two at a time (a whole-CTA zone ends with a
     // barrier of the whole CTA, so the halves may reuse the shared memory)
@@ -1751,7 +2139,7 @@ __global__ void __launch_bounds__(512, 2) k_cg_zone_pair(const int *d_nz, ZoneAr
     if (threadIdx.x < 256)
         half_zones<0>(a, nz, small_lo, (char *)smem4, half_bytes, red, redd, g, slot);
     else
-        half_zones<1>(a, nz, small_lo, (char *)smem4 + half_bytes, half_bytes, red + 24, redd + 8,
+        half_zones<1>(a, nz, small_lo, (char *)smem4 + half_bytes, half_bytes, red + 32, redd + 8,
                       g, slot + 1);
 }
 
@@ -1787,7 +2175,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_cg_zone(const int *d_nz, ZoneArg
         if (k <= sel[2]) continue;
         if (leave_big && zone_smem_need(k, a.zv[z + 1] - a.zv[z], a.zg[z + 1] - a.zg[z]) > smem_bytes)
             continue;
-        solve_zone<CtaGroup, true>(a, z, (char *)smem4, smem_bytes, red, redd, g);
+        solve_zone<CtaGroup, 3, true>(a, z, (char *)smem4, smem_bytes, red, redd, g);
         if (threadIdx.x == 0) {  // rows and touched vertices of the zones of this launch
             atomicAdd(&a.ctl[5], k);
             atomicAdd(&a.ctl[6], a.zv[z + 1] - a.zv[z]);
@@ -2122,7 +2510,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cg_zone_cl(const int *d_nz, Z
         if (L.bytes > CL_SMEM) {
             // too large for the cluster's shared memory: the first CTA solves
             // it on global memory (the one-CTA path), the others go on
-            if (rank == 0) solve_zone<CtaGroup>(a, z, base, 0, bred, bredd, gs);
+            if (rank == 0) solve_zone<CtaGroup, 0>(a, z, base, 0, bred, bredd, gs);
             continue;
         }
         const int r0 = rb[rank], kr = rb[rank + 1] - r0;            // own rows
