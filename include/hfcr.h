@@ -133,8 +133,9 @@ typedef struct {
     int32_t traverse_variant; /* traversal kernel variant 0..8 used until hfcr_autotune picks one
                                  (default 0; every variant finds the same pairs) */
     int32_t setup_path;     /* response setup (vertex CSR, impact zones, preconditioner groups):
-                               0 (default) one cooperative launch, 1 a sequence of about 25
-                               kernels; both build the same arrays, so the results are identical */
+                               0 (default) one CTA and a grid over the rows up to 4,096 stencils,
+                               one cooperative launch above, 1 a sequence of about 25 kernels; every
+                               sum keeps its order, so the results are identical */
     int32_t diffuse_max_iters; /* harmonic diffusion: iteration limit (0: default 1000) */
     double diffuse_tol;     /* harmonic diffusion: stop at |r| <= diffuse_tol |b| per coordinate,
                                0 < tol < 1 (0: default 1e-10) */

@@ -950,64 +950,110 @@ __device__ __forceinline__ void store_inv_row(double4_32a *p, const double *row)
     *p = make_double4_32a(row[0], row[1], row[2], row[3]);
 }
 
-// R: float4 rows for the mixed solver, double4_32a rows for the float64 one
+// Groups first + i (i = 0, step, ...) below n, eight per warp: the four lanes
+// of a quad hold the block's rows and run Gauss-Jordan with partial pivoting
+// in registers, exchanging rows by shuffles.  A (near-)singular block falls
+// back to the inverse of its diagonal.  Called by whole warps; gi: the
+// warp's first group, step: the groups of all warps taking part.  Bound by
+// the latency of the loads and of float64 arithmetic: one thread per group
+// with the block in local memory took 33 us (1,000 to 2,000 groups), a quad
+// 14 us.  R: float4 rows for the mixed solver, double4_32a rows for the
+// float64 one; perm: row t is row perm[t] of ids and n64.
 template <class G, typename R>
-__device__ __forceinline__ void group_inverse_one(int g, const int *gst, const int4 *ids,
-                                                  const double4_32a *n64, int nA, const float *wA,
-                                                  const float *wB, R *pinv) {
-    {
-        const int a0 = G::ld(gst + g), m = G::ld(gst + g + 1) - a0;
-        double A[GMAX][2 * GMAX];
-        for (int a = 0; a < m; ++a) {
-            const int4 va = G::ld(ids + a0 + a);
-            const double4_32a na = ld_n64<G>(n64 + a0 + a);
-            for (int b = 0; b < m; ++b) {
-                const int4 vb = G::ld(ids + a0 + b);
-                const double4_32a nb = ld_n64<G>(n64 + a0 + b);
-                double w = inv_mass_of(va.x, nA, wA, wB);
-                const int fa[3] = {va.y, va.z, va.w}, fb[3] = {vb.y, vb.z, vb.w};
-                for (int p = 0; p < 3; ++p)
-                    for (int q = 0; q < 3; ++q)
-                        if (fa[p] == fb[q]) w += inv_mass_of(fa[p], nA, wA, wB) / 9.0;
-                A[a][b] = (na.x * nb.x + na.y * nb.y + na.z * nb.z) * w;
-                A[a][GMAX + b] = a == b ? 1.0 : 0.0;
+__device__ __forceinline__ void group_inverses(int gi, int step, int n, const int *gst, const int4 *ids,
+                                               const double4_32a *n64, int nA, const float *wA,
+                                               const float *wB, R *pinv, const int *perm = nullptr) {
+    static_assert(GMAX == 4, "a quad holds one block");
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, a = lane & 3, q0 = lane & ~3;
+    for (; gi < n; gi += step) {
+        const int g = gi + (lane >> 2);
+        const int a0 = g < n ? G::ld(gst + g) : 0, m = g < n ? G::ld(gst + g + 1) - a0 : 0;
+        const int mmax = (int)__reduce_max_sync(ALL, (unsigned)m);
+        int4 v = make_int4(0, 0, 0, 0);
+        double4_32a nv = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+        double w0 = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;  // inverse masses of x0 and the face
+        if (a < m) {
+            const int t = perm ? G::ld(perm + a0 + a) : a0 + a;
+            v = G::ld(ids + t);
+            nv = ld_n64<G>(n64 + t);
+            w0 = inv_mass_of(v.x, nA, wA, wB);
+            w1 = inv_mass_of(v.y, nA, wA, wB);
+            w2 = inv_mass_of(v.z, nA, wA, wB);
+            w3 = inv_mass_of(v.w, nA, wA, wB);
+        }
+        auto ninth = [](double w) { return w == 1.0 ? 1.0 / 9.0 : w / 9.0; };  // no division without masses
+        const double d1 = ninth(w1), d2 = ninth(w2), d3 = ninth(w3);
+        double A[2 * GMAX], diag = 0.0;
+#pragma unroll
+        for (int b = 0; b < GMAX; ++b) {
+            A[b] = 0.0;
+            A[GMAX + b] = 0.0;
+            if (b >= mmax) continue;
+            const int fb[3] = {__shfl_sync(ALL, v.y, q0 + b), __shfl_sync(ALL, v.z, q0 + b),
+                               __shfl_sync(ALL, v.w, q0 + b)};
+            const double bx = __shfl_sync(ALL, nv.x, q0 + b), by = __shfl_sync(ALL, nv.y, q0 + b),
+                         bz = __shfl_sync(ALL, nv.z, q0 + b);
+            if (a >= m || b >= m) continue;
+            double w = w0;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (v.y == fb[q]) w += d1;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (v.z == fb[q]) w += d2;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (v.w == fb[q]) w += d3;
+            A[b] = (nv.x * bx + nv.y * by + nv.z * bz) * w;
+            A[GMAX + b] = a == b ? 1.0 : 0.0;
+            if (a == b) diag = fabs(A[b]);
+        }
+        double dmax = fmax(diag, __shfl_xor_sync(ALL, diag, 1));
+        dmax = fmax(dmax, __shfl_xor_sync(ALL, dmax, 2));
+        bool ok = true;
+#pragma unroll
+        for (int c = 0; c < GMAX; ++c) {
+            if (c >= mmax) break;
+            const double mag = fabs(A[c]);
+            int piv = c;
+            double best = __shfl_sync(ALL, mag, q0 + c);
+#pragma unroll
+            for (int r = c + 1; r < GMAX; ++r) {
+                const double o = __shfl_sync(ALL, mag, q0 + r);
+                if (r < m && o > best) {
+                    piv = r;
+                    best = o;
+                }
+            }
+            if (c < m && !(best > 1e-12 * dmax)) ok = false;
+            const bool act = c < m && ok;
+            if (__any_sync(ALL, act && piv != c)) {
+                const int from = q0 + (act && a == c ? piv : act && a == piv ? c : a);
+#pragma unroll
+                for (int q = 0; q < 2 * GMAX; ++q) A[q] = __shfl_sync(ALL, A[q], from);
+            }
+            if (act && a == c) {
+                const double inv = 1.0 / A[c];
+#pragma unroll
+                for (int q = 0; q < 2 * GMAX; ++q) A[q] *= inv;
+            }
+            if (mmax == 1) break;  // no other rows
+            const double f = A[c];
+#pragma unroll
+            for (int q = 0; q < 2 * GMAX; ++q) {
+                const double p = __shfl_sync(ALL, A[q], q0 + c);
+                if (act && a != c) A[q] -= f * p;
             }
         }
-        // Gauss-Jordan with partial pivoting; a (near-)singular block falls
-        // back to the inverse of its diagonal
-        bool ok = true;
-        double dmax = 0.0;
-        for (int a = 0; a < m; ++a) dmax = fmax(dmax, fabs(A[a][a]));
-        for (int c = 0; c < m && ok; ++c) {
-            int piv = c;
-            for (int r = c + 1; r < m; ++r)
-                if (fabs(A[r][c]) > fabs(A[piv][c])) piv = r;
-            if (!(fabs(A[piv][c]) > 1e-12 * dmax)) { ok = false; break; }
-            if (piv != c)
-                for (int q = 0; q < 2 * GMAX; ++q) {
-                    double tmp = A[c][q];
-                    A[c][q] = A[piv][q];
-                    A[piv][q] = tmp;
-                }
-            const double inv = 1.0 / A[c][c];
-            for (int q = 0; q < 2 * GMAX; ++q) A[c][q] *= inv;
-            for (int r = 0; r < m; ++r)
-                if (r != c) {
-                    const double f = A[r][c];
-                    for (int q = 0; q < 2 * GMAX; ++q) A[r][q] -= f * A[c][q];
-                }
-        }
-        for (int a = 0; a < m; ++a) {
-            double row[GMAX] = {0.0, 0.0, 0.0, 0.0};
-            if (ok) {
-                for (int b = 0; b < m; ++b) row[b] = A[a][GMAX + b];
-            } else {
-                // diagonal fallback computed from the untouched inputs
-                const int4 va = G::ld(ids + a0 + a);
-                double w = inv_mass_of(va.x, nA, wA, wB) +
-                           (inv_mass_of(va.y, nA, wA, wB) + inv_mass_of(va.z, nA, wA, wB) +
-                            inv_mass_of(va.w, nA, wA, wB)) / 9.0;
-                row[a] = w > 0.0 ? 1.0 / w : 0.0;
+        if (a < m) {
+            double row[GMAX];
+#pragma unroll
+            for (int b = 0; b < GMAX; ++b) row[b] = A[GMAX + b];
+            if (!ok) {
+                const double w = w0 + (w1 + w2 + w3) / 9.0, x = w > 0.0 ? 1.0 / w : 0.0;
+#pragma unroll
+                for (int b = 0; b < GMAX; ++b) row[b] = a == b ? x : 0.0;
             }
             store_inv_row(pinv + a0 + a, row);
         }
@@ -1018,9 +1064,9 @@ __global__ void k_group_inverse(const int *d_ng, const int *gst, const int4 *ids
                                 const double4_32a *n64, int nA, const float *wA, const float *wB,
                                 float4 *pinv) {
     HFCR_PDL_WAIT();
-    const int ng = *d_ng;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x)
-        group_inverse_one<PlainLd>(g, gst, ids, n64, nA, wA, wB, pinv);
+    const int nw = blockDim.x >> 5;
+    group_inverses<PlainLd>(8 * (int)(blockIdx.x * nw + (threadIdx.x >> 5)), 8 * (int)gridDim.x * nw,
+                            *d_ng, gst, ids, n64, nA, wA, wB, pinv);
 }
 
 // float64 residual r = b - J M^-1 J^T lam of one zone (the float64 normals;
@@ -2298,8 +2344,8 @@ __global__ void __launch_bounds__(ZONE64_THREADS) k_cg_zone64(const int *d_nz, Z
         const double bb = zone_start<CtaGroup>(a, s0, k, redd);  // lam = 0 on the zone's rows
         // the zone's block-Jacobi inverses in float64 (a block of nearly
         // dependent rows has a large inverse that float32 would not hold)
-        for (int gi = threadIdx.x; gi < G; gi += blockDim.x)
-            group_inverse_one<PlainLd>(g0 + gi, a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv64);
+        group_inverses<PlainLd>(g0 + 8 * (int)(threadIdx.x >> 5), 8 * (int)(blockDim.x >> 5), g0 + G,
+                                a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv64);
         double *r = g.r + s0, *p = g.p + s0, *sv = g.s + s0, *w = g.w + s0, *zz = g.z + s0;
         double *x = a.lam + s0, *u = a.u64 + 3 * (size_t)j0;
         for (int t = threadIdx.x; t < k; t += blockDim.x) {
@@ -2875,13 +2921,14 @@ __global__ void k_displace(const int *d_U, const int *seg, const int *cval, cons
 // rows sharing x0 and the inverses of their blocks.  It computes exactly
 // what the multi-kernel sequence of build_vertex_csr computes (the same
 // stable sorts, the same union-find roots, hence the same arrays), in one
-// launch instead of about twenty-five.  The elementwise phases run on every
-// CTA taking part, separated by bounded grid-wide barriers, and data
-// written by another CTA is read through L2.  Up to SETUP_SMALL_K stencils
-// few CTAs take part (one per 1,024 entries) and the first CTA alone runs
-// the sorts, the union-find (in shared memory) and the scans between two
-// barriers; above, every CTA takes part in those too (the multi-CTA sort,
-// union-find in global memory, the two-level scan).
+// launch instead of about twenty-five.  Up to SETUP_CTA_K stencils k_setup_cta
+// has built the arrays and only the rows are left (setup_rows).  The
+// elementwise phases run on every CTA taking part, separated by bounded
+// grid-wide barriers, and data written by another CTA is read through L2.  Up
+// to SETUP_SMALL_K stencils few CTAs take part (one per 1,024 entries) and the
+// first CTA alone runs the sorts, the union-find (in shared memory) and the
+// scans between two barriers; above, every CTA takes part in those too (the
+// multi-CTA sort, union-find in global memory, the two-level scan).
 // ---------------------------------------------------------------------------
 constexpr int SETUP_SMALL_K = 8192;  // 4k <= SMALL_N sort keys, 32 KB of parents
 constexpr int SETUP_SCAN_CHUNK = 4096;
@@ -2913,6 +2960,7 @@ struct SetupArgs {
     int *d_n4, *d_U, *d_nz, *d_ng;
     unsigned *hist, *tot, *bar;
     uint32_t *status;
+    int indexed;  // k_setup_cta ran before: up to SETUP_CTA_K stencils only the rows are left
 };
 
 // the CTAs taking part (blockIdx.x < parts) and their barrier
@@ -3098,9 +3146,8 @@ constexpr int SETUP_READY = 1;
 // the inverse blocks of CTAs first .. first + n - 1 (consecutive groups on
 // different CTAs)
 __device__ __forceinline__ void setup_inverses(const SetupArgs &a, int first, int n) {
-    const int ng = __ldcg(a.d_ng);
-    for (int gi = threadIdx.x * n + (blockIdx.x - first); gi < ng; gi += n * TPB)
-        group_inverse_one<L2Ld>(gi, a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv);
+    group_inverses<L2Ld>(8 * ((int)(threadIdx.x >> 5) * n + (int)blockIdx.x - first), 8 * n * (TPB / 32),
+                         __ldcg(a.d_ng), a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv);
 }
 
 // a CTA not taking part in the phases (first = the first such CTA): waits
@@ -3316,6 +3363,433 @@ __device__ bool setup_phases(SetupSync &g, const SetupArgs &a, int k, SortSmem &
     return true;
 }
 
+// ---------------------------------------------------------------------------
+// The setup of up to SETUP_CTA_K stencils without a sort of the entries: one
+// CTA of 1,024 threads builds every index array in shared memory, then the
+// rows (gather and inverse blocks, all elementwise) go to a grid.
+//   - A hash table of the touched vertices; each vertex's first entry (its
+//     smallest 4 s + role) is its head, and a stencil and the heads of its
+//     vertices are of one zone (sweeps of hooking roots; a zone's root is its
+//     smallest stencil).
+//   - Zones numbered by their roots (scan), rows placed by a stable counting
+//     sort of the zone numbers (8 bits a pass, ranks by warp matches).
+//   - Vertices numbered in the order of their heads among the placed rows,
+//     which is zone by zone; one scan gives the number and the start of each
+//     one's list, a cursor places the entries, and every list is sorted (each
+//     entry counts the smaller ones; a warp, or, past SETUP_LONG entries, a
+//     bitmap by the whole CTA), so the result does not depend on the order of
+//     the atomics.
+// The numbering of a zone's vertices differs from the sorted one of the other
+// paths; every sum over a list or a zone's rows keeps its order, hence its
+// bits.  Bound by the latency of about 25 barriers and shared-memory phases:
+// 1,955 rows in 21 zones 186 -> 37 us, 107 rows 85 -> 12 us, 1,219 rows in one
+// zone 100 -> 24 us, and 13 us more for the rows' grid, against the
+// cooperative launch's sorts.
+// ---------------------------------------------------------------------------
+constexpr int SETUP_CTA_K = 4096;
+constexpr int SETUP_CTA_THREADS = 1024;
+constexpr int SETUP_ROWS = SETUP_CTA_K / SETUP_CTA_THREADS;  // rows of a thread at most
+constexpr int SETUP_TAB = 21 * SETUP_CTA_K / 4;              // slots: 1.3 x the entries
+constexpr int SETUP_SHORT = 16, SETUP_LONG = 128;            // list lengths
+static_assert(SETUP_TAB <= 0x8000, "a slot and a flag fit 16 bits");
+static_assert(4 * SETUP_CTA_K <= 0x8000, "entries fit 16 bits");
+
+struct SetupCtaSmem {
+    // a slot's vertex, then its head, then its list's length, then the vertex's
+    // number and its list's cursor
+    unsigned tab[SETUP_TAB];
+    uint16_t slot[4 * SETUP_CTA_K];  // of each entry; bit 15: the entry is its vertex's head
+    union {
+        int par[SETUP_CTA_K];
+        uint16_t hist[256 * 32];     // digit-major, one column per warp
+        uint16_t cval[4 * SETUP_CTA_K];
+    } u;
+    uint16_t key[2][SETUP_CTA_K], src[2][SETUP_CTA_K];
+    uint16_t pos[SETUP_CTA_K];
+    uint16_t start[4 * SETUP_CTA_K + 2];  // of each vertex's list
+    unsigned bits[4 * SETUP_CTA_K / 32];
+    unsigned ws[2][32];
+    int n_list;
+};
+
+// exclusive scan (sum, or maximum) over the CTA; flip alternates the two
+// rows of ws, so that one barrier is enough
+template <bool MAX>
+__device__ __forceinline__ unsigned setup_cta_scan(unsigned v, unsigned (*ws)[32], int &flip, unsigned &total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto op = [](unsigned a, unsigned b) { return MAX ? max(a, b) : a + b; };
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x = op(x, y);
+    }
+    if (lane == 31) ws[flip][w] = x;
+    __syncthreads();
+    unsigned y = ws[flip][lane];
+    flip ^= 1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) y = op(y, t);
+    }
+    total = __shfl_sync(0xffffffffu, y, 31);
+    unsigned before = __shfl_sync(0xffffffffu, y, w ? w - 1 : 0);
+    if (w == 0) before = 0;
+    unsigned ex = __shfl_up_sync(0xffffffffu, x, 1);
+    if (lane == 0) ex = 0;
+    return op(before, ex);
+}
+
+__global__ void __launch_bounds__(SETUP_CTA_THREADS, 1) k_setup_cta(SetupArgs a) {
+    HFCR_PDL_WAIT();
+    extern __shared__ float4 smem4[];
+    SetupCtaSmem &m = *(SetupCtaSmem *)smem4;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int k = max(0, min(*a.d_k, a.cap));
+    if (tid < 2) a.bar[tid] = 0u;  // k_setup's barrier counter and ready flag
+    if (k > SETUP_CTA_K) return;
+    const int n4 = 4 * k;
+    if (tid == 0) *a.d_n4 = n4;
+    if (k == 0) {
+        if (tid == 0) { *a.d_U = 0; *a.d_nz = 0; *a.d_ng = 0; }
+        return;
+    }
+    // a thread's rows: per consecutive ones
+    const int per = (k + SETUP_CTA_THREADS - 1) / SETUP_CTA_THREADS;
+    const int r0 = tid * per, nr = max(0, min(per, k - r0));
+    const unsigned T = 21u * (unsigned)k / 4u;
+    int flip = 0;
+    int4 q[SETUP_ROWS];
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i)
+        q[i] = i < nr ? a.ids_raw[r0 + i] : make_int4(0, 0, 0, 0);
+    for (int i = tid; i < (int)T; i += SETUP_CTA_THREADS) m.tab[i] = 0xffffffffu;
+    __syncthreads();
+    // the table (Fibonacci hashing, linear probing; reads first, since most
+    // entries find their vertex there)
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const unsigned v[4] = {(unsigned)q[i].x, (unsigned)q[i].y, (unsigned)q[i].z, (unsigned)q[i].w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            unsigned h = __umulhi(v[r] * 0x9e3779b1u, T);
+            while (true) {  // ends: there are more slots than entries
+                unsigned old = *(volatile unsigned *)&m.tab[h];
+                if (old == 0xffffffffu) old = atomicCAS(&m.tab[h], 0xffffffffu, v[r]);
+                if (old == 0xffffffffu || old == v[r]) break;
+                if (++h == T) h = 0;
+            }
+            m.slot[4 * (r0 + i) + r] = (uint16_t)h;
+        }
+    }
+    __syncthreads();
+    for (int e = 4 * r0; e < 4 * (r0 + nr); ++e) m.tab[m.slot[e]] = 0xffffffffu;
+    __syncthreads();
+    for (int e = 4 * r0; e < 4 * (r0 + nr); ++e) atomicMin(&m.tab[m.slot[e]], (unsigned)e);
+    __syncthreads();
+    // a stencil's first parent: the smallest of its vertices' heads.  Then
+    // sweeps: every tree hooks the roots its stencils' vertices reach under
+    // the smallest of them, until no vertex joins two trees (parents are
+    // smaller than children, so a zone's root is its smallest stencil)
+    uint16_t *snap = m.start;  // the roots of a sweep
+    unsigned hd[SETUP_ROWS][2];
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        unsigned lo = r0 + i, h[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int e = 4 * (r0 + i) + r;
+            const unsigned sl = m.slot[e];
+            h[r] = m.tab[sl];
+            if ((int)h[r] == e) m.slot[e] = (uint16_t)(sl | 0x8000u);
+            h[r] >>= 2;
+            lo = min(lo, h[r]);
+        }
+        m.u.par[r0 + i] = (int)lo;
+        hd[i][0] = h[0] | h[1] << 16;
+        hd[i][1] = h[2] | h[3] << 16;
+    }
+    __syncthreads();
+    while (true) {
+#pragma unroll
+        for (int i = 0; i < SETUP_ROWS; ++i)
+            if (i < nr) snap[r0 + i] = (uint16_t)uf_find_s((volatile int *)m.u.par, r0 + i);
+        __syncthreads();
+        bool hooked = false;
+#pragma unroll
+        for (int i = 0; i < SETUP_ROWS; ++i) {
+            if (i >= nr) break;
+            const int x[5] = {snap[r0 + i], snap[hd[i][0] & 0xffffu], snap[hd[i][0] >> 16],
+                              snap[hd[i][1] & 0xffffu], snap[hd[i][1] >> 16]};
+            const int lo = min(min(min(x[0], x[1]), min(x[2], x[3])), x[4]);
+#pragma unroll
+            for (int r = 0; r < 5; ++r)
+                if (x[r] > lo) {
+                    atomicMin(&m.u.par[x[r]], lo);
+                    hooked = true;
+                }
+        }
+        if (!__syncthreads_or(hooked)) break;
+    }
+    // zones in the order of their roots; the list lengths start at 0
+    int root[SETUP_ROWS];
+    unsigned cnt = 0;
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        root[i] = -1;
+        if (i >= nr) continue;
+        root[i] = snap[r0 + i];
+        cnt += root[i] == r0 + i;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned sl = m.slot[4 * (r0 + i) + r];
+            if (sl & 0x8000u) m.tab[sl & 0x7fffu] = 0u;
+        }
+    }
+    unsigned nz;
+    unsigned zi = setup_cta_scan<false>(cnt, m.ws, flip, nz);
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i)
+        if (root[i] >= 0 && root[i] == r0 + i) m.pos[r0 + i] = (uint16_t)zi++;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        m.key[0][r0 + i] = m.pos[root[i]];
+        m.src[0][r0 + i] = (uint16_t)(r0 + i);
+    }
+    // the list lengths
+    for (int e = 4 * r0; e < 4 * (r0 + nr); ++e) atomicAdd(&m.tab[m.slot[e] & 0x7fffu], 1u);
+    int f = 0;
+    for (int shift = 0; (int)nz - 1 >> shift; shift += 8) {
+        __syncthreads();  // the keys; par and the previous counts are no longer read
+        for (int i = tid; i < 256 * 32 / 2; i += SETUP_CTA_THREADS) ((unsigned *)m.u.hist)[i] = 0u;
+        __syncthreads();
+        // rows 32 per * w + 32 i + lane of warp w
+        unsigned dig[SETUP_ROWS], rank[SETUP_ROWS];
+#pragma unroll
+        for (int i = 0; i < SETUP_ROWS; ++i) {
+            if (i >= per) break;
+            const int t = 32 * (per * w + i) + lane;
+            dig[i] = t < k ? (m.key[f][t] >> shift) & 255u : 256u;
+            const unsigned same = __match_any_sync(0xffffffffu, dig[i]);
+            const unsigned before = dig[i] < 256u ? m.u.hist[dig[i] * 32 + w] : 0u;
+            rank[i] = before + __popc(same & ((1u << lane) - 1u));
+            __syncwarp();
+            if (dig[i] < 256u && lane == __ffs(same) - 1)
+                m.u.hist[dig[i] * 32 + w] = (uint16_t)(before + __popc(same));
+            __syncwarp();
+        }
+        __syncthreads();
+        uint4 h = ((uint4 *)m.u.hist)[tid];
+        unsigned hv[8] = {h.x & 0xffffu, h.x >> 16, h.y & 0xffffu, h.y >> 16,
+                          h.z & 0xffffu, h.z >> 16, h.w & 0xffffu, h.w >> 16};
+        unsigned sum = 0, all;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sum += hv[i];
+        unsigned at = setup_cta_scan<false>(sum, m.ws, flip, all);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const unsigned c = hv[i];
+            hv[i] = at;
+            at += c;
+        }
+        ((uint4 *)m.u.hist)[tid] = make_uint4(hv[0] | hv[1] << 16, hv[2] | hv[3] << 16,
+                                              hv[4] | hv[5] << 16, hv[6] | hv[7] << 16);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SETUP_ROWS; ++i) {
+            if (i >= per) break;
+            const int t = 32 * (per * w + i) + lane;
+            if (t >= k) continue;
+            const unsigned d = m.u.hist[dig[i] * 32 + w] + rank[i];
+            m.key[f ^ 1][d] = m.key[f][t];
+            m.src[f ^ 1][d] = m.src[f][t];
+        }
+        f ^= 1;
+    }
+    __syncthreads();
+    // rows: zone, source, the groups of rows sharing x0 (GMAX rows at most)
+    const uint16_t *key = m.key[f], *src = m.src[f];
+    unsigned last_run = 0, heads = 0;  // this thread's last run start + 1; its vertices and entries
+    unsigned run[SETUP_ROWS];
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const int t = r0 + i, sr = src[t], z = key[t];
+        const bool first = t == 0 || key[t - 1] != z;
+        const unsigned x0 = m.slot[4 * sr] & 0x7fffu;
+        q[i] = a.ids_raw[sr];
+        a.szone[t] = z;
+        a.zsrc[t] = sr;
+        if (first) a.zs[z] = t;
+        if (first || (m.slot[4 * src[t - 1]] & 0x7fffu) != x0) last_run = (unsigned)t + 1u;
+        run[i] = last_run;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned sl = m.slot[4 * sr + r];
+            if (sl & 0x8000u) heads += 0x10000u + m.tab[sl & 0x7fffu];
+        }
+    }
+    unsigned total;
+    const unsigned run_before = setup_cta_scan<true>(last_run, m.ws, flip, total);
+    cnt = 0;
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const int t = r0 + i, rs = (int)(run[i] ? run[i] : run_before) - 1;
+        run[i] = (t - rs) % GMAX == 0;
+        cnt += run[i];
+    }
+    unsigned ng, Un;
+    unsigned gi = setup_cta_scan<false>(cnt, m.ws, flip, ng);
+    const unsigned base = setup_cta_scan<false>(heads, m.ws, flip, Un);
+    const int U = (int)(Un >> 16);
+    unsigned at = base;  // vertex number << 16 | list start
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const int t = r0 + i, sr = src[t], z = key[t];
+        const bool first = t == 0 || key[t - 1] != z;
+        if (run[i]) {
+            a.gst[gi] = t;
+            if (first) a.zg[z] = (int)gi;
+            ++gi;
+        }
+        if (first) a.zv[z] = (int)(at >> 16);  // a zone's first entry is a head
+        const int v[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned sl = m.slot[4 * sr + r];
+            if (!(sl & 0x8000u)) continue;
+            const int j = (int)(at >> 16);
+            const unsigned c = m.tab[sl & 0x7fffu];
+            m.tab[sl & 0x7fffu] = at;
+            a.seg[j] = (int)(at & 0xffffu);
+            m.start[j] = (uint16_t)(at & 0xffffu);
+            a.gvert[j] = v[r];
+            const float *wm = v[r] < a.nA ? a.wA : a.wB;
+            a.winv[j] = wm ? wm[v[r] < a.nA ? v[r] : v[r] - a.nA] : 1.0f;
+            at += 0x10000u + c;
+        }
+    }
+    if (tid == 0) {
+        a.zs[nz] = k;
+        a.gst[ng] = k;
+        a.zg[nz] = (int)ng;
+        a.seg[U] = n4;
+        a.zv[nz] = U;
+        *a.d_nz = (int)nz;
+        *a.d_ng = (int)ng;
+        *a.d_U = U;
+        m.start[U] = (uint16_t)n4;
+        m.n_list = 0;
+    }
+    __syncthreads();
+    // the entries into their vertices' lists
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const int t = r0 + i, sr = src[t];
+        int j[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned o = atomicAdd(&m.tab[m.slot[4 * sr + r] & 0x7fffu], 1u);
+            j[r] = (int)(o >> 16);
+            m.u.cval[o & 0xffffu] = (uint16_t)(4 * t + r);
+        }
+        q[i] = make_int4(j[0], j[1], j[2], j[3]);
+        a.vidx[t] = q[i];
+    }
+    __syncthreads();
+    // each list ascending: a short list's entries find their own ranks, a
+    // longer one is noted by its first entry to be placed
+#pragma unroll
+    for (int i = 0; i < SETUP_ROWS; ++i) {
+        if (i >= nr) break;
+        const int j[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int e = 4 * (r0 + i) + r, lo = m.start[j[r]], hi = m.start[j[r] + 1];
+            if (hi - lo <= SETUP_SHORT) {
+                int at = lo;
+                for (int x = lo; x < hi; ++x) at += (int)m.u.cval[x] < e;
+                a.v2[at] = e;
+            } else if ((int)m.u.cval[lo] == e) {
+                const int n = atomicAdd(&m.n_list, 1);  // at most 4 k / 17 lists
+                m.pos[2 * n] = (uint16_t)lo;
+                m.pos[2 * n + 1] = (uint16_t)hi;
+            }
+        }
+    }
+    __syncthreads();
+    const int nl = m.n_list;
+    for (int x = w; x < nl; x += 32) {
+        const int b = m.pos[2 * x], n = m.pos[2 * x + 1] - b;
+        if (n > SETUP_LONG) continue;
+        uint16_t c[SETUP_LONG / 32];
+        int rk[SETUP_LONG / 32];
+#pragma unroll
+        for (int i = 0; i < SETUP_LONG / 32; ++i) {
+            c[i] = lane + 32 * i < n ? m.u.cval[b + lane + 32 * i] : 0;
+            rk[i] = 0;
+        }
+        for (int y = 0; y < n; ++y) {
+            const uint16_t o = m.u.cval[b + y];
+#pragma unroll
+            for (int i = 0; i < SETUP_LONG / 32; ++i) rk[i] += o < c[i];
+        }
+#pragma unroll
+        for (int i = 0; i < SETUP_LONG / 32; ++i)
+            if (lane + 32 * i < n) a.v2[b + rk[i]] = c[i];
+    }
+    for (int x = 0; x < nl; ++x) {
+        const int b = m.pos[2 * x], n = m.pos[2 * x + 1] - b;
+        if (n <= SETUP_LONG) continue;
+        constexpr int W = 4 * SETUP_CTA_K / 32;
+        if (tid < W) m.bits[tid] = 0u;
+        __syncthreads();
+        for (int y = tid; y < n; y += SETUP_CTA_THREADS) {
+            const unsigned c = m.u.cval[b + y];
+            atomicOr(&m.bits[c >> 5], 1u << (c & 31));
+        }
+        __syncthreads();
+        unsigned word = tid < W ? m.bits[tid] : 0u, all;
+        unsigned o = (unsigned)b + setup_cta_scan<false>((unsigned)__popc(word), m.ws, flip, all);
+        while (word) {
+            a.v2[o++] = 32 * tid + __ffs(word) - 1;
+            word &= word - 1u;
+        }
+    }
+}
+
+// the rows of an indexed setup: gathered in the zones' order, and the
+// groups' inverse blocks (float64, from the rows as assembled)
+__device__ __forceinline__ void setup_rows(const SetupArgs &a, int k) {
+    // a warp's share: consecutive warps of work on different CTAs (float64 is
+    // slow on one SM)
+    const int nw = gridDim.x * (blockDim.x >> 5), wi = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (int t = 32 * wi + (threadIdx.x & 31); t < k; t += 32 * nw) {
+        const int src = a.zsrc[t];
+        a.ids[t] = a.ids_raw[src];
+        a.n64[t] = a.n64_raw[src];
+        a.n32[t] = a.n32_raw[src];
+        a.b[t] = a.b_raw[src];
+    }
+    group_inverses<PlainLd>(8 * wi, 8 * nw, *a.d_ng, a.gst, a.ids_raw, a.n64_raw, a.nA,
+                            a.wA, a.wB, a.pinv, a.zsrc);
+}
+
+constexpr int SETUP_ROWS_THREADS = 64;
+
+__global__ void __launch_bounds__(SETUP_ROWS_THREADS) k_setup_rows(SetupArgs a) {
+    HFCR_PDL_WAIT();
+    setup_rows(a, max(0, min(*a.d_k, a.cap)));
+}
+
 union SetupSmem {
     SortSmem sort;
     int par[SETUP_SMALL_K];
@@ -3324,6 +3798,10 @@ union SetupSmem {
 __global__ void __launch_bounds__(TPB) k_setup(SetupArgs a) {
     HFCR_PDL_WAIT();
     const int k = max(0, min(*a.d_k, a.cap));
+    if (a.indexed && k <= SETUP_CTA_K) {
+        setup_rows(a, k);
+        return;
+    }
     // CTAs taking part: every CTA on large inputs, one per 1,024 entries on
     // small ones (the others leave at once; every CTA reads the same count)
     unsigned parts = gridDim.x;
@@ -3355,6 +3833,7 @@ void assemble(const MeshPair &mp, const hfcr_stencil *st, const int *d_k, int ca
 // dynamic shared memory granted to the zone CG kernels (0: the global-memory
 // path runs); set once per process, outside any stream capture
 static int g_fast_smem = -1, g_zone_pair_smem = 0, g_warp_zone_smem = 0;
+static bool g_setup_cta = false;  // k_setup_cta has its shared memory
 static bool g_cluster_ok = false;  // k_cg_zone_cl can be launched on this device
 
 void solver_init() {
@@ -3369,6 +3848,9 @@ void solver_init() {
     g_warp_zone_smem = cudaFuncSetAttribute(k_cg_zone_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             wz) == cudaSuccess ? wz : 0;
     if (!g_warp_zone_smem) cudaGetLastError();
+    g_setup_cta = cudaFuncSetAttribute(k_setup_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       sizeof(SetupCtaSmem)) == cudaSuccess;
+    if (!g_setup_cta) cudaGetLastError();
     // the cluster solver of large zones: its shared memory, and whether a
     // cluster of CL such CTAs fits on this device at all
     g_cluster_ok = false;
@@ -3413,11 +3895,15 @@ static int setup_grid_max() {
     return g[dev];
 }
 
-// the whole setup as one cooperative launch; false when it cannot be launched
+// the whole setup: up to SETUP_CTA_K stencils by k_setup_cta and a grid over
+// the rows, above in one cooperative launch (which is then also the rows'
+// grid, when the count turns out small); false when it cannot be launched
 static bool build_setup_fused(const MeshPair &mp, const int *d_k, int cap, SolveBuffers &sb,
                               SortTemp &t, int *d_n4, uint32_t *d_status, cudaStream_t s) {
-    int grid = setup_grid_max();
-    if (grid <= 0 || !d_status || t.max_blocks < 3) return false;
+    if (!d_status || t.max_blocks < 3) return false;
+    const bool small = g_setup_cta && cap <= SETUP_CTA_K;
+    int grid = small ? 1 : setup_grid_max();
+    if (grid <= 0) return false;
     const int tiles = (4 * cap + TILE - 1) / TILE;
     if (grid > tiles) grid = tiles > 0 ? tiles : 1;
     SetupArgs a;
@@ -3468,14 +3954,24 @@ static bool build_setup_fused(const MeshPair &mp, const int *d_k, int cap, Solve
     a.tot = t.hist + 256 * (size_t)(t.max_blocks - 1);
     a.bar = t.hist + 256 * (size_t)(t.max_blocks - 2);
     a.status = d_status;
-    cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), s);  // barrier counter, ready flag
+    a.indexed = g_setup_cta ? 1 : 0;
+    if (g_setup_cta) {
+        { launch_pdl(k_setup_cta, 1, SETUP_CTA_THREADS, sizeof(SetupCtaSmem), s, a); note_launch(); }
+    } else {
+        cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), s);  // barrier counter, ready flag
+    }
+    sb.cval_s = a.v2;
+    if (small) {
+        { launch_pdl(k_setup_rows, (4 * cap + SETUP_ROWS_THREADS - 1) / SETUP_ROWS_THREADS, SETUP_ROWS_THREADS,
+                     0, s, a); note_launch(); }
+        return true;
+    }
     void *args[] = {&a};
     if (cudaLaunchCooperativeKernel((const void *)k_setup, grid, TPB, args, 0, s) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     note_launch();
-    sb.cval_s = a.v2;
     return true;
 }
 
