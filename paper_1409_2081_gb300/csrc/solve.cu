@@ -2327,17 +2327,219 @@ __device__ __forceinline__ void zone64_precond(const ZoneArgs &a, int s0, int g0
     }
 }
 
-// rescue: only the zones whose recorded |r|^2 (the mixed solver's) misses
+// A zone's float64 CG with everything an iteration touches in shared memory
+// and the rows' vectors in registers.  float64 runs at two lanes per clock and
+// SM, half a lane in each quarter: a warp's operation takes 64 cycles, a
+// division about a thousand, and an iteration is a chain of them.  So a
+// warp's sums are halved, warps without rows or vertices take no part, and one
+// warp forms the step's scalars for all, the reciprocals of the step before
+// while the others update their rows.  Products stay J M^-1 (J^T z): with the
+// merged matrix of solve_zone_rows an iteration was a quarter shorter, but
+// the rounding of its entries cost an ill-conditioned zone two digits of dx.
+// Every result is bit for bit that of the vectors in global memory (the same
+// tree of sums over RESCUE_NT threads, correctly rounded divisions).  A zone
+// of 97 rows (93 iterations) 853 -> 584 us, one of 354 rows (75) 1,175 -> 835.
+// False when the zone does not fit (nothing done); otherwise lambda is stored and the count in its.
+constexpr int RESCUE_THREADS = 512, RESCUE_NT = ZONE64_THREADS, RESCUE_ROWS = 4;  // threads with rows, rows each
+constexpr int RESCUE_VT = RESCUE_THREADS - 32;                                   // threads with vertices
+constexpr int RESCUE_SMEM = 220 * 1024;
+
+// a / b from y = 1 / b rounded to nearest (Markstein, 1990): a y, corrected by
+// its residual, is a / b rounded to nearest
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+    const double q = a * y, c = fma(fma(-b, q, a), y, q);
+    return isfinite(q) && fabs(q) > 1e-280 && fabs(a) > 1e-280 ? c : a / b;
+}
+
+__device__ __forceinline__ double warp_halve3d(double a, double b, double c) {  // as warp_halve3
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, q = lane & 8;
+    const double x = (h ? c : a) + __shfl_xor_sync(0xffffffffu, h ? a : c, 16);
+    const double y = (h ? 0.0 : b) + __shfl_xor_sync(0xffffffffu, h ? b : 0.0, 16);
+    double t = (q ? y : x) + __shfl_xor_sync(0xffffffffu, q ? x : y, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+__device__ __forceinline__ bool zone64_staged(const ZoneArgs &a, int z, char *base, int bytes, double bb,
+                                              int maxit, double *red, double *sc, int &its) {
+    constexpr int NT = RESCUE_NT, RPT = RESCUE_ROWS;
+    static_assert(NT == 256 && RESCUE_VT == 480, "the named barriers below; eight warps' sums");
+    const int tid = threadIdx.x, lane = tid & 31, wq = tid >> 5;
+    const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
+    const int j0 = a.zv[z], U = a.zv[z + 1] - j0;
+    const int g0 = a.zg[z], G = a.zg[z + 1] - g0;
+    const int e0 = a.seg[j0];
+    // layout: blocks' inverse rows | normals | z, -z / 3 | r | u | vidx | winv | seg | cval | groups
+    const long long need = 98ll * k + 30ll * U + 64;
+    if (k > RPT * NT || need > bytes) return false;
+    double4_32a *pS = (double4_32a *)base;
+    double *nS = (double *)(pS + k), *zS = nS + 3 * k, *rS = zS + 2 * k, *uS = rS + k;
+    ushort4 *vidx = (ushort4 *)(uS + 3 * U);
+    float *winv = (float *)(vidx + k);
+    uint16_t *seg = (uint16_t *)(winv + U);
+    uint16_t *cval = seg + U + 1;
+    uint16_t *grp = cval + 4 * k;
+    const double third = 1.0 / 3.0;
+    for (int t = tid; t < k; t += RESCUE_THREADS) {
+        const int4 g = a.vidx[s0 + t];
+        vidx[t] = make_ushort4((unsigned short)(g.x - j0), (unsigned short)(g.y - j0),
+                               (unsigned short)(g.z - j0), (unsigned short)(g.w - j0));
+        const double4_32a n = a.n64[s0 + t];
+        nS[3 * t] = n.x;
+        nS[3 * t + 1] = n.y;
+        nS[3 * t + 2] = n.z;
+        pS[t] = a.pinv64[s0 + t];
+    }
+    for (int g = tid; g < G; g += RESCUE_THREADS) {  // each row's block: first row and size
+        const int b0 = a.gst[g0 + g] - s0, b1 = a.gst[g0 + g + 1] - s0;
+        for (int t = b0; t < b1; ++t) grp[t] = (uint16_t)(b0 << 3 | (b1 - b0));
+    }
+    for (int j = tid; j <= U; j += RESCUE_THREADS) seg[j] = (uint16_t)(a.seg[j0 + j] - e0);
+    for (int j = tid; j < U; j += RESCUE_THREADS) winv[j] = a.winv[j0 + j];
+    for (int e = tid; e < 4 * k; e += RESCUE_THREADS) cval[e] = (uint16_t)(a.cval[e0 + e] - 4 * s0);
+    __syncthreads();
+    its = 0;
+    if (tid >= RESCUE_VT) {
+        const double stop = a.rel_tol * a.rel_tol * bb;
+        double gamma = 1.0, alpha = 1.0, rg = 1.0, ra = 1.0;  // of the step before, and their reciprocals
+        for (bool first = true;; first = false) {
+            __syncthreads();  // the warps' sums
+            double t = red[4 * (lane & 7) + (lane >> 3)];
+#pragma unroll
+            for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            const double gn = __shfl_sync(0xffffffffu, t, 0), dn = __shfl_sync(0xffffffffu, t, 8),
+                         rn = __shfl_sync(0xffffffffu, t, 16);
+            double beta = 0.0;
+            if (first) {
+                alpha = gn / dn;
+            } else {
+                beta = div_by(gn, gamma, rg);
+                alpha = gn / (dn - div_by(beta * gn, alpha, ra));
+            }
+            const bool go = its < maxit && rn > stop && alpha > 0.0 && isfinite(alpha);
+            if (lane == 0) {
+                sc[0] = alpha;
+                sc[1] = beta;
+                *(int *)(sc + 2) = go;
+            }
+            __syncthreads();
+            if (!go) break;
+            ++its;
+            gamma = gn;
+            rg = 1.0 / gn;
+            ra = 1.0 / alpha;
+        }
+    } else {
+        double r[RPT], x[RPT], p[RPT], s[RPT], w[RPT], zz[RPT];
+        const bool rows = tid < NT;
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            const int t = tid + v * NT;
+            r[v] = rows && t < k ? a.b64[s0 + t] : 0.0;
+            x[v] = p[v] = s[v] = w[v] = zz[v] = 0.0;
+        }
+        while (true) {
+            if (rows) {  // z = P^-1 r
+#pragma unroll
+                for (int v = 0; v < RPT; ++v)
+                    if (tid + v * NT < k) rS[tid + v * NT] = r[v];
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll
+                for (int v = 0; v < RPT; ++v) {
+                    const int t = tid + v * NT;
+                    if (t >= k) continue;
+                    const int b0 = grp[t] >> 3, m = grp[t] & 7;
+                    double rr[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) rr[q] = q < m ? rS[b0 + q] : 0.0;
+                    const double4_32a pi = pS[t];
+                    zz[v] = pi.x * rr[0] + pi.y * rr[1] + pi.z * rr[2] + pi.w * rr[3];
+                    zS[2 * t] = zz[v];
+                    zS[2 * t + 1] = -third * zz[v];
+                }
+            }
+            asm volatile("bar.sync 2, 480;" ::: "memory");
+            for (int j = tid; j < U; j += RESCUE_VT) {  // u = M^-1 J^T z
+                double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+                const int e1 = seg[j + 1];
+#pragma unroll 2
+                for (int e = seg[j]; e < e1; ++e) {
+                    const int c = cval[e], sl = c >> 2;
+                    const double ps = zS[2 * sl + ((c & 3) ? 1 : 0)];
+                    a0 += ps * nS[3 * sl];
+                    a1 += ps * nS[3 * sl + 1];
+                    a2 += ps * nS[3 * sl + 2];
+                }
+                const double wv = (double)winv[j];
+                uS[3 * j] = wv * a0;
+                uS[3 * j + 1] = wv * a1;
+                uS[3 * j + 2] = wv * a2;
+            }
+            asm volatile("bar.sync 2, 480;" ::: "memory");
+            if (rows) {  // w = J u and the sums (r, z), (w, z), |r|^2
+                double t = 0.0;
+                if (wq * 32 < k) {
+                    double g = 0.0, d = 0.0, h = 0.0;
+#pragma unroll
+                    for (int v = 0; v < RPT; ++v) {
+                        const int t = tid + v * NT;
+                        if (t >= k) continue;
+                        const ushort4 i = vidx[t];
+                        const double *ux = uS + 3 * i.x, *ua = uS + 3 * i.y, *ub = uS + 3 * i.z, *uc = uS + 3 * i.w;
+                        const double nx = nS[3 * t], ny = nS[3 * t + 1], nz = nS[3 * t + 2];
+                        w[v] = nx * (ux[0] - (ua[0] + ub[0] + uc[0]) * third) +
+                               ny * (ux[1] - (ua[1] + ub[1] + uc[1]) * third) +
+                               nz * (ux[2] - (ua[2] + ub[2] + uc[2]) * third);
+                        g += r[v] * zz[v];
+                        d += w[v] * zz[v];
+                        h += r[v] * r[v];
+                    }
+                    t = warp_halve3d(g, d, h);
+                }
+                if ((lane & 7) == 0) red[4 * wq + (lane >> 3)] = t;
+            }
+            __syncthreads();
+            __syncthreads();  // the scalars
+            if (!*(volatile int *)(sc + 2)) break;
+            ++its;
+            const double al = sc[0], be = sc[1];
+            if (rows) {
+#pragma unroll
+                for (int v = 0; v < RPT; ++v) {
+                    if (tid + v * NT >= k) continue;
+                    p[v] = zz[v] + be * p[v];
+                    s[v] = w[v] + be * s[v];
+                    x[v] += al * p[v];
+                    r[v] -= al * s[v];
+                }
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < RPT; ++v)
+            if (rows && tid + v * NT < k) a.lam[s0 + tid + v * NT] = x[v];
+    }
+    __syncthreads();
+    return true;
+}
+
+// RESCUE: only the zones whose recorded |r|^2 (the mixed solver's) misses
 // the target, solved again from lam = 0 (zones on which the float32 runs
-// stopped reducing the float64 residual)
-__global__ void __launch_bounds__(ZONE64_THREADS) k_cg_zone64(const int *d_nz, ZoneArgs a,
-                                                              Zone64Scratch g, int maxit, int rescue) {
+// stopped reducing the float64 residual), staged where they fit; otherwise
+// every zone (several CTAs per SM), its vectors in global memory
+template <bool RESCUE>
+__global__ void __launch_bounds__(RESCUE ? RESCUE_THREADS : ZONE64_THREADS)
+    k_cg_zone64(const int *d_nz, ZoneArgs a, Zone64Scratch g, int maxit, int smem_bytes) {
     HFCR_PDL_WAIT();
-    __shared__ double red[3 * (ZONE64_THREADS / 32)];
-    __shared__ double redd[ZONE64_THREADS / 32];
+    extern __shared__ float4 smem4[];
+    constexpr int WARPS = (RESCUE ? RESCUE_THREADS : ZONE64_THREADS) / 32;
+    __shared__ double red[4 * WARPS];
+    __shared__ double redd[WARPS];
+    __shared__ double sc[3];
     const int nz = *d_nz;
     for (int z = blockIdx.x; z < nz; z += gridDim.x) {
-        if (rescue && a.zres[z] <= a.rel_tol * a.rel_tol * a.zbb[z]) continue;
+        if (RESCUE && a.zres[z] <= a.rel_tol * a.rel_tol * a.zbb[z]) continue;
         const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
         const int j0 = a.zv[z], U = a.zv[z + 1] - j0;
         const int g0 = a.zg[z], G = a.zg[z + 1] - g0;
@@ -2346,46 +2548,24 @@ __global__ void __launch_bounds__(ZONE64_THREADS) k_cg_zone64(const int *d_nz, Z
         // dependent rows has a large inverse that float32 would not hold)
         group_inverses<PlainLd>(g0 + 8 * (int)(threadIdx.x >> 5), 8 * (int)(blockDim.x >> 5), g0 + G,
                                 a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv64);
+        __syncthreads();  // the blocks, read by other threads below
         double *r = g.r + s0, *p = g.p + s0, *sv = g.s + s0, *w = g.w + s0, *zz = g.z + s0;
         double *x = a.lam + s0, *u = a.u64 + 3 * (size_t)j0;
-        for (int t = threadIdx.x; t < k; t += blockDim.x) {
-            r[t] = a.b64[s0 + t];
-            p[t] = 0.0;
-            sv[t] = 0.0;
-        }
-        __syncthreads();
-        zone64_precond(a, s0, g0, G, r, zz);
-        __syncthreads();
-        zone64_vertex(a, s0, j0, U, zz, u);
-        __syncthreads();
-        double ga = 0.0, de = 0.0, rh = 0.0;
-        for (int t = threadIdx.x; t < k; t += blockDim.x) {
-            const double wt = zone64_stencil(a, s0, j0, t, u);
-            w[t] = wt;
-            ga += r[t] * zz[t];
-            de += wt * zz[t];
-            rh += r[t] * r[t];
-        }
-        double gamma, delta, rho;
-        block_sum3d(ga, de, rh, red, gamma, delta, rho);
-        const double stop = a.rel_tol * a.rel_tol * bb;
-        double alpha = gamma / delta, beta = 0.0;
         int it = 0;
-        while (it < maxit && rho > stop && alpha > 0.0 && isfinite(alpha)) {
+        bool staged = false;
+        if constexpr (RESCUE) staged = zone64_staged(a, z, (char *)smem4, smem_bytes, bb, maxit, red, sc, it);
+        if (!staged) {
             for (int t = threadIdx.x; t < k; t += blockDim.x) {
-                const double pt = zz[t] + beta * p[t];
-                const double st = w[t] + beta * sv[t];
-                p[t] = pt;
-                sv[t] = st;
-                x[t] += alpha * pt;
-                r[t] -= alpha * st;
+                r[t] = a.b64[s0 + t];
+                p[t] = 0.0;
+                sv[t] = 0.0;
             }
             __syncthreads();
             zone64_precond(a, s0, g0, G, r, zz);
             __syncthreads();
             zone64_vertex(a, s0, j0, U, zz, u);
             __syncthreads();
-            ga = de = rh = 0.0;
+            double ga = 0.0, de = 0.0, rh = 0.0;
             for (int t = threadIdx.x; t < k; t += blockDim.x) {
                 const double wt = zone64_stencil(a, s0, j0, t, u);
                 w[t] = wt;
@@ -2393,13 +2573,41 @@ __global__ void __launch_bounds__(ZONE64_THREADS) k_cg_zone64(const int *d_nz, Z
                 de += wt * zz[t];
                 rh += r[t] * r[t];
             }
-            double gn, dn, rn;
-            block_sum3d(ga, de, rh, red, gn, dn, rn);
-            beta = gn / gamma;
-            alpha = gn / (dn - beta * gn / alpha);
-            gamma = gn;
-            rho = rn;
-            ++it;
+            double gamma, delta, rho;
+            block_sum3d(ga, de, rh, red, gamma, delta, rho);
+            const double stop = a.rel_tol * a.rel_tol * bb;
+            double alpha = gamma / delta, beta = 0.0;
+            it = 0;
+            while (it < maxit && rho > stop && alpha > 0.0 && isfinite(alpha)) {
+                for (int t = threadIdx.x; t < k; t += blockDim.x) {
+                    const double pt = zz[t] + beta * p[t];
+                    const double st = w[t] + beta * sv[t];
+                    p[t] = pt;
+                    sv[t] = st;
+                    x[t] += alpha * pt;
+                    r[t] -= alpha * st;
+                }
+                __syncthreads();
+                zone64_precond(a, s0, g0, G, r, zz);
+                __syncthreads();
+                zone64_vertex(a, s0, j0, U, zz, u);
+                __syncthreads();
+                ga = de = rh = 0.0;
+                for (int t = threadIdx.x; t < k; t += blockDim.x) {
+                    const double wt = zone64_stencil(a, s0, j0, t, u);
+                    w[t] = wt;
+                    ga += r[t] * zz[t];
+                    de += wt * zz[t];
+                    rh += r[t] * r[t];
+                }
+                double gn, dn, rn;
+                block_sum3d(ga, de, rh, red, gn, dn, rn);
+                beta = gn / gamma;
+                alpha = gn / (dn - beta * gn / alpha);
+                gamma = gn;
+                rho = rn;
+                ++it;
+            }
         }
         // the zone's true residual b - A lam (not the recurrence's)
         __syncthreads();
@@ -3833,6 +4041,7 @@ void assemble(const MeshPair &mp, const hfcr_stencil *st, const int *d_k, int ca
 // dynamic shared memory granted to the zone CG kernels (0: the global-memory
 // path runs); set once per process, outside any stream capture
 static int g_fast_smem = -1, g_zone_pair_smem = 0, g_warp_zone_smem = 0;
+static int g_rescue_smem = 0;  // of k_cg_zone64<true> (0: every zone on global memory)
 static bool g_setup_cta = false;  // k_setup_cta has its shared memory
 static bool g_cluster_ok = false;  // k_cg_zone_cl can be launched on this device
 
@@ -3848,6 +4057,9 @@ void solver_init() {
     g_warp_zone_smem = cudaFuncSetAttribute(k_cg_zone_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             wz) == cudaSuccess ? wz : 0;
     if (!g_warp_zone_smem) cudaGetLastError();
+    g_rescue_smem = cudaFuncSetAttribute(k_cg_zone64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         RESCUE_SMEM) == cudaSuccess ? RESCUE_SMEM : 0;
+    if (!g_rescue_smem) cudaGetLastError();
     g_setup_cta = cudaFuncSetAttribute(k_setup_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        sizeof(SetupCtaSmem)) == cudaSuccess;
     if (!g_setup_cta) cudaGetLastError();
@@ -4077,7 +4289,7 @@ void solve(const SolveParams &p, const MeshPair &mp, const int *d_k, int cap, So
         g64.r = sb.cg64; g64.p = sb.cg64 + cap; g64.s = sb.cg64 + 2 * (size_t)cap;
         g64.w = sb.cg64 + 3 * (size_t)cap; g64.z = sb.cg64 + 4 * (size_t)cap;
         int zg = cap < 4 * 152 ? cap : 4 * 152;
-        { launch_pdl(k_cg_zone64, zg, ZONE64_THREADS, 0, s, sb.d_nz, za, g64,
+        { launch_pdl(k_cg_zone64<false>, zg, ZONE64_THREADS, 0, s, sb.d_nz, za, g64,
                      p.max_cg_iters * p.max_refine, 0); note_launch(); }
         { launch_pdl(k_zone_final, 1, 256, 0, s, sb.d_nz, sb.r64, sb.q64, p.rel_tol, sb.dwork,
                      sb.iwork); note_launch(); }
@@ -4172,8 +4384,8 @@ void solve(const SolveParams &p, const MeshPair &mp, const int *d_k, int cap, So
         g64.r = sb.cg64; g64.p = sb.cg64 + cap; g64.s = sb.cg64 + 2 * (size_t)cap;
         g64.w = sb.cg64 + 3 * (size_t)cap; g64.z = sb.cg64 + 4 * (size_t)cap;
         int zr = cap < 152 ? cap : 152;
-        { launch_pdl(k_cg_zone64, zr, ZONE64_THREADS, 0, s, sb.d_nz, za, g64,
-                     p.max_cg_iters * p.max_refine, 1); note_launch(); }
+        { launch_pdl(k_cg_zone64<true>, zr, RESCUE_THREADS, g_rescue_smem, s, sb.d_nz, za, g64,
+                     p.max_cg_iters * p.max_refine, g_rescue_smem); note_launch(); }
     }
     { launch_pdl(k_zone_final, 1, 256, 0, s, sb.d_nz, sb.r64, sb.q64, p.rel_tol, sb.dwork,
                  sb.iwork); note_launch(); }
