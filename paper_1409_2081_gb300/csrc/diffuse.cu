@@ -61,12 +61,32 @@ __global__ void k_adj_fill(const int2 *edges, int ne, int nv, const int *ptr, in
     nbr[ptr[ed.y] + atomicAdd(&cur[ed.y], 1)] = ed.x;
 }
 
-// ascending order within each vertex's list (the fill order is arbitrary)
+// a list of at most N entries in registers: every entry's rank, one store each
+template <int N>
+__device__ __forceinline__ void adj_sort_regs(int *nbr, int d) {
+    int x[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = i < d ? nbr[i] : 0x7fffffff;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        int r = 0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) r += x[j] < x[i] || (j < i && x[j] == x[i]);
+        if (i < d) nbr[r] = x[i];
+    }
+}
+
+// ascending order within each vertex's list (the fill order is arbitrary).
+// Bound by the latency of the loads: all of a list's at once (262,144 vertices
+// of degree 6: 18 -> 9 us against an insertion sort in place, which the lists
+// past 16 entries keep).
 __global__ void k_adj_sort(const int *ptr, int nv, int *nbr) {
     HFCR_PDL_WAIT();
     int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nv) return;
     const int a = ptr[v], b = ptr[v + 1];
+    if (b - a <= 8) return adj_sort_regs<8>(nbr + a, b - a);
+    if (b - a <= 16) return adj_sort_regs<16>(nbr + a, b - a);
     for (int i = a + 1; i < b; ++i) {
         const int x = nbr[i];
         int j = i - 1;
