@@ -129,16 +129,15 @@ def measured_peak_hbm():
 
 # kernel -> (source files whose code lines it depends on, its ncu summary)
 KERNELS = {
-    "k_traverse": (("detect.cu", "predicates.cuh"), "k_traverse_frame_sequence.md"),
-    "k_traverse_batch": (("detect.cu", "predicates.cuh"), "k_traverse_batch.md"),
-    "k_band_cl": (("diffuse.cu",), "k_band_cl_frame_sequence.md"),
+    "k_broad": (("detect.cu", "predicates.cuh"), "k_broad_frame_sequence.md"),
+    "k_broad_batch": (("detect.cu", "predicates.cuh"), "k_broad_batch.md"),
+    "k_band_pipe": (("diffuse.cu",), "k_band_pipe_frame_sequence.md"),
     "k_cg_zone_pair": (("solve.cu",), "k_cg_zone_pair_cloth_torus.md"),
-    "k_refit": (("bvh.cu",), "k_refit_frame_sequence.md"),
     "k_cg_zone_big": (("solve.cu",), "k_cg_zone_big_frame_sequence.md"),
 }
 
 
-def kernel_source_hash(kernel: str = "k_traverse") -> str:
+def kernel_source_hash(kernel: str = "k_broad") -> str:
     """First 16 hex digits of the SHA-256 of the kernel's source files, code
     lines only (lines that are blank or hold only a // comment are left out,
     so a comment edit keeps a profile valid)."""
@@ -475,7 +474,7 @@ def cloth_torus(api, torch, dev, stream, flush, steps, warmup, timed, cpu=True):
            "ef_tests_per_s_bruteforce": round(info.stats.brute_force_equiv / (statistics.mean(ms) / 1e3), 1),
            "stage_ms_per_frame": stage_ms, "traverse_variant": variant, "variant_ms": variant_ms,
            "rooflines": {
-               "k_traverse": {"bound": "hbm", "achieved": round(alg_trav / (trav_ms * 1e-3) / 1e9, 2),
+               "k_broad": {"bound": "hbm", "achieved": round(alg_trav / (trav_ms * 1e-3) / 1e9, 2),
                               "peak": peak, "peak_kind": kind, "unit": "GB/s",
                               "frac": round(alg_trav / (trav_ms * 1e-3) / 1e9 / peak, 6),
                               "alg_bytes_per_launch": alg_trav, "avg_launch_ms": round(trav_ms, 5)},
@@ -566,9 +565,9 @@ def batched(api, torch, dev, steps, warmup, timed, cpu=True):
            "pairs": P, "stencils": int(info.total_stencils),
            "ef_tests_per_s_bruteforce": round(info.stats.brute_force_equiv / (statistics.mean(ms) / 1e3), 1),
            "stage_ms_per_step": {k: round(val[0] / n_it, 4) for k, val in prof.items()},
-           "roofline": {"kernel": "k_traverse", "bound": "hbm", "achieved": round(ach, 2),
+           "roofline": {"kernel": "k_broad + k_narrow", "bound": "hbm", "achieved": round(ach, 2),
                         "peak": peak, "peak_kind": kind, "unit": "GB/s", "frac": round(ach / peak, 5),
-                        "traffic": profiled_traffic("k_traverse_batch"),
+                        "traffic": profiled_traffic("k_broad_batch"),
                         "alg_bytes_per_launch": alg, "avg_launch_ms": round(trav_ms / max(1, trav_n), 5),
                         "traverse_variant": variant, "variant_ms": variant_ms}}
     if cpu:
@@ -990,17 +989,17 @@ def main():
     alg_zb = int(116 * zb_rows + 8 * zb_verts)
     ach_zb = alg_zb / (zb_ms * 1e-3) / 1e9
     roof = {
-        "k_traverse": {"kernel": "k_traverse (BVH traversal + exact narrow phase)", "bound": "hbm",
-                       "achieved": round(ach_trav, 2), "peak": peak, "peak_kind": peak_kind,
-                       "unit": "GB/s", "frac": round(ach_trav / peak, 5),
-                       "traffic": profiled_traffic("k_traverse"), "alg_bytes_per_launch": alg_trav,
-                       "avg_launch_ms": round(trav_ms, 5), "launches_timed": prof["traverse"][1]},
-        "k_band_cl": {"kernel": "k_band_cl (harmonic diffusion: CG on the band Laplacian on one "
-                                "thread-block cluster; k_band_cg, the grid-wide form, takes bands "
-                                "beyond the cluster's capacity)", "bound": "hbm",
+        "k_broad": {"kernel": "k_broad + k_narrow (BVH traversal, exact narrow phase)", "bound": "hbm",
+                    "achieved": round(ach_trav, 2), "peak": peak, "peak_kind": peak_kind,
+                    "unit": "GB/s", "frac": round(ach_trav / peak, 5),
+                    "traffic": profiled_traffic("k_broad"), "alg_bytes_per_launch": alg_trav,
+                    "avg_launch_ms": round(trav_ms, 5), "launches_timed": prof["traverse"][1]},
+        "k_band_pipe": {"kernel": "k_band_pipe (harmonic diffusion: CG on the band Laplacian on one "
+                                "thread-block cluster; k_band_cl and k_band_cg, the grid-wide form, "
+                                "take the bands beyond its capacity)", "bound": "hbm",
                       "achieved": round(ach_band, 3), "peak": peak, "peak_kind": peak_kind,
                       "unit": "GB/s", "frac": round(ach_band / peak, 7),
-                      "traffic": profiled_traffic("k_band_cl"), "alg_bytes_per_launch": alg_band,
+                      "traffic": profiled_traffic("k_band_pipe"), "alg_bytes_per_launch": alg_band,
                       "avg_launch_ms": round(band_ms, 5), "launches_timed": prof["band_cg"][1],
                       "band_vertices_mean": round(nb_mean, 1), "cg_iters_mean": round(band_iters, 2),
                       "us_per_cg_iter": round(1e3 * band_ms / band_iters, 3) if band_iters else None},
@@ -1020,7 +1019,7 @@ def main():
     }
     # the headline roofline: the single kernel with the most time per frame
     # in the profiled pass (the traversal, the band CG, the large-zone solver)
-    kernel_ms = {"k_traverse": prof["traverse"][0] / F, "k_band_cl": prof["band_cg"][0] / F,
+    kernel_ms = {"k_broad": prof["traverse"][0] / F, "k_band_pipe": prof["band_cg"][0] / F,
                  "k_cg_zone_big": prof["zone_big"][0] / F}
     top = max(kernel_ms, key=kernel_ms.get)
     roofline = dict(roof[top], ms_per_frame=round(kernel_ms[top], 4),
