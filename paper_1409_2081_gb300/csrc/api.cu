@@ -319,20 +319,23 @@ hfcr_status check_pair(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B) {
 
 hfcr_status read_back(hfcr_ctx *ctx, cudaStream_t s);
 
-// Unique edges of a triangle list into out (room for 3 n_tris), their number
-// to *ne; synchronises.  C_SLOW is zero before.
-hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts, int *out, int slot,
-                         int *ne, cudaStream_t s) {
+// Unique edges of a triangle list, their number to *ne; synchronises.  They
+// go to out by the buckets and to own by the sort (each with room for
+// 3 n_tris of them, 8-byte aligned); *at says which.  With an index out of
+// range nothing went to out.  C_SLOW is zero before.
+hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts, int *out, int *own,
+                         int slot, const int **at, int *ne, cudaStream_t s) {
     // the buckets' words fit the vertex scratch of the reservation; a caller
     // with more vertices than reserved takes the sort
     bool fast = n_tris > 0 && n_verts > 0 &&
                 bucket_words(n_verts) * sizeof(int) <= sizeof(double) * 6 * (size_t)ctx->max_verts;
     for (;; fast = false) {
+        *at = fast ? out : own;
         if (fast)
             build_edges(tris, n_tris, n_verts, out, ctx->d_cnt + slot, ctx->d_cnt + C_SLOW, ctx->ekeys,
                         ctx->ekeys_alt, (int *)ctx->field_alt, ctx->d_status, s);
         else
-            build_edges_sorted(tris, n_tris, n_verts, out, ctx->d_cnt + slot, ctx->ekeys, ctx->ekeys_alt,
+            build_edges_sorted(tris, n_tris, n_verts, own, ctx->d_cnt + slot, ctx->ekeys, ctx->ekeys_alt,
                                ctx->eflags, ctx->sort, ctx->d_status, s);
         hfcr_status st = read_back(ctx, s);
         if (st) return st;
@@ -340,6 +343,19 @@ hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts
     }
     *ne = ctx->h_cnt[slot];
     return HFCR_OK;
+}
+
+// Whether a kernel of this context may store pairs of ints to p: device
+// memory of this GPU, 8-byte aligned (an int32_t * need only be a multiple
+// of 4).
+bool pair_stores_ok(const hfcr_ctx *ctx, const int *p) {
+    if ((uintptr_t)p & 7) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == ctx->device;
 }
 
 // Edges of mesh `which` (0 = A, 1 = B): the caller's, or built into the
@@ -351,9 +367,8 @@ hfcr_status mesh_edges(hfcr_ctx *ctx, const hfcr_mesh *m, int which, const int *
         *ne = m->n_edges;
         return HFCR_OK;
     }
-    *edges = ctx->edges[which];
-    return derive_edges(ctx, m->tris, m->n_tris, m->n_verts, ctx->edges[which],
-                        which ? C_EDGES_B : C_EDGES_A, ne, s);
+    return derive_edges(ctx, m->tris, m->n_tris, m->n_verts, ctx->edges[which], ctx->edges[which],
+                        which ? C_EDGES_B : C_EDGES_A, edges, ne, s);
 }
 
 struct DetectPlan {
@@ -1086,14 +1101,17 @@ hfcr_status hfcr_build_edges(hfcr_ctx *ctx, const int32_t *tris, int32_t n_tris,
     if (n_tris == 0) return HFCR_OK;
     hfcr_status st = reset_words(ctx, s);
     if (st) return st;
-    // straight into the caller's buffer when it holds any possible count
-    const bool direct = cap >= 3 * (int64_t)n_tris;
+    // by the buckets straight into the caller's buffer when it holds any
+    // possible count and takes their stores; otherwise through the context's
+    const bool direct = cap >= 3 * (int64_t)n_tris && pair_stores_ok(ctx, out);
+    const int *at = nullptr;
     int ne = 0;
-    if ((st = derive_edges(ctx, tris, n_tris, n_verts, direct ? out : ctx->edges[0], C_EDGES_A, &ne, s)))
+    if ((st = derive_edges(ctx, tris, n_tris, n_verts, direct ? out : ctx->edges[0], ctx->edges[0], C_EDGES_A,
+                           &at, &ne, s)))
         return st;
     *n_out = ne;
     if (ne > cap) return fail(ctx, HFCR_ERR_CAPACITY, "%d edges exceed cap %lld", ne, (long long)cap);
-    if (direct) return HFCR_OK;
+    if (at == out) return HFCR_OK;
     CK(cudaMemcpyAsync(out, ctx->edges[0], sizeof(int) * 2 * (size_t)ne, cudaMemcpyDeviceToDevice, s));
     CK(cudaStreamSynchronize(s));
     return HFCR_OK;

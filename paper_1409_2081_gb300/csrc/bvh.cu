@@ -238,9 +238,12 @@ __device__ __forceinline__ int sort_unique(int *list, int n) {
 }
 
 __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_edges(const int *ptr, int nv, int *bucket, int2 *edges,
-                                                             int *d_count, unsigned long long *state,
-                                                             int *ticket, uint32_t *status) {
+                                                             int *d_count, const int *slow,
+                                                             unsigned long long *state, int *ticket,
+                                                             uint32_t *status) {
     HFCR_PDL_WAIT();
+    // a void result is not written (edges may be the caller's own buffer)
+    if (*slow || (*(volatile uint32_t *)status & ST_BAD_INDEX)) return;
     __shared__ int list[BUCKET_SM], out[BUCKET_SM];
     __shared__ unsigned char owner[BUCKET_SM];
     __shared__ unsigned ws[BUCKET_TPB / 32], base;
@@ -722,7 +725,7 @@ void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *
     { launch_pdl(k_bucket_fill, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, (const int *)cnt,
                  (const unsigned char *)rank, bucket); note_launch(); }
     { launch_pdl(k_bucket_edges, vb, BUCKET_TPB, 0, s, (const int *)cnt, n_verts, bucket, (int2 *)edges_out,
-                 d_count, state + nscan, tickets + 1, d_status); note_launch(); }
+                 d_count, (const int *)d_slow, state + nscan, tickets + 1, d_status); note_launch(); }
 }
 
 void check_segments(const int *segs, int nseg, const hfcr_mesh &A, const hfcr_mesh &B,

@@ -158,9 +158,10 @@ void scan_flags_dev(unsigned *flags, const int *d_n, int cap, int *d_total, Sort
 // ---- topology ----
 // Unique sorted edges of a triangle list, by buckets of the smaller vertex
 // (n_tris, n_verts >= 1).  Scratch: keys/keys_alt of 3 * n_tris u64 and
-// bucket_words(n_verts) words, 8-byte aligned.  *d_slow (zero before) is set
-// when a vertex has too many: the result is then void, build_edges_sorted
-// gives it.
+// bucket_words(n_verts) words, both 8-byte aligned, as edges_out is.  *d_slow
+// (zero before) is set when a vertex has too many: build_edges_sorted then
+// gives the result.  After that, and after an index out of range, neither
+// edges_out nor *d_count has been written.
 void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
                  unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
                  cudaStream_t s);
