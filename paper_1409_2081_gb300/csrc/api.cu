@@ -393,8 +393,14 @@ hfcr_status plan_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, b
         pl.segs = ctx->d_segs;
         pl.nseg = 1;
     }
-    if (dir0 && A->n_tris > 0 && (st = mesh_edges(ctx, A, 0, &pl.edges[0], &pl.ne[0], s))) return st;
-    if (dir1 && B->n_tris > 0 && (st = mesh_edges(ctx, B, 1, &pl.edges[1], &pl.ne[1], s))) return st;
+    if ((dir0 && A->n_tris > 0 && (st = mesh_edges(ctx, A, 0, &pl.edges[0], &pl.ne[0], s))) ||
+        (dir1 && B->n_tris > 0 && (st = mesh_edges(ctx, B, 1, &pl.edges[1], &pl.ne[1], s)))) {
+        // an index out of range: bad positions are reported before it, as
+        // they are when the edges are the caller's
+        if (st != HFCR_ERR_ARG) return st;
+        validate_pair(*A, *B, ctx->d_status, s);
+        return read_back(ctx, s);
+    }
     for (int d = 0; d < 2; ++d) {
         if (!pl.edges[d] || pl.ne[d] <= 0) continue;
         if (ctx->eorder_src[d] == pl.edges[d] && ctx->eorder_n[d] == pl.ne[d]) continue;
