@@ -917,6 +917,22 @@ __device__ __forceinline__ void warp_sums(T (&t)[K]) {
     for (int k = 0; k < K; ++k) t[k] = __shfl_sync(0xffffffffu, t[k], 0);
 }
 
+// barrier of the CTAs that work
+__device__ __forceinline__ void bcl_sync(cgx::cluster_group &cl, int ncta) {
+    if (ncta > 1) cl.sync();
+    else __syncthreads();
+}
+
+// A CTA's shared memory may be stored to once that CTA runs: every CTA that
+// works arrives before it sets its vertices up, and waits before its first
+// stores to the others (one pair, with no other cluster barrier between).
+__device__ __forceinline__ void bcl_arrive(cgx::cluster_group &cl, int ncta) {
+    if (ncta > 1) cl.barrier_arrive();
+}
+__device__ __forceinline__ void bcl_started(cgx::cluster_group &cl, int ncta) {
+    if (ncta > 1) cl.barrier_wait();
+}
+
 // the K sums of v over the cluster into out (shared, identical in every
 // CTA): warp sums, warp 0 folds the warps' values into this CTA's sums and
 // stores them into every CTA's receive slots (recv[par][rank], remote
@@ -924,12 +940,6 @@ __device__ __forceinline__ void warp_sums(T (&t)[K]) {
 // received sums in rank order (lane q holds CTA q's).  A parity's slots are
 // rewritten two calls later, after every CTA has passed the barrier that
 // follows its reads.
-// barrier of the CTAs that work
-__device__ __forceinline__ void bcl_sync(cgx::cluster_group &cl, int ncta) {
-    if (ncta > 1) cl.sync();
-    else __syncthreads();
-}
-
 template <typename T, int K, bool SYNC_END = true, int THREADS = BCL_THREADS>
 __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K], T *scr, T *recv,
                                          T *const *recv_of, int par, int rank, int ncta, T *out) {
@@ -1065,6 +1075,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
     if (n > ncta * PIPE_CAP) return;  // the same n in every CTA
     if (n < ncta * BCL_PER) ncta = n > BCL_PER ? (n + BCL_PER - 1) / BCL_PER : 1;
     if (rank >= ncta) return;
+    bcl_arrive(cl, ncta);
     extern __shared__ float4 bsm[];
     __shared__ BclState st;
     const int chunk = n > 0 ? (n + ncta - 1) / ncta : 1;
@@ -1186,6 +1197,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
         __syncthreads();
         pd ^= 1;
     };
+    bcl_started(cl, ncta);
     sums64();
     int act = 0;  // coordinates not yet converged (bit c), the same in every thread
 #pragma unroll
@@ -1410,6 +1422,7 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
     int ncta = (int)cl.num_blocks();
     if (n < ncta * BCL_PER) ncta = n > BCL_PER ? (n + BCL_PER - 1) / BCL_PER : 1;
     if (rank >= ncta) return;
+    bcl_arrive(cl, ncta);
     const int chunk = n > 0 ? (n + ncta - 1) / ncta : 1;
     const int lo = rank * chunk;
     const int cnt = n - lo < chunk ? (n - lo > 0 ? n - lo : 0) : chunk;
@@ -1434,6 +1447,7 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
         xq[li] = z4;
     }
     int pf = 0, pd = 0;  // parities of the float and float64 receive slots
+    bcl_started(cl, ncta);
     bcl_sums<double, 3>(cl, dl, st.scrd, &st.recvd[0][0][0], st.recvd_of, pd, rank, ncta, st.sumsd);
     pd ^= 1;
     int act = 0;  // coordinates not yet converged (bit c), the same in every thread
