@@ -340,6 +340,7 @@ hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts
         hfcr_status st = read_back(ctx, s);
         if (st) return st;
         if (!fast || !ctx->h_cnt[C_SLOW]) break;
+        CK(cudaMemsetAsync(ctx->d_cnt + C_SLOW, 0, sizeof(int), s));  // the other mesh's result may be good
     }
     *ne = ctx->h_cnt[slot];
     return HFCR_OK;
