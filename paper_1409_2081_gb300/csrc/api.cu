@@ -327,20 +327,24 @@ hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts
                          int slot, const int **at, int *ne, cudaStream_t s) {
     // the buckets' words fit the vertex scratch of the reservation; a caller
     // with more vertices than reserved takes the sort
-    bool fast = n_tris > 0 && n_verts > 0 &&
-                bucket_words(n_verts) * sizeof(int) <= sizeof(double) * 6 * (size_t)ctx->max_verts;
-    for (;; fast = false) {
-        *at = fast ? out : own;
-        if (fast)
-            build_edges(tris, n_tris, n_verts, out, ctx->d_cnt + slot, ctx->d_cnt + C_SLOW, ctx->ekeys,
+    bool buckets = n_tris > 0 && n_verts > 0 &&
+                   bucket_words(n_verts) * sizeof(int) <= sizeof(double) * 6 * (size_t)ctx->max_verts;
+    bool hubs = bucket_hubs_first(n_tris);
+    while (true) {
+        *at = buckets ? out : own;
+        if (buckets)
+            build_edges(tris, n_tris, n_verts, hubs, out, ctx->d_cnt + slot, ctx->d_cnt + C_SLOW, ctx->ekeys,
                         ctx->ekeys_alt, (int *)ctx->field_alt, ctx->d_status, s);
         else
             build_edges_sorted(tris, n_tris, n_verts, own, ctx->d_cnt + slot, ctx->ekeys, ctx->ekeys_alt,
                                ctx->eflags, ctx->sort, ctx->d_status, s);
         hfcr_status st = read_back(ctx, s);
         if (st) return st;
-        if (!fast || !ctx->h_cnt[C_SLOW]) break;
-        CK(cudaMemsetAsync(ctx->d_cnt + C_SLOW, 0, sizeof(int), s));  // the other mesh's result may be good
+        if (!buckets || !ctx->h_cnt[C_SLOW]) break;
+        // the next form, and the other mesh, start from a clear word
+        CK(cudaMemsetAsync(ctx->d_cnt + C_SLOW, 0, sizeof(int), s));
+        buckets = !hubs;
+        hubs = true;
     }
     *ne = ctx->h_cnt[slot];
     return HFCR_OK;

@@ -133,27 +133,59 @@ __global__ void k_write_edges(const unsigned long long *keys, const unsigned *po
 //
 // Four kernels instead of a radix sort of the 3 n_tris (v0, v1) keys: the
 // half-edges are counted per v0 (each keeps the rank the counter gave it), the
-// counts scanned, the v1 placed, and each vertex's few v1 sorted and made
-// unique in shared memory by one thread.  A vertex that is v0 of more than
-// BUCKET_MAX half-edges (a fan; a manifold mesh has some twelve) raises
-// *slow: the caller then takes the sort (build_edges_sorted), which does not
-// care.  Both scans are single-pass: a CTA publishes its sum and looks back
-// over its predecessors' (tickets in starting order, so they are running).
+// counts scanned, the v1 placed, and each vertex's v1 sorted and made unique.
+// The few of an ordinary vertex (a manifold mesh has some twelve) by one
+// thread in shared memory; with HUBS up to BUCKET_WARP by a warp (ranks), and
+// the list of a hub (a fan, a pole) by the CTA through a bitmap.  Whatever the
+// form does not take raises *slow: without HUBS a vertex of more than
+// BUCKET_SHORT half-edges, with them a block of vertices that has more long
+// lists than the sort would cost, or a vertex of more half-edges than a rank
+// holds.  The caller then tries the next form, at last the sort
+// (build_edges_sorted), which does not care.  Both scans are single-pass: a
+// CTA publishes its sum and looks back over its predecessors' (tickets in
+// starting order, so they are running).
 // 522,242 triangles: 166 us of kernels by the sort (five passes of scattered
-// 8-byte keys), 43 by buckets.
-constexpr int BUCKET_MAX = 128;
-constexpr int BUCKET_SM = 4096;          // v1 of one CTA's vertices kept in shared memory
+// 8-byte keys), 45 by buckets; whole calls 158 and 55 us, and 59 with HUBS,
+// which costs nothing that shows up to BUCKET_HUBS_TRIS.
+// With a pole of 200 half-edges, 10,000 triangles: 238 us by the sort, 40 with
+// HUBS; of 1,024, 262,144 triangles: 112 by the sort, 82 by both tries.  A call
+// that ends at the sort has paid about 20 us for the tries (a fan of 20,000
+// triangles 106 us, 85 by the sort alone).
+constexpr int BUCKET_SHORT = 32;         // sorted by one thread: 256 moves of some 30 cycles
+constexpr int BUCKET_WARP = 128;         // by a warp: n^2 / 32 comparisons
+constexpr int BUCKET_RANK = 65535;       // a hub's half-edges at most
+constexpr int BUCKET_HUBS_TRIS = 100000; // triangles of a mesh whose first try has HUBS
+constexpr int BUCKET_SM = 3968;          // v1 of one CTA's vertices kept in shared memory (six CTAs per SM)
 constexpr int BUCKET_TPB = TPB;
 constexpr int BUCKET_SCAN = 2048;        // counts per CTA of the scan
+static_assert(BUCKET_SCAN / BUCKET_TPB * 32 == BUCKET_TPB, "a warp of the scan has the counts of one CTA of k_bucket_edges");
 
+// Cycles, roughly, that a CTA of k_bucket_edges spends on a list of n half-
+// edges beyond an ordinary one's, one of its eight warps (measured: 780 at 34,
+// 3,700 at 120) or the whole CTA (5,500 at 1,000, more where the ids spread over
+// further passes of the bitmap), and what the sort costs more
+// than the buckets do, their own start and the read-back among it: 60 vertices
+// of 34 half-edges in a block 61 us either way, one of 30,000 85.
+__device__ __forceinline__ unsigned bucket_cost(unsigned n, unsigned passes) {
+    return n <= (unsigned)BUCKET_WARP ? 600 + n * n / 5 : 15000 * passes - 12500 + 3 * n;
+}
+__device__ __forceinline__ unsigned bucket_cost_limit(unsigned n_tris) { return 100000 + n_tris / 8; }
+
+template <bool HUBS>
+struct BucketRank { typedef unsigned char T; };
+template <>
+struct BucketRank<true> { typedef uint16_t T; };
+
+template <bool HUBS>
 __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_count(const int *tris, int nt, int nv, int *cnt,
-                                                             unsigned char *rank, int *slow,
+                                                             typename BucketRank<HUBS>::T *rank, int *slow,
                                                              uint32_t *status) {
     HFCR_PDL_WAIT();
     const int t = blockIdx.x * BUCKET_TPB + threadIdx.x;
+    const unsigned live = __ballot_sync(0xffffffffu, t < nt);
     if (t >= nt) return;
     const int v[3] = {tris[3 * t], tris[3 * t + 1], tris[3 * t + 2]};
-    int r[3];
+    int u[3], r[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         int a = v[k], b = v[(k + 1) % 3];
@@ -161,18 +193,41 @@ __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_count(const int *tris, in
             atomicOr(status, ST_BAD_INDEX);
             a = b = 0;
         }
-        r[k] = atomicAdd(cnt + min(a, b), 1);
+        u[k] = min(a, b);
     }
+    bool hubs = false;
+    if constexpr (HUBS) {
+        // around a hub a warp's triangles all have it: one addition for its two
+        // half-edges of each
+        const int hub = min(u[0], min(u[1], u[2])), first = __ffs(live) - 1;
+        const int hub0 = __shfl_sync(live, hub, first);
+        hubs = __all_sync(live, hub == hub0 && (u[0] == hub) + (u[1] == hub) + (u[2] == hub) == 2);
+        if (hubs) {
+            const int lane = threadIdx.x & 31;
+            int base = 0;
+            if (lane == first) base = atomicAdd(cnt + hub, 2 * __popc(live));
+            base = __shfl_sync(live, base, first) + 2 * __popc(live & ((1u << lane) - 1u));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r[k] = u[k] == hub ? base++ : atomicAdd(cnt + u[k], 1);
+        }
+    }
+    if (!hubs) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) r[k] = atomicAdd(cnt + u[k], 1);
+    }
+    constexpr int most = HUBS ? BUCKET_RANK : BUCKET_SHORT;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        if (r[k] >= BUCKET_MAX) *slow = 1;
-        rank[3 * t + k] = (unsigned char)min(r[k], 255);
+        if (r[k] >= most) *slow = 1;
+        rank[3 * t + k] = (typename BucketRank<HUBS>::T)min(r[k], most);
     }
 }
 
 // cnt[0 .. n) -> exclusive offsets in place, the total to cnt[n]
-__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_scan(int *cnt, int n, unsigned long long *state,
-                                                            int *ticket, uint32_t *status) {
+template <bool HUBS>
+__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_scan(int *cnt, int n, int nt, int *slow,
+                                                            unsigned long long *state, int *ticket,
+                                                            uint32_t *status) {
     HFCR_PDL_WAIT();
     __shared__ int cta;
     __shared__ unsigned ws[BUCKET_TPB / 32], base;
@@ -192,6 +247,18 @@ __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_scan(int *cnt, int n, uns
         const unsigned b = lookback(state, cta, total, status);
         if (threadIdx.x == 0) base = b;
     }
+    if constexpr (HUBS) {  // meanwhile: the long lists of one CTA of k_bucket_edges
+        unsigned cost = 0;
+        if (sum > (unsigned)BUCKET_SHORT) {
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (v[k] > (unsigned)BUCKET_SHORT) cost += bucket_cost(v[k], (unsigned)n / (32 * BUCKET_SM) + 1);
+        }
+        if (__any_sync(0xffffffffu, cost != 0)) {
+            cost = __reduce_add_sync(0xffffffffu, cost);
+            if ((threadIdx.x & 31) == 0 && cost > bucket_cost_limit(nt)) *slow = 1;
+        }
+    }
     __syncthreads();
     e += base;
 #pragma unroll
@@ -202,18 +269,20 @@ __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_scan(int *cnt, int n, uns
     }
 }
 
+template <bool HUBS>
 __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_fill(const int *tris, int nt, int nv, const int *ptr,
-                                                            const unsigned char *rank, int *bucket) {
+                                                            const typename BucketRank<HUBS>::T *rank, const int *slow, int *bucket) {
     HFCR_PDL_WAIT();
     const int t = blockIdx.x * BUCKET_TPB + threadIdx.x;
     if (t >= nt) return;
     const int v[3] = {tris[3 * t], tris[3 * t + 1], tris[3 * t + 2]};
+    const int r[3] = {rank[3 * t], rank[3 * t + 1], rank[3 * t + 2]};
+    if (*slow) return;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         int a = v[k], b = v[(k + 1) % 3];
         if ((unsigned)a >= (unsigned)nv || (unsigned)b >= (unsigned)nv) a = b = 0;
-        const int r = rank[3 * t + k];
-        if (r < BUCKET_MAX) bucket[ptr[min(a, b)] + r] = max(a, b);
+        bucket[ptr[min(a, b)] + r[k]] = max(a, b);
     }
 }
 
@@ -237,30 +306,181 @@ __device__ __forceinline__ int sort_unique(int *list, int n) {
     return m;
 }
 
-__global__ void __launch_bounds__(BUCKET_TPB) k_bucket_edges(const int *ptr, int nv, int *bucket, int2 *edges,
-                                                             int *d_count, const int *slow,
-                                                             unsigned long long *state, int *ticket,
-                                                             uint32_t *status) {
+// One warp: src[0 .. n) ascending to tmp, then without repeats to dst (which
+// may be src or tmp); returns the length
+__device__ __forceinline__ int warp_sort_unique(const int *src, int n, int *tmp, int *dst) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {  // an entry's place: the smaller ones, and equal ones before it
+        const int x = src[i];
+        int r = 0;
+#pragma unroll 4
+        for (int q = 0; q < n; ++q) {
+            const int y = src[q];
+            r += y < x || (y == x && q < i);
+        }
+        tmp[r] = x;
+    }
+    __syncwarp();
+    int m = 0, last = -1;
+#pragma unroll 1
+    for (int q = 0; q < n; q += 32) {  // never writes past what it has read
+        const int y = q + lane < n ? tmp[q + lane] : -1;
+        int prev = __shfl_up_sync(0xffffffffu, y, 1);
+        if (lane == 0) prev = last;
+        const bool keep = q + lane < n && y != prev;
+        const unsigned k = __ballot_sync(0xffffffffu, keep);
+        if (keep) dst[m + __popc(k & ((1u << lane) - 1u))] = y;
+        m += __popc(k);
+        last = __shfl_sync(0xffffffffu, y, 31);
+        __syncwarp();
+    }
+    return m;
+}
+
+// The CTA: src[0 .. n) ascending and without repeats to dst, through a bitmap
+// of bits words (as many passes as its range needs); returns the length
+__device__ __forceinline__ int cta_sort_unique(const int *src, int n, int *dst, unsigned *bits, unsigned *ws,
+                                               int *range) {
+    constexpr int SPAN = 32 * BUCKET_SM;
+    if (threadIdx.x == 0) {
+        range[0] = 0x7fffffff;
+        range[1] = 0;
+    }
+    __syncthreads();
+    int lo = 0x7fffffff, hi = 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += BUCKET_TPB) {
+        const int x = src[i];
+        lo = min(lo, x);
+        hi = max(hi, x);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(range, lo);
+        atomicMax(range + 1, hi);
+    }
+    __syncthreads();
+    const int first = range[0] & ~31, last = range[1];
+    unsigned m = 0;
+    for (long long b = first; b <= last; b += SPAN) {
+        const int words = (int)min((last - b) / 32 + 1, (long long)BUCKET_SM);
+        for (int i = threadIdx.x; i < words; i += BUCKET_TPB) bits[i] = 0u;
+        __syncthreads();
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n; i += BUCKET_TPB) {
+            const unsigned x = (unsigned)src[i] - (unsigned)b;
+            if (x < (unsigned)SPAN) atomicOr(bits + (x >> 5), 1u << (x & 31));
+        }
+        __syncthreads();
+        const int per = (words + BUCKET_TPB - 1) / BUCKET_TPB, i0 = min((int)threadIdx.x * per, words);
+        const int i1 = min(i0 + per, words);
+        unsigned c = 0, total;
+        for (int i = i0; i < i1; ++i) c += __popc(bits[i]);
+        unsigned at = m + cta_scan(c, ws, total);
+        for (int i = i0; i < i1; ++i)
+            for (unsigned y = bits[i]; y; y &= y - 1u) dst[at++] = (int)b + 32 * i + __ffs(y) - 1;
+        m += total;
+        __syncthreads();  // bits and ws are the next pass's
+    }
+    return (int)m;
+}
+
+// The lists of more than BUCKET_SHORT half-edges of one CTA of k_bucket_edges
+// (out of line: the ordinary path then keeps its registers)
+struct LongLists {
+    unsigned at[BUCKET_TPB];         // each vertex's first edge
+    uint16_t len[BUCKET_TPB];        // and its number of them
+    unsigned char v[BUCKET_TPB];     // the vertices, in any order
+    int n, range[2];
+};
+
+// all of them sorted: in place in list (the CTA's in shared memory, or null),
+// out as scratch; hubs, and the others without it, to spare
+__device__ __noinline__ void sort_long_lists(LongLists &l, const int *ptr, int p0, int *list, int *out,
+                                             const int *bucket, int *spare, unsigned *ws) {
+    for (int x = threadIdx.x >> 5; x < l.n; x += BUCKET_TPB / 32) {
+        const int q = l.v[x], l0 = ptr[q], n = ptr[q + 1] - l0;
+        if (n > BUCKET_WARP) continue;
+        const int m = list ? warp_sort_unique(list + (l0 - p0), n, out + (l0 - p0), list + (l0 - p0))
+                           : warp_sort_unique(bucket + l0, n, spare + l0, spare + l0);
+        if ((threadIdx.x & 31) == 0) l.len[q] = (uint16_t)m;
+    }
+    for (int x = 0; x < l.n; ++x) {
+        const int q = l.v[x], l0 = ptr[q], n = ptr[q + 1] - l0;
+        if (n <= BUCKET_WARP) continue;
+        const int m = cta_sort_unique(bucket + l0, n, spare + l0, (unsigned *)out, ws, l.range);
+        if (threadIdx.x == 0) l.len[q] = (uint16_t)m;
+    }
+    __syncthreads();
+}
+
+// their edges, vertex q's from its thread's `at` on: to out and owner, or
+// straight to edges (list null)
+__device__ __noinline__ void put_long_lists(LongLists &l, const int *ptr, int p0, const int *list,
+                                            const int *spare, unsigned at, int v0, int *out,
+                                            unsigned char *owner, int2 *edges) {
+    l.at[threadIdx.x] = at;
+    __syncthreads();
+    auto put = [&](int q, const int *from, int first, int step) {
+        const unsigned to = l.at[q];
+        const int m = l.len[q];
+#pragma unroll 4
+        for (int i = first; i < m; i += step) {
+            const int y = from[i];
+            if (list) {
+                out[to + i] = y;
+                owner[to + i] = (unsigned char)q;
+            } else {
+                edges[to + i] = make_int2(v0 + q, y);
+            }
+        }
+    };
+    for (int x = threadIdx.x >> 5; x < l.n; x += BUCKET_TPB / 32) {
+        const int q = l.v[x], l0 = ptr[q], n = ptr[q + 1] - l0;
+        if (n <= BUCKET_WARP) put(q, list ? list + (l0 - p0) : spare + l0, threadIdx.x & 31, 32);
+    }
+    for (int x = 0; x < l.n; ++x) {
+        const int q = l.v[x], l0 = ptr[q], n = ptr[q + 1] - l0;
+        if (n > BUCKET_WARP) put(q, spare + l0, threadIdx.x, BUCKET_TPB);
+    }
+}
+
+// spare (HUBS): [the half-edges], the sorted lists of more than BUCKET_SHORT
+template <bool HUBS>
+__global__ void __launch_bounds__(BUCKET_TPB, 6) k_bucket_edges(const int *ptr, int nv, int *bucket, int *spare,
+                                                                int2 *edges, int *d_count, const int *slow,
+                                                                unsigned long long *state, int *ticket,
+                                                                uint32_t *status) {
     HFCR_PDL_WAIT();
     // a void result is not written (edges may be the caller's own buffer)
-    if (*slow || (*(volatile uint32_t *)status & ST_BAD_INDEX)) return;
+    const bool is_void = *slow || (*(volatile uint32_t *)status & ST_BAD_INDEX);
     __shared__ int list[BUCKET_SM], out[BUCKET_SM];
     __shared__ unsigned char owner[BUCKET_SM];
+    __shared__ LongLists longs[1];  // (no room is taken where nothing uses it)
     __shared__ unsigned ws[BUCKET_TPB / 32], base;
     __shared__ int cta;
-    if (threadIdx.x == 0) cta = atomicAdd(ticket, 1);
+    if (threadIdx.x == 0) {
+        cta = atomicAdd(ticket, 1);
+        if (HUBS) longs->n = 0;
+    }
     __syncthreads();
+    if (is_void) return;
     const int v0 = cta * BUCKET_TPB, v = v0 + threadIdx.x, ve = min(v0 + BUCKET_TPB, nv);
     const int p0 = ptr[v0], m = ptr[ve] - p0;
     const bool in_sm = m <= BUCKET_SM;
     const int a = v < nv ? ptr[v] - p0 : 0, n = v < nv ? ptr[v + 1] - p0 - a : 0;
-    int u = 0;
-    if (in_sm) {
+    const bool is_long = HUBS && n > BUCKET_SHORT;
+    if (is_long) longs->v[atomicAdd(&longs->n, 1)] = (unsigned char)threadIdx.x;
+    if (in_sm)
         for (int i = threadIdx.x; i < m; i += BUCKET_TPB) list[i] = bucket[p0 + i];
-        __syncthreads();
-        if (n <= BUCKET_MAX) u = sort_unique(list + a, n);
-    } else if (n <= BUCKET_MAX) {
-        u = sort_unique(bucket + p0 + a, n);
+    __syncthreads();
+    int u = 0;
+    if (!is_long) u = in_sm ? sort_unique(list + a, n) : sort_unique(bucket + p0 + a, n);
+    if (HUBS && longs->n) {
+        sort_long_lists(*longs, ptr + v0, p0, in_sm ? list : nullptr, out, bucket, spare, ws);
+        if (is_long) u = longs->len[threadIdx.x];
     }
     unsigned total;
     const unsigned at = cta_scan((unsigned)u, ws, total);
@@ -272,16 +492,21 @@ __global__ void __launch_bounds__(BUCKET_TPB) k_bucket_edges(const int *ptr, int
         }
     }
     if (in_sm) {  // compacted first, then written in order
-        for (int i = 0; i < u; ++i) {
-            out[at + i] = list[a + i];
-            owner[at + i] = (unsigned char)threadIdx.x;
-        }
+        if (!is_long)
+            for (int i = 0; i < u; ++i) {
+                out[at + i] = list[a + i];
+                owner[at + i] = (unsigned char)threadIdx.x;
+            }
+        if (HUBS && longs->n) put_long_lists(*longs, ptr + v0, p0, list, spare, at, v0, out, owner, edges);
         __syncthreads();
         for (int i = threadIdx.x; i < (int)total; i += BUCKET_TPB)
             edges[base + i] = make_int2(v0 + owner[i], out[i]);
     } else {
         __syncthreads();
-        for (int i = 0; i < u; ++i) edges[base + at + i] = make_int2(v, bucket[p0 + a + i]);
+        if (!is_long)
+            for (int i = 0; i < u; ++i) edges[base + at + i] = make_int2(v, bucket[p0 + a + i]);
+        if (HUBS && longs->n)
+            put_long_lists(*longs, ptr + v0, p0, nullptr, spare, base + at, v0, out, owner, edges);
     }
 }
 
@@ -709,23 +934,36 @@ size_t bucket_words(int n_verts) {
     return ((c + 1) & ~(size_t)1) + 2 * st;
 }
 
-void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
-                 unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
-                 cudaStream_t s) {
-    int *bucket = (int *)keys;                              // [3 n_tris]
-    unsigned char *rank = (unsigned char *)keys_alt;        // [3 n_tris]
+template <bool HUBS>
+static void bucket_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
+                         unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
+                         cudaStream_t s) {
+    typedef typename BucketRank<HUBS>::T Rank;
+    int *bucket = (int *)keys, *spare = bucket + 3 * (size_t)n_tris;  // [3 n_tris] each
+    Rank *rank = (Rank *)keys_alt;                                    // [3 n_tris]
     int *cnt = words, *tickets = words + n_verts + 1;
     const int nscan = (n_verts + BUCKET_SCAN - 1) / BUCKET_SCAN;
     unsigned long long *state = (unsigned long long *)(words + (((size_t)n_verts + 4 + 1) & ~(size_t)1));
     cudaMemsetAsync(words, 0, sizeof(int) * bucket_words(n_verts), s);
     const int nb = (n_tris + BUCKET_TPB - 1) / BUCKET_TPB, vb = (n_verts + BUCKET_TPB - 1) / BUCKET_TPB;
-    { launch_pdl(k_bucket_count, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, cnt, rank, d_slow,
+    { launch_pdl(k_bucket_count<HUBS>, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, cnt, rank, d_slow,
                  d_status); note_launch(); }
-    { launch_pdl(k_bucket_scan, nscan, BUCKET_TPB, 0, s, cnt, n_verts, state, tickets, d_status); note_launch(); }
-    { launch_pdl(k_bucket_fill, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, (const int *)cnt,
-                 (const unsigned char *)rank, bucket); note_launch(); }
-    { launch_pdl(k_bucket_edges, vb, BUCKET_TPB, 0, s, (const int *)cnt, n_verts, bucket, (int2 *)edges_out,
-                 d_count, (const int *)d_slow, state + nscan, tickets + 1, d_status); note_launch(); }
+    { launch_pdl(k_bucket_scan<HUBS>, nscan, BUCKET_TPB, 0, s, cnt, n_verts, n_tris, d_slow, state, tickets,
+                 d_status); note_launch(); }
+    { launch_pdl(k_bucket_fill<HUBS>, nb, BUCKET_TPB, 0, s, tris, n_tris, n_verts, (const int *)cnt,
+                 (const Rank *)rank, (const int *)d_slow, bucket); note_launch(); }
+    { launch_pdl(k_bucket_edges<HUBS>, vb, BUCKET_TPB, 0, s, (const int *)cnt, n_verts, bucket, spare,
+                 (int2 *)edges_out, d_count, (const int *)d_slow, state + nscan, tickets + 1, d_status);
+      note_launch(); }
+}
+
+bool bucket_hubs_first(int n_tris) { return n_tris <= BUCKET_HUBS_TRIS; }
+
+void build_edges(const int *tris, int n_tris, int n_verts, bool hubs, int *edges_out, int *d_count, int *d_slow,
+                 unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
+                 cudaStream_t s) {
+    (hubs ? bucket_edges<true> : bucket_edges<false>)(tris, n_tris, n_verts, edges_out, d_count, d_slow, keys,
+                                                      keys_alt, words, d_status, s);
 }
 
 void check_segments(const int *segs, int nseg, const hfcr_mesh &A, const hfcr_mesh &B,

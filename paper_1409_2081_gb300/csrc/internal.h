@@ -157,14 +157,17 @@ void scan_flags_dev(unsigned *flags, const int *d_n, int cap, int *d_total, Sort
 
 // ---- topology ----
 // Unique sorted edges of a triangle list, by buckets of the smaller vertex
-// (n_tris, n_verts >= 1).  Scratch: keys/keys_alt of 3 * n_tris u64 and
-// bucket_words(n_verts) words, both 8-byte aligned, as edges_out is.  *d_slow
-// (zero before) is set when a vertex has too many: build_edges_sorted then
-// gives the result.  After that, and after an index out of range, neither
-// edges_out nor *d_count has been written.
-void build_edges(const int *tris, int n_tris, int n_verts, int *edges_out, int *d_count, int *d_slow,
+// (n_tris, n_verts >= 1); hubs: the form that takes vertices of many half-
+// edges too (the first to try when bucket_hubs_first says so).  Scratch:
+// keys/keys_alt of 3 * n_tris u64 and bucket_words(n_verts) words, both 8-byte
+// aligned, as edges_out is.  *d_slow (zero before) is set when the form does
+// not take the mesh: the form with hubs, or build_edges_sorted after it, is to
+// be tried.  After that, and after an index out of range, neither edges_out
+// nor *d_count has been written.
+void build_edges(const int *tris, int n_tris, int n_verts, bool hubs, int *edges_out, int *d_count, int *d_slow,
                  unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
                  cudaStream_t s);
+bool bucket_hubs_first(int n_tris);
 size_t bucket_words(int n_verts);
 // The same by a radix sort of all the edges' keys.  Scratch: keys/keys_alt of
 // 3 * n_tris u64 and flags of 3 * n_tris unsigned.
