@@ -240,7 +240,12 @@ hfcr_status hfcr_destroy(hfcr_ctx *ctx);
 /* Allocate the context's device scratch for meshes of up to max_verts
  * vertices and max_tris triangles each and up to max_pairs E-F pairs per
  * detection (stencils <= pairs).  May be called again to grow; calls that
- * exceed the reserved sizes return HFCR_ERR_CAPACITY.  Synchronous. */
+ * exceed the reserved sizes return HFCR_ERR_CAPACITY.  Synchronous.
+ *
+ * A detection lists the edges and faces whose boxes overlap in scratch of
+ * max(6 max_tris, 12 max_pairs) entries.  More of them (layers that lie on one
+ * another have 6 to 20 a face) are not an error: they are then tested as they
+ * are met, which costs up to the broad phase once more. */
 hfcr_status hfcr_reserve(hfcr_ctx *ctx, int64_t max_verts, int64_t max_tris, int64_t max_pairs);
 
 /* Unique undirected edges (v0 < v1, lexicographic) of a triangle list: the

@@ -46,7 +46,7 @@ struct DevWords {
     uint32_t status;
     uint32_t pad0;
     DevStats stats;
-    int cnt[16];
+    int cnt[24];
     int iwork[16];
     double dwork[16];
     int touched;
@@ -66,9 +66,9 @@ struct hfcr_ctx {
     int *scan_words() const { return (int *)(d_words + 1); }
     uint32_t *d_status = nullptr;
     DevStats *d_stats = nullptr;
-    int *d_cnt = nullptr;         // [16] device counters
+    int *d_cnt = nullptr;         // [24] device counters
     uint32_t *h_status = nullptr;
-    int *h_cnt = nullptr;         // [16]
+    int *h_cnt = nullptr;         // [24]
     DevStats *h_stats = nullptr;
     double *h_dw = nullptr;       // solver scalars
     int trav_variant = 0;         // traversal variant (hfcr_autotune)
@@ -123,8 +123,9 @@ struct hfcr_ctx {
 
 // device counter slots
 enum { C_PAIRS = 0, C_STENCILS = 1, C_EDGES_A = 2, C_EDGES_B = 3, C_N4 = 4, C_NPAIRS_IN = 5, C_PEFF = 6,
-       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_QUEUE = 10 /* to 13: two words per direction */,
-       C_SLOW = 14, C_BAND_DONE = C_DIFF_ITERS + 8 /* the diffusion's ctl word 8 */ };
+       C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_SLOW = 14,
+       C_BAND_DONE = C_DIFF_ITERS + 8 /* the diffusion's ctl word 8 */,
+       C_QUEUE = 16 /* to 21: three words per direction */ };
 
 namespace {
 
@@ -156,7 +157,7 @@ cudaError_t dalloc(T **p, size_t n) {
 
 void free_all(hfcr_ctx *c) {
     void *ptrs[] = {c->d_words, c->sort.hist, c->edges[0], c->edges[1],
-                    c->ekeys, c->ekeys_alt, c->eflags, c->pkeys, c->pkeys_alt,
+                    c->ekeys, c->eflags, c->pkeys, c->pkeys_alt,
                     c->skeys, c->skeys_alt, c->stencils,
                     c->sb.ids_raw, c->sb.n64_raw, c->sb.n32_raw, c->sb.b_raw, c->sb.parent,
                     c->sb.zkey, c->sb.zkey_alt, c->sb.szone, c->sb.zs, c->sb.zv, c->sb.d_nz,
@@ -471,6 +472,16 @@ void bvh_note(hfcr_ctx *ctx, int d, const hfcr_mesh &F, const DetectPlan &pl, bo
     }
 }
 
+// The list between the two phases of a traversal, in the larger of two
+// buffers that are free there: the edge builds' keys (six entries a reserved
+// triangle) and the solver's vertex sums (twelve a reserved pair).
+void leaf_list(hfcr_ctx *ctx, DetectArgs &a) {
+    const int64_t keys = 6 * ctx->max_tris, sums = 12 * ctx->max_pairs, most = 1 << 30;
+    a.leaves = keys > sums ? (int2 *)ctx->ekeys : (int2 *)ctx->sb.u64;
+    const int64_t cap = keys > sums ? keys : sums;
+    a.leaf_cap = (int)(cap < most ? cap : most);
+}
+
 // Launches the traversal of the active directions; positions validated and
 // the BVHs refitted (built first when `build`).  Pair keys -> ctx->pkeys.
 void launch_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bool dir0, bool dir1,
@@ -504,9 +515,8 @@ void launch_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bool d
             a.cap = (int)ctx->max_pairs;
             a.stats = ctx->d_stats;
             a.variant = variant;
-            a.queue = ctx->d_cnt + C_QUEUE + 2 * d;
-            a.leaves = (int2 *)ctx->ekeys;  // free outside the edge builds
-            a.leaf_cap = (int)(3 * ctx->max_tris);
+            a.queue = ctx->d_cnt + C_QUEUE + 3 * d;
+            leaf_list(ctx, a);
             detect_launch(a, s, ctx->d_status);
         }
         return;
@@ -549,9 +559,8 @@ void launch_detect(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B, bool d
         a.cap = (int)ctx->max_pairs;
         a.stats = ctx->d_stats;
         a.variant = ctx->trav_variant;
-        a.queue = ctx->d_cnt + C_QUEUE + 2 * d;
-        a.leaves = (int2 *)ctx->ekeys;  // free outside the edge builds
-        a.leaf_cap = (int)(3 * ctx->max_tris);
+        a.queue = ctx->d_cnt + C_QUEUE + 3 * d;
+        leaf_list(ctx, a);
         prof_begin(ctx, HFCR_STAGE_TRAVERSE, s);
         detect_launch(a, s, ctx->d_status);
         prof_end(ctx, HFCR_STAGE_TRAVERSE, s);
@@ -1008,8 +1017,9 @@ hfcr_status hfcr_reserve(hfcr_ctx *ctx, int64_t max_verts, int64_t max_tris, int
         CK(dalloc(&ctx->edges[i], 2 * E3));
         CK(dalloc(&ctx->eorder[i], E3));
     }
-    CK(dalloc(&ctx->ekeys, E3));
-    CK(dalloc(&ctx->ekeys_alt, E3));
+    const size_t E3a = (E3 + 31) & ~(size_t)31;  // both start on 256 bytes
+    CK(dalloc(&ctx->ekeys, 2 * E3a));            // one list to the traversal
+    ctx->ekeys_alt = ctx->ekeys + E3a;
     CK(dalloc(&ctx->eflags, E3));
     CK(dalloc(&ctx->pkeys, P));
     CK(dalloc(&ctx->pkeys_alt, P));
@@ -1407,7 +1417,7 @@ hfcr_status hfcr_autotune(hfcr_ctx *ctx, const hfcr_mesh *A, const hfcr_mesh *B,
         double vbest = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
             CK(cudaMemsetAsync(ctx->d_cnt + C_PAIRS, 0, sizeof(int), s));
-            CK(cudaMemsetAsync(ctx->d_cnt + C_QUEUE, 0, 4 * sizeof(int), s));
+            CK(cudaMemsetAsync(ctx->d_cnt + C_QUEUE, 0, 6 * sizeof(int), s));
             CK(cudaEventRecord(e0, s));
             launch_detect(ctx, A, B, dir0, dir1, pl, built, s, true, v);
             CK(cudaEventRecord(e1, s));

@@ -158,16 +158,26 @@ __device__ __forceinline__ void ld_node(const float4 *nodes, int i, float *f) {
     }
 }
 
+// what a walk is over: the edges of one direction and the trees they cross
 template <typename T>
-__global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
-    const int2 *edges, const int *order, int ne, int chunk, const T *ex, const T *ey, const T *ez,
-    int nv, const float4 *nodes, int nfaces, const int *segs, int nseg, int ecol, int fcol, LeafList out,
-    int *queue, uint32_t *status) {
-    HFCR_PDL_WAIT();
-    // malformed input (reported by the host): its tree is not walked
-    if (__any_sync(0xffffffffu, (*(volatile uint32_t *)status & ST_BAD_INDEX) != 0)) return;
-    __shared__ PoolSmem smw[POOL_WARPS];
-    PoolSmem &sm = smw[threadIdx.x >> 5];
+struct WalkArgs {
+    const int2 *edges;
+    const int *order;
+    int ne, chunk;
+    const T *ex, *ey, *ez;
+    int nv;
+    const float4 *nodes;
+    int nfaces;
+    const int *segs;
+    int nseg, ecol, fcol;
+    int *queue;  // edges taken beyond every warp's first
+    uint32_t *status;
+};
+
+// One warp's share of the walk (CTAs of POOL_WARPS warps).  sink(leaves, n): n <=
+// 32 leaves met, 32 of them but for the last of a batch; false ends the walk.
+template <typename T, class Sink>
+__device__ __forceinline__ void pool_walk(PoolSmem &sm, const WalkArgs<T> &g, Sink sink) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
@@ -177,27 +187,21 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
     // leaves wait (all the same in every lane)
     int top = 0, n = 0, nl = 0, spilled = 0;
     int2 spill[POOL_SPILL];
-    int base = (blockIdx.x * POOL_WARPS + (threadIdx.x >> 5)) * chunk;  // the next edges
+    int base = (blockIdx.x * POOL_WARPS + (threadIdx.x >> 5)) * g.chunk;  // the next edges
     // steps since the last edges were taken: guards against a corrupted tree
     // (an edge visits each of the 2 nfaces - 1 nodes at most once)
     unsigned steps = 0;
-    const unsigned most = (unsigned)min(64ll * nfaces + 256, 0xffffffffll);
+    const unsigned most = (unsigned)min(64ll * g.nfaces + 256, 0xffffffffll);
     while (true) {
         if (++steps > most) {
-            if (lane == 0) atomicOr(status, ST_BAD_INDEX);
+            if (lane == 0) atomicOr(g.status, ST_BAD_INDEX);
             break;
         }
-        const bool fresh = n < 32 && spilled == 0 && base < ne;
+        const bool fresh = n < 32 && spilled == 0 && base < g.ne;
         if (nl >= 32 || (nl > 0 && n == 0 && spilled == 0 && !fresh)) {
             const int take = min(nl, 32);
             nl -= take;
-            int at = 0;
-            if (lane == 0) {  // once over the capacity the count only has to stay there
-                at = *(volatile int *)out.n;
-                if (at <= out.cap) at = atomicAdd(out.n, take);
-            }
-            at = __shfl_sync(full, at, 0) + lane;
-            if (lane < take && at < out.cap) out.items[at] = sm.leaf[nl + lane];
+            if (!sink(sm.leaf + nl, take)) break;
             __syncwarp();
             continue;
         }
@@ -207,18 +211,18 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
         if (fresh) {
             const int i = base + lane;
             int t0 = 0, nleaf = 0;
-            if (lane < chunk && i < ne) {
-                e = order ? order[i] : i;
-                const int2 ev = edges[e];
-                if (nseg > 1 && !(segs[4 * hint + ecol] <= ev.x && ev.x < segs[4 * (hint + 1) + ecol]))
-                    hint = seg_of(segs, ecol, nseg, ev.x);
-                seg_range(segs, fcol, hint, nfaces, t0, nleaf);
+            if (lane < g.chunk && i < g.ne) {
+                e = g.order ? g.order[i] : i;
+                const int2 ev = g.edges[e];
+                if (g.nseg > 1 && !(g.segs[4 * hint + g.ecol] <= ev.x && ev.x < g.segs[4 * (hint + 1) + g.ecol]))
+                    hint = seg_of(g.segs, g.ecol, g.nseg, ev.x);
+                seg_range(g.segs, g.fcol, hint, g.nfaces, t0, nleaf);
                 T p[3], q[3];
-                ld_edge(ev, ex, ey, ez, nv, p, q, status);
+                ld_edge(ev, g.ex, g.ey, g.ez, g.nv, p, q, g.status);
                 edge_box(p, q, lo, hi);
             }
             steps = 0;
-            if (lane == 0) base = gridDim.x * POOL_WARPS * chunk + atomicAdd(queue, chunk);
+            if (lane == 0) base = gridDim.x * POOL_WARPS * g.chunk + atomicAdd(g.queue, g.chunk);
             base = __shfl_sync(full, base, 0);
             const bool one = nleaf == 1;  // a tree of one leaf: tested outright
             const unsigned m = __ballot_sync(full, one);
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
             if (lane < 16) {
                 const int2 s = spill[spilled];
                 T p[3], q[3];
-                ld_edge(edges[s.x], ex, ey, ez, nv, p, q, status);
+                ld_edge(g.edges[s.x], g.ex, g.ey, g.ez, g.nv, p, q, g.status);
                 edge_box(p, q, lo, hi);
                 e = s.x;
                 node = s.y;
@@ -260,7 +264,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
         bool h0 = false, h1 = false;
         if (on) {
             float f[16];
-            ld_node(nodes, node, f);
+            ld_node(g.nodes, node, f);
             c0 = __float_as_int(f[12]);
             c1 = __float_as_int(f[13]);
             h0 = overlap(lo, hi, f[0], f[1], f[2], f[3], f[4], f[5]);
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
             if (lane < 16) {
                 const float4 s = sm.b[(top - n + lane) & (POOL_CAP - 1)];
                 if (spilled < POOL_SPILL) spill[spilled] = make_int2(__float_as_int(s.z), __float_as_int(s.w));
-                else atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
+                else atomicOr(g.status, ST_BAD_INDEX);  // unreachable: depth < 64
             }
             spilled = min(spilled + 1, POOL_SPILL);
             n -= 16;
@@ -301,6 +305,27 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(
     }
 }
 
+// Once the list is over its capacity the count stays there and the warps
+// leave: k_narrow then walks on its own.
+template <typename T>
+__global__ void __launch_bounds__(32 * POOL_WARPS, 8) k_broad(WalkArgs<T> g, LeafList out) {
+    HFCR_PDL_WAIT();
+    // malformed input (reported by the host): its tree is not walked
+    if (__any_sync(0xffffffffu, (*(volatile uint32_t *)g.status & ST_BAD_INDEX) != 0)) return;
+    __shared__ PoolSmem smw[POOL_WARPS];
+    pool_walk(smw[threadIdx.x >> 5], g, [&](const int2 *leaf, int take) {
+        const int lane = threadIdx.x & 31;
+        int at = 0;
+        if (lane == 0) {
+            at = *(volatile int *)out.n;
+            if (at <= out.cap) at = atomicAdd(out.n, take);
+        }
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (lane < take && at + lane < out.cap) out.items[at + lane] = leaf[lane];
+        return at <= out.cap;
+    });
+}
+
 // leaf lf against an edge, the hit appended
 template <typename T, bool F32F>
 __device__ __forceinline__ void narrow_test(const T *p, const T *q, int e, int lf, const void *leaf_tri,
@@ -314,65 +339,46 @@ __device__ __forceinline__ void narrow_test(const T *p, const T *q, int e, int l
     }
 }
 
+// the same out of line
+template <typename T, bool F32F>
+__device__ __noinline__ void narrow_test_call(const int2 l, const WalkArgs<T> &g, const void *leaf_tri,
+                                              const HitList &o) {
+    T p[3], q[3];
+    ld_edge(g.edges[l.x], g.ex, g.ey, g.ez, g.nv, p, q, g.status);
+    narrow_test<T, F32F>(p, q, l.x, l.y, leaf_tri, o);
+}
+
 // Narrow phase: the exact test of every (edge, leaf) of the broad phase, one
 // per thread, consecutive warps' work on different CTAs (few tests spread
 // over many SMs: the float64 stages are slow on one).  When the list
-// overflowed, every edge is walked again from its root by one thread, each
-// leaf tested as it is met.
+// overflowed, it walks the edges itself as the broad phase does and tests
+// the leaves 32 at a time as they are met.
 template <typename T, bool F32F>
-__global__ void __launch_bounds__(128) k_narrow(
-    const int2 *edges, int ne, const T *ex, const T *ey, const T *ez, int nv, const float4 *nodes,
-    const void *leaf_tri, int nfaces, const int *segs, int nseg, int ecol, int fcol, HitList o, LeafList in,
-    uint32_t *status) {
+__global__ void __launch_bounds__(32 * POOL_WARPS) k_narrow(const __grid_constant__ WalkArgs<T> g,
+                                                            const void *leaf_tri,
+                                                            const __grid_constant__ HitList o, LeafList in) {
     HFCR_PDL_WAIT();
-    if (*(volatile uint32_t *)status & ST_BAD_INDEX) return;
+    if (*(volatile uint32_t *)g.status & ST_BAD_INDEX) return;
     const int n = *in.n, lane = threadIdx.x & 31;
-    const int first = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + lane, stride = gridDim.x * 128;
     if (n <= in.cap) {
+        const int first = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + lane;
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&o.st->narrow_tests, (unsigned long long)n);
-        for (int i = first; i < n; i += stride) {
+        for (int i = first; i < n; i += gridDim.x * 128) {
             const int2 l = in.items[i];
             T p[3], q[3];
-            ld_edge(edges[l.x], ex, ey, ez, nv, p, q, status);
+            ld_edge(g.edges[l.x], g.ex, g.ey, g.ez, g.nv, p, q, g.status);
             narrow_test<T, F32F>(p, q, l.x, l.y, leaf_tri, o);
         }
         return;
     }
+    __shared__ PoolSmem smw[POOL_WARPS];
     unsigned tests = 0;
-    for (int e = first; e < ne; e += stride) {
-        const int2 ev = edges[e];
-        int t0, nleaf;
-        seg_range(segs, fcol, seg_of(segs, ecol, nseg, ev.x), nfaces, t0, nleaf);
-        if (nleaf < 1) continue;
-        T p[3], q[3];
-        ld_edge(ev, ex, ey, ez, nv, p, q, status);
-        float lo[3], hi[3];
-        edge_box(p, q, lo, hi);
-        int stack[STACK];
-        int sp = 0, node = nleaf == 1 ? ~t0 : t0, visits = 0;
-        while (true) {
-            if (++visits > 2 * nleaf + 8) {  // a corrupted tree
-                atomicOr(status, ST_BAD_INDEX);
-                break;
-            }
-            if (node < 0) {
-                narrow_test<T, F32F>(p, q, e, ~node, leaf_tri, o);
-                ++tests;
-            } else {
-                float f[16];
-                ld_node(nodes, node, f);
-                if (sp + 2 > STACK) {
-                    atomicOr(status, ST_BAD_INDEX);  // unreachable: depth < 64
-                    break;
-                }
-                if (overlap(lo, hi, f[6], f[7], f[8], f[9], f[10], f[11])) stack[sp++] = __float_as_int(f[13]);
-                if (overlap(lo, hi, f[0], f[1], f[2], f[3], f[4], f[5])) stack[sp++] = __float_as_int(f[12]);
-            }
-            if (sp == 0) break;
-            node = stack[--sp];
-        }
-    }
-    if (tests) atomicAdd(&o.st->narrow_tests, (unsigned long long)tests);
+    pool_walk(smw[threadIdx.x >> 5], g, [&](const int2 *leaf, int take) {
+        if (lane < take) narrow_test_call<T, F32F>(leaf[lane], g, leaf_tri, o);
+        tests += take;
+        return true;
+    });
+    if (lane == 0 && tests) atomicAdd(&o.st->narrow_tests, (unsigned long long)tests);
 }
 
 __global__ void k_keys_to_pairs(const unsigned long long *keys, const int *d_n, int cap,
@@ -596,14 +602,14 @@ static void launch_phases(const DetectArgs &a, cudaStream_t s, uint32_t *d_statu
     const int need = (a.n_edges + chunk * POOL_WARPS - 1) / (chunk * POOL_WARPS);
     if (grid > need) grid = need;
     const LeafList l = {a.leaves, a.queue + 1, a.leaf_cap};
-    { launch_pdl(k_broad<T>, grid, 32 * POOL_WARPS, 0, s, (const int2 *)a.edges, a.order, a.n_edges, chunk, x,
-                 y, z, m.n_verts, a.bvh->nodes, a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, l, a.queue, d_status);
-      note_launch(); }
+    WalkArgs<T> g = {(const int2 *)a.edges, a.order, a.n_edges, chunk, x, y, z, m.n_verts, a.bvh->nodes,
+                     a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, a.queue, d_status};
+    { launch_pdl(k_broad<T>, grid, 32 * POOL_WARPS, 0, s, g, l); note_launch(); }
     const HitList o = {a.keys, a.d_count, dirbit, a.cap, a.face_bits, a.stats};
     int gn = (a.n_edges + 127) / 128;
     if (gn > 8 * 152) gn = 8 * 152;
-    { launch_pdl(k_narrow<T, F32F>, gn, 128, 0, s, (const int2 *)a.edges, a.n_edges, x, y, z, m.n_verts,
-                 a.bvh->nodes, a.bvh->leaf_tri, a.bvh->n, a.segs, a.nseg, a.ecol, a.fcol, o, l, d_status);
+    g.queue = a.queue + 2;
+    { launch_pdl(k_narrow<T, F32F>, gn, 32 * POOL_WARPS, 0, s, g, (const void *)a.bvh->leaf_tri, o, l);
       note_launch(); }
 }
 

@@ -213,7 +213,7 @@ struct DetectArgs {
     int cap;
     DevStats *stats;
     int variant = 0;       // traversal variant (0 to 8; see detect.cu)
-    int *queue = nullptr;  // [2] edges taken, leaves listed (zero before the launch)
+    int *queue = nullptr;  // [3] edges taken, leaves listed, edges taken by a walk past the list (zero before)
     int2 *leaves = nullptr;  // [leaf_cap] (edge, leaf) between the broad and the narrow phase
     int leaf_cap = 0;
 };
