@@ -1856,12 +1856,13 @@ __device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *b
         float gamma, delta, rho;
         apply(gamma, delta, rho);
         const float stop = (float)a.tol * (float)a.tol * rho;
-        float alpha = __fdividef(gamma, delta), beta = 0.f;
+        float alpha = gamma / delta, beta = 0.f;
         int it = 0;
         while (it < cap_it && rho > stop && rho > 0.f && alpha > 0.f && isfinite(alpha)) {
-            // beta = g' / g and alpha' = g' / (d' - beta g' / alpha): the
-            // reciprocals that do not wait for the sums
-            const float rg = __fdividef(1.0f, gamma), ra = __fdividef(1.0f, alpha);
+            // beta = g' / g and alpha' = g' / (d' - g' g' / (g alpha)): two
+            // divisions deep, and rounded ones (a product with 1 / g would
+            // overflow where g' / g does not)
+            const float ga = gamma * alpha;
 #pragma unroll
             for (int v = 0; v < RPT; ++v) {
                 p[v] = zz[v] + beta * p[v];
@@ -1871,8 +1872,8 @@ __device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *b
             }
             float gn, dn, rn;
             apply(gn, dn, rn);
-            beta = gn * rg;
-            alpha = __fdividef(gn, dn - beta * (gn * ra));
+            beta = gn / gamma;
+            alpha = gn / (dn - gn * (gn / ga));
             gamma = gn;
             rho = rn;
             ++it;
