@@ -1662,11 +1662,27 @@ __device__ __forceinline__ ZoneResult solve_zone_smem(const ZoneArgs &a, int z, 
 // passes: against a gather of u and four vertex products per row, a zone of
 // 1,219 rows (74 iterations, 3 rounds) 440 -> 227 us, zones of 33 to 255 rows
 // in pairs 185 -> 124 us, zones of up to 32 rows in a warp each 96 -> 45 us.
+// On an ill-conditioned zone the rounds get weak: the entries are rounded, and
+// so are the products of the other form.  Where a round reduces the float64
+// residual by less than ROWS_WEAK and more than one such step is left, the zone
+// is given to the float64 rescue at once if that is staged (rescue_fits): a zone
+// of 354 rows left at 7e-6 went on for three rounds of 104 to 180 iterations
+// before (its call 1.91 -> 1.27 ms).
 // Returns 0 when done (res filled, lambda stored), 1 when the zone does not
 // fit (rows, shared memory) and nothing was done, 2 when a run of a
 // BLK zone took block_switch iterations: lambda holds the best so far, and the
 // blocks are to take over.
 // ---------------------------------------------------------------------------
+constexpr double ROWS_WEAK = 30.0;
+
+// the float64 rescue (zone64_staged): its threads with rows, the rows of each,
+// its shared memory, and whether a zone fits `bytes` of it
+constexpr int RESCUE_NT = 256, RESCUE_ROWS = 4;
+constexpr int RESCUE_SMEM = 220 * 1024;
+__device__ __forceinline__ bool rescue_fits(int k, int U, int bytes) {
+    return k <= RESCUE_ROWS * RESCUE_NT && 98ll * k + 30ll * U + 64 <= bytes;
+}
+
 template <class Gp, int RPT, bool BLK>
 __device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *base, int bytes, double bb,
                                                float *red, double *redd, ZoneResult &res) {
@@ -1942,7 +1958,9 @@ __device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *b
             for (int v = 0; v < RPT; ++v) lam[v] -= (double)x[v];
             break;
         }
+        const bool weak = rr_new * (ROWS_WEAK * ROWS_WEAK) > rr;
         rr = rr_new;
+        if (weak && rr > ROWS_WEAK * ROWS_WEAK * target && rescue_fits(k, U, RESCUE_SMEM)) break;
 #pragma unroll
         for (int v = 0; v < RPT; ++v) r[v] = rn[v];
         if (may_switch && it >= cap_it && rr > target) {
@@ -2341,9 +2359,8 @@ __device__ __forceinline__ void zone64_precond(const ZoneArgs &a, int s0, int g0
 // tree of sums over RESCUE_NT threads, correctly rounded divisions).  A zone
 // of 97 rows (93 iterations) 853 -> 584 us, one of 354 rows (75) 1,175 -> 835.
 // False when the zone does not fit (nothing done); otherwise lambda is stored and the count in its.
-constexpr int RESCUE_THREADS = 512, RESCUE_NT = ZONE64_THREADS, RESCUE_ROWS = 4;  // threads with rows, rows each
-constexpr int RESCUE_VT = RESCUE_THREADS - 32;                                   // threads with vertices
-constexpr int RESCUE_SMEM = 220 * 1024;
+constexpr int RESCUE_THREADS = 512;
+constexpr int RESCUE_VT = RESCUE_THREADS - 32;  // threads with vertices
 
 // a / b from y = 1 / b rounded to nearest (Markstein, 1990): a y, corrected by
 // its residual, is a / b rounded to nearest
@@ -2366,15 +2383,14 @@ __device__ __forceinline__ double warp_halve3d(double a, double b, double c) {  
 __device__ __forceinline__ bool zone64_staged(const ZoneArgs &a, int z, char *base, int bytes, double bb,
                                               int maxit, double *red, double *sc, int &its) {
     constexpr int NT = RESCUE_NT, RPT = RESCUE_ROWS;
-    static_assert(NT == 256 && RESCUE_VT == 480, "the named barriers below; eight warps' sums");
+    static_assert(NT == 256 && NT == ZONE64_THREADS && RESCUE_VT == 480, "the named barriers below; eight warps' sums");
     const int tid = threadIdx.x, lane = tid & 31, wq = tid >> 5;
     const int s0 = a.zs[z], k = a.zs[z + 1] - s0;
     const int j0 = a.zv[z], U = a.zv[z + 1] - j0;
     const int g0 = a.zg[z], G = a.zg[z + 1] - g0;
     const int e0 = a.seg[j0];
     // layout: blocks' inverse rows | normals | z, -z / 3 | r | u | vidx | winv | seg | cval | groups
-    const long long need = 98ll * k + 30ll * U + 64;
-    if (k > RPT * NT || need > bytes) return false;
+    if (!rescue_fits(k, U, bytes)) return false;
     double4_32a *pS = (double4_32a *)base;
     double *nS = (double *)(pS + k), *zS = nS + 3 * k, *rS = zS + 2 * k, *uS = rS + k;
     ushort4 *vidx = (ushort4 *)(uS + 3 * U);
