@@ -124,8 +124,9 @@ struct hfcr_ctx {
 // device counter slots
 enum { C_PAIRS = 0, C_STENCILS = 1, C_EDGES_A = 2, C_EDGES_B = 3, C_N4 = 4, C_NPAIRS_IN = 5, C_PEFF = 6,
        C_DIFF_ITERS = 7, C_DIFF_FAIL = 8, C_NFREE = 9, C_SLOW = 14,
-       C_BAND_DONE = C_DIFF_ITERS + 8 /* the diffusion's ctl word 8 */,
+       C_BAND_DONE = C_DIFF_ITERS + BAND_DONE /* the diffusion's ctl begins at C_DIFF_ITERS */,
        C_QUEUE = 16 /* to 21: three words per direction */ };
+static_assert(C_BAND_DONE > C_SLOW && C_BAND_DONE < C_QUEUE, "the words of ctl that are in use have no other user");
 
 namespace {
 

@@ -355,7 +355,7 @@ struct BandArgs {
     double *part;        // [2][grid][9] per-CTA partial sums (doubles, or floats in the same space)
     unsigned *bar;       // grid barrier counter, zeroed before the launch
     int *ctl;            // [0] CG iterations run, [1] set when a coordinate stopped unconverged,
-                         // [BAND_DONE] set when the pipelined kernel solved the band
+                         // [BAND_DONE] (zero before) what the pipelined kernel did
     uint32_t *status;
     double tol;
     int max_iters;
@@ -797,10 +797,11 @@ namespace cgx = cooperative_groups;
 // that have not exited), and a band of one CTA needs no cluster barrier.
 constexpr int BCL_THREADS = 1024;
 constexpr int BCL_PER = 256;                 // vertices of a CTA when fewer CTAs do
-constexpr int BAND_DONE = 8;                 // word of ctl set when the pipelined kernel solved the band
+enum { PIPE_SOLVED = 1, PIPE_HANDED = 2 };   // solved it; left its u in u64 for k_band_cl to go on from
 constexpr int PIPE_RINGS = 8;
 constexpr float PIPE_TOL = 6e-6f;            // reduction of one pipelined round
 constexpr int PIPE_ITERS = 200;              // its iterations at most
+constexpr int PIPE_STALL = 8;                // and those in which a coordinate's |r|^2 does not halve
 constexpr int BCL_MAX = 16;                  // CTAs per cluster at most
 constexpr int BCL_SMEM = 220 * 1024;  // dynamic shared memory per CTA
 constexpr int BCL_NB = 8;             // neighbour codes kept in shared memory per vertex
@@ -940,7 +941,7 @@ __device__ __forceinline__ void bcl_started(cgx::cluster_group &cl, int ncta) {
 // received sums in rank order (lane q holds CTA q's).  A parity's slots are
 // rewritten two calls later, after every CTA has passed the barrier that
 // follows its reads.
-template <typename T, int K, bool SYNC_END = true, int THREADS = BCL_THREADS>
+template <typename T, int K, bool SYNC_END = true>
 __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K], T *scr, T *recv,
                                          T *const *recv_of, int par, int rank, int ncta, T *out) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -955,7 +956,7 @@ __device__ __forceinline__ void bcl_sums(cgx::cluster_group &cl, const T (&v)[K]
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) t[k] = lane < THREADS / 32 ? scr[lane * K + k] : (T)0;
+        for (int k = 0; k < K; ++k) t[k] = lane < BCL_THREADS / 32 ? scr[lane * K + k] : (T)0;
         warp_sums<T, K>(t);
         if (lane < ncta) {
             T *dst = recv_of[lane] + (par * BCL_MAX + rank) * K;
@@ -1053,9 +1054,13 @@ __device__ __forceinline__ void bcl_setup(const BandArgs &a, int lo, int cnt, in
 // spill, and with this much shared memory the spills go to L2).
 // In float32 the recurrences are good to a reduction of a few 1e-6 on narrow
 // bands (simulated on bands of 870 to 14,000 vertices, 2 to 8 rings: the
-// iterations of the plain form, within two); where a round reduces the float64
-// residual by less than a factor of 30, or the iterations run out, the band is
-// left to k_band_cl.
+// iterations of the plain form, within two).  On wide bands, above all on those
+// that end at an open border, they stall above that and then grow: a coordinate
+// leaves the round once its |r|^2 has not halved for PIPE_STALL iterations (at
+// most five on bands where they do not stall), and its further rounds stop
+// above where it stalled.  Where a round reduces the float64 residual by less
+// than a factor of 30, k_band_cl goes on from the u reached; where the
+// iterations run out it starts anew, with all of them.
 // 10,653 band vertices (33 iterations) 243 -> 193 us, 7,172 (31) 195 -> 118,
 // 710 (44 -> 37 iterations, on three CTAs) 206 -> 123.
 constexpr int PIPE_VT = 480;                       // threads with vertices; one more warp folds the sums
@@ -1208,6 +1213,12 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
         st.before[threadIdx.x] = st.sumsd[threadIdx.x];
     }
     int it = 0;
+    // lane c of the folding warp, of coordinate c: |r|^2 at the round's start and
+    // the least so far, the iterations since that halved, the reduction of
+    // |r|^2 that a round is to reach
+    float rho0 = 0.f, best = 0.f, reach = PIPE_TOL * PIPE_TOL;
+    int since = 0;
+    int worse = 0;  // coordinates whose last correction is taken back (bit c)
     bool good = true;
     for (int rounds = 0; act && good; ++rounds) {
         const int it_round = it;
@@ -1289,12 +1300,23 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
                         // this round's reduction: what is left to the target, with some room
                         const float room = (float)(0.25 * st.target[c] / fmax(st.sumsd[c], 1e-300));
                         al = __fdividef(t, de);
-                        st.stop[c] = fmaxf(PIPE_TOL * PIPE_TOL, room) * rho;
+                        st.stop[c] = fmaxf(reach, room) * rho;
+                        rho0 = best = rho;
+                        since = 0;
                         go = (act >> c & 1) && rho > 0.f && al > 0.f && isfinite(al);
                     } else {
                         be = __fdividef(t, st.gam[c]);
                         al = __fdividef(t, de - be * __fdividef(t, st.alp[c]));
+                        ++since;
+                        if (rho < 0.5f * best) {
+                            best = rho;
+                            since = 0;
+                        }
                         go = (st.in >> c & 1) && rho > st.stop[c] && al > 0.f && isfinite(al);
+                        if (go && since >= PIPE_STALL) {
+                            go = false;
+                            reach = fminf(fmaxf(reach, 2.f * __fdividef(best, rho0)), 1e-3f);
+                        }
                     }
                     if (go) {
                         st.bet[c] = be;
@@ -1347,6 +1369,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
             if (!own[v]) continue;
             const float4 x4 = xq[li];
             const float *x = &x4.x;
+            // the u before in the place of m and p, which the next round sets anew
+            *(double2 *)(zq + li) = make_double2(uq[3 * li], uq[3 * li + 1]);
+            *(double *)(pq + li) = uq[3 * li + 2];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const double t = uq[3 * li + c] + (double)x[c];
@@ -1389,10 +1414,26 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
             if (!(act >> c & 1)) continue;
             if (st.sumsd[c] <= st.target[c]) act &= ~(1 << c);
             else if (!(st.sumsd[c] < st.before[c] * (1.0 / 900.0))) good = false;
+            if (!(st.sumsd[c] < st.before[c])) worse |= 1 << c;
         }
         if (it >= a.max_iters || it == it_round || rounds >= BAND_MAX_ROUNDS) good = false;
         __syncthreads();
         if (threadIdx.x < 3) st.before[threadIdx.x] = st.sumsd[threadIdx.x];
+    }
+    if (act && it < a.max_iters) {
+        if (worse) {
+            for (int li = threadIdx.x; li < cnt; li += PIPE_THREADS) {
+                const double2 w2 = *(const double2 *)(zq + li);
+                const double w[3] = {w2.x, w2.y, *(const double *)(pq + li)};
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (worse >> c & 1) gu[3 * (size_t)(lo + li) + c] = w[c];
+            }
+        }
+        if (rank == 0 && threadIdx.x == 0) {
+            a.ctl[0] += it;
+            a.ctl[BAND_DONE] = PIPE_HANDED;
+        }
     }
     if (!act) {
         for (int li = threadIdx.x; li < cnt; li += PIPE_THREADS) {
@@ -1402,7 +1443,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_band_pipe(BandArgs a) {
         }
         if (rank == 0 && threadIdx.x == 0) {
             a.ctl[0] += it;
-            a.ctl[BAND_DONE] = 1;
+            a.ctl[BAND_DONE] = PIPE_SOLVED;
         }
     }
     bcl_sync(cl, ncta);  // no CTA leaves while another may still write its shared memory
@@ -1413,9 +1454,10 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
     HFCR_PDL_WAIT();
     cgx::cluster_group cl = cgx::this_cluster();
     const int n = *a.d_nfree;
-    // the grid kernel's band, or one the pipelined kernel has done (the same in
+    // the grid kernel's band, or one the pipelined kernel has solved (the same in
     // every CTA)
-    if (n > limit || a.ctl[BAND_DONE] != 0) return;
+    const int piped = a.ctl[BAND_DONE];
+    if (n > limit || piped == PIPE_SOLVED) return;
     extern __shared__ float4 bsm[];
     __shared__ BclState st;
     const int rank = (int)cl.block_rank();
@@ -1445,6 +1487,10 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
         pq[li] = z4;
         sq[li] = z4;
         xq[li] = z4;
+        if (piped == PIPE_HANDED) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) uq[3 * li + c] = gu[3 * (size_t)(lo + li) + c];
+        }
     }
     int pf = 0, pd = 0;  // parities of the float and float64 receive slots
     bcl_started(cl, ncta);
@@ -1459,12 +1505,12 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
         for (int c = 0; c < 3; ++c) st.target[c] = a.tol * a.tol * st.sumsd[c];
     }
     int it = 0, rounds = 0;
-    bool fail = false;
+    bool fail = false, warm = piped == PIPE_HANDED;  // warm: u and its residual before the first round
     while (act) {
         if (++rounds > BAND_MAX_ROUNDS) { fail = true; break; }
         const int it_round = it;
         bool first = true;
-        while (true) {
+        while (!warm) {
             __syncthreads();  // this CTA's r visible
             // z = M^-1 r from this CTA's r
             for (int li = threadIdx.x; li < cnt; li += BCL_THREADS) {
@@ -1625,7 +1671,8 @@ __global__ void __launch_bounds__(BCL_THREADS, 1) k_band_cl(BandArgs a, int limi
 #pragma unroll
         for (int c = 0; c < 3; ++c)
             if ((act >> c & 1) && st.sumsd[c] <= st.target[c]) act &= ~(1 << c);
-        if (act && (it >= a.max_iters || it == it_round)) { fail = true; break; }
+        if (act && !warm && (it >= a.max_iters || it == it_round)) { fail = true; break; }
+        warm = false;
     }
     for (int li = threadIdx.x; li < cnt; li += BCL_THREADS) {
         double *ug = a.u + 3 * (size_t)a.fv[lo + li];

@@ -357,6 +357,8 @@ void vertex_rank(const hfcr_mesh &m, int *rank, const struct DiffScratch &ds, So
 // CSR of an edge list: ptr [nv + 1], nbr [2 ne], cur [nv] scratch
 void build_adjacency(const int *edges, int ne, int nv, int *ptr, int *nbr, int *cur, SortTemp &t,
                      uint32_t *d_status, cudaStream_t s);
+// the last word of DiffScratch::ctl that the kernels use
+constexpr int BAND_DONE = 8;
 // scratch of the harmonic diffusion (capacity cap = vertices of both meshes)
 struct DiffScratch {
     int cap = 0;
@@ -372,7 +374,8 @@ struct DiffScratch {
     double *part = nullptr;     // [2 * 9 * 1024] per-CTA partial sums
     unsigned *bar = nullptr;    // [1] grid barrier counter
     int *d_nfree = nullptr;     // band size (device)
-    int *ctl = nullptr;         // [2] CG iterations (accumulated), unconverged flag
+    int *ctl = nullptr;         // zero before: [0] CG iterations (accumulated), [1] unconverged flag,
+                                // [BAND_DONE] what the pipelined kernel did (the words between are not used)
 };
 // Diffusion of the field u (AoS float64 over A's then B's vertices) over
 // `rings` rings: the harmonic field (sweeps 0: conjugate gradients to the
