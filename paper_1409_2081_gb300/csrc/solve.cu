@@ -2355,17 +2355,19 @@ __device__ __forceinline__ void zone64_precond(const ZoneArgs &a, int s0, int g0
 // while the others update their rows.  Products stay J M^-1 (J^T z): with the
 // merged matrix of solve_zone_rows an iteration was a quarter shorter, but
 // the rounding of its entries cost an ill-conditioned zone two digits of dx.
-// Every result is bit for bit that of the vectors in global memory (the same
-// tree of sums over RESCUE_NT threads, correctly rounded divisions).  A zone
-// of 97 rows (93 iterations) 853 -> 584 us, one of 354 rows (75) 1,175 -> 835.
+// An iteration sums over the tree of the float64 solver's RESCUE_NT threads and
+// divides as it does (the unstaged form below has twice the threads, hence
+// another tree).  A zone of 97 rows (93 iterations) 853 -> 584 us, one of 354 rows (75) 1,175 -> 835.
 // False when the zone does not fit (nothing done); otherwise lambda is stored and the count in its.
 constexpr int RESCUE_THREADS = 512;
 constexpr int RESCUE_VT = RESCUE_THREADS - 32;  // threads with vertices
 
-// a / b from y = 1 / b rounded to nearest (Markstein, 1990): a y, corrected by
-// its residual, is a / b rounded to nearest
+// a / b rounded to nearest from y = 1 / b rounded to nearest.  a y is off by up to
+// 1.5 ulp; corrected by its residual it is within an ulp, and from there the
+// second correction is a / b rounded to nearest (Markstein 1990, which asks for
+// such a start).  Results and residuals that may be subnormal divide instead.
 __device__ __forceinline__ double div_by(double a, double b, double y) {
-    const double q = a * y, c = fma(fma(-b, q, a), y, q);
+    const double q = a * y, f = fma(fma(-b, q, a), y, q), c = fma(fma(-b, f, a), y, f);
     return isfinite(q) && fabs(q) > 1e-280 && fabs(a) > 1e-280 ? c : a / b;
 }
 
