@@ -210,7 +210,8 @@ typedef struct {
 typedef enum {
     HFCR_STAGE_VALIDATE = 0,  /* input range / finiteness checks */
     HFCR_STAGE_BVH = 1,       /* hierarchy build and refit */
-    HFCR_STAGE_TRAVERSE = 2,  /* the traversal + exact narrow-phase kernel, one interval per launch */
+    HFCR_STAGE_TRAVERSE = 2,  /* the traversal and the exact narrow phase (two kernels), one interval
+                                 per direction */
     HFCR_STAGE_STENCILS = 3,  /* pair sort, pair records, stencil keys, sort, unique */
     HFCR_STAGE_ASSEMBLE = 4,  /* constraint rows and the vertex CSR */
     HFCR_STAGE_SOLVE = 5,     /* Eq. 7 / Eq. 8 solve */

@@ -324,7 +324,7 @@ hfcr_status read_back(hfcr_ctx *ctx, cudaStream_t s);
 // Unique edges of a triangle list, their number to *ne; synchronises.  They
 // go to out by the buckets and to own by the sort (each with room for
 // 3 n_tris of them, 8-byte aligned); *at says which.  With an index out of
-// range nothing went to out.  C_SLOW is zero before.
+// range nothing went to out.  C_SLOW is zero before and after.
 hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts, int *out, int *own,
                          int slot, const int **at, int *ne, cudaStream_t s) {
     // the buckets' words fit the vertex scratch of the reservation; a caller

@@ -400,9 +400,6 @@ __device__ __forceinline__ double block_sum_uniform(double x, double *redd) {
     return s;
 }
 
-// The thread group that solves one zone: a whole CTA (CtaGroup) or one
-// warp (WarpGroup, for small zones; barriers are __syncwarp and every
-// reduction stays in shuffles).  Sums are identical in every lane.
 // a, b, c summed over the warp by halving (six shuffles instead of fifteen):
 // the lanes 8 k .. 8 k + 7 end with sum k (k < 3)
 __device__ __forceinline__ float warp_halve3(float a, float b, float c) {
@@ -433,6 +430,9 @@ __device__ __forceinline__ void group_halve3(float a, float b, float c, float *s
     sc = __shfl_sync(0xffffffffu, t, 16);
 }
 
+// The thread group that solves one zone: a whole CTA (CtaGroup) or one
+// warp (WarpGroup, for small zones; barriers are __syncwarp and every
+// reduction stays in shuffles).  Sums are identical in every lane.
 struct CtaGroup {
     static constexpr int SIZE = 512;  // of the solvers by rows
     __device__ static void sum3h(float a, float b, float c, float *scr, float &sa, float &sb, float &sc) {
@@ -2357,8 +2357,9 @@ __device__ __forceinline__ void zone64_precond(const ZoneArgs &a, int s0, int g0
 // the rounding of its entries cost an ill-conditioned zone two digits of dx.
 // An iteration sums over the tree of the float64 solver's RESCUE_NT threads and
 // divides as it does (the unstaged form below has twice the threads, hence
-// another tree).  A zone of 97 rows (93 iterations) 853 -> 584 us, one of 354 rows (75) 1,175 -> 835.
-// False when the zone does not fit (nothing done); otherwise lambda is stored and the count in its.
+// another tree).  A zone of 97 rows (93 iterations) 853 -> 584 us, one of 354
+// rows (75) 1,175 -> 835.  False when the zone does not fit (nothing done);
+// otherwise lambda is stored and the count in its.
 constexpr int RESCUE_THREADS = 512;
 constexpr int RESCUE_VT = RESCUE_THREADS - 32;  // threads with vertices
 

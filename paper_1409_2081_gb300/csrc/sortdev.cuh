@@ -202,8 +202,8 @@ __device__ __forceinline__ void sort_small_body(K *k0, int *v0, K *k1, int *v1, 
     }
 }
 
-// sum of state[0 .. i) for CTA i of a single-pass scan (its own sum published
-// first); a state word is 0, or (1: the CTA's sum, 2: the sum up to it) << 32
+// sum of state[0 .. i) for CTA i of a single-pass scan with decoupled look-back
+// (Merrill and Garland 2016; its own sum published first); a state word is 0, or (1: the CTA's sum, 2: the sum up to it) << 32
 // | value.  The waits are bounded: after the limit ST_TIMEOUT is recorded
 // and what was seen is returned.  Called by one warp.
 __device__ __forceinline__ unsigned lookback(unsigned long long *state, int i, unsigned sum,
