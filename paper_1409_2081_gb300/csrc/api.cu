@@ -328,8 +328,8 @@ hfcr_status read_back(hfcr_ctx *ctx, cudaStream_t s);
 hfcr_status derive_edges(hfcr_ctx *ctx, const int *tris, int n_tris, int n_verts, int *out, int *own,
                          int slot, const int **at, int *ne, cudaStream_t s) {
     // the buckets' words fit the vertex scratch of the reservation; a caller
-    // with more vertices than reserved takes the sort
-    bool buckets = n_tris > 0 && n_verts > 0 &&
+    // with more vertices than reserved, or many more than triangles, takes the sort
+    bool buckets = n_tris > 0 && n_verts > 0 && bucket_worth(n_tris, n_verts) &&
                    bucket_words(n_verts) * sizeof(int) <= sizeof(double) * 6 * (size_t)ctx->max_verts;
     bool hubs = bucket_hubs_first(n_tris);
     while (true) {

@@ -959,6 +959,16 @@ static void bucket_edges(const int *tris, int n_tris, int n_verts, int *edges_ou
 
 bool bucket_hubs_first(int n_tris) { return n_tris <= BUCKET_HUBS_TRIS; }
 
+// The buckets pass over every vertex id (some 40 us a million), the sort over the
+// half-edges (by ranks up to RANK_MAX of them, 50 us; 85 us and 0.27 a thousand
+// triangles above): a short list over many ids is the sort's.  1,000 triangles
+// of 2,000,000 ids 107 us by buckets and 50 by the sort, 100,000 of 10,000,000
+// 427 and 108; 20,000 of 1,000,000 79 and 89.
+bool bucket_worth(int n_tris, int n_verts) {
+    const long long most = 3ll * n_tris <= RANK_MAX ? 300000 : 1000000 + 5ll * n_tris;
+    return n_verts <= most;
+}
+
 void build_edges(const int *tris, int n_tris, int n_verts, bool hubs, int *edges_out, int *d_count, int *d_slow,
                  unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
                  cudaStream_t s) {

@@ -168,6 +168,7 @@ void build_edges(const int *tris, int n_tris, int n_verts, bool hubs, int *edges
                  unsigned long long *keys, unsigned long long *keys_alt, int *words, uint32_t *d_status,
                  cudaStream_t s);
 bool bucket_hubs_first(int n_tris);
+bool bucket_worth(int n_tris, int n_verts);  // against build_edges_sorted
 size_t bucket_words(int n_verts);
 // The same by a radix sort of all the edges' keys.  Scratch: keys/keys_alt of
 // 3 * n_tris u64 and flags of 3 * n_tris unsigned.

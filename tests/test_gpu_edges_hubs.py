@@ -42,7 +42,7 @@ LISTS = {f"fan_{k}": (fan(k), 4) for k in (15, 16, 17, 63, 64, 65, 128, 1983, 19
 LISTS |= {f"mixed_{k}": (shuffled(fan(k)), 4) for k in (17, 60, 300, 3000, 15000)}
 LISTS |= {f"sphere_{k}": (sphere(k), 4) for k in (20, 100, 1000, 3000)}
 LISTS |= {
-    "spread_1000": (hubs(1, 1000, 600_000), 4), "spread_100": (hubs(3, 100, 100_000), 4),
+    "spread_1000": (hubs(1, 1000, 290_000), 4), "spread_100": (hubs(3, 100, 100_000), 4),
     "hubs_60": (hubs(60, 17, 4000), 4), "hubs_8": (hubs(8, 200, 900), 4), "hubs_5": (hubs(5, 700, 4000), 4),
     "too_many": (hubs(256, 17, 4000), 0), "too_many_hubs": (hubs(30, 1000, 4000), 0),
     "large": (sphere(16, 3200), 4), "large_17": (sphere(17, 3000), 8), "large_hub": (sphere(1000, 60), 8),
