@@ -576,13 +576,28 @@ __device__ __forceinline__ void cg_precond_blocks(const V &v, int k) {
     }
 }
 
+// A vertex's list is summed by one thread, the list of a hub (more than HUB_LIST
+// entries) by its warp: a response around a hub of 300 rows 460 -> 365 us, of
+// 1,300 2,510 -> 1,420 (with the early rejection of its matrix, solve_zone_rows).
+// A warp sums its hubs one after another, so shorter lists stay with the
+// threads, which sum 32 at a time (with 32 here 1,024 pairs of spheres, whose
+// coarse ones have lists of 40 to 60, took 140 us more).
+constexpr int HUB_LIST = 128;
+
+// whether one of this warp's vertices is a hub
 template <class Gp, class V>
-__device__ __forceinline__ void cg_matvec_vertex(const V &v, int U) {
+__device__ __forceinline__ bool cg_hubs(const V &v, int U) {
+    bool hub = false;
+    for (int j = Gp::rank(); j < U; j += Gp::size()) hub = hub || (int)v.seg[j + 1] - (int)v.seg[j] > HUB_LIST;
+    return __any_sync(0xffffffffu, hub);
+}
+
+template <class Gp, class V>
+__device__ __forceinline__ void cg_matvec_vertex(const V &v, int U, bool hubs) {
     const float third = 1.0f / 3.0f;
-    for (int j = Gp::rank(); j < U; j += Gp::size()) {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-        const int e1 = (int)v.seg[j + 1] - v.eoff;
-        for (int e = (int)v.seg[j] - v.eoff; e < e1; ++e) {
+    // u of vertex j, its list's entries from, from + step, ... below e1 added up
+    auto sum = [&](int from, int e1, int step, float &a0, float &a1, float &a2) {
+        for (int e = from; e < e1; e += step) {
             int c = (int)v.cval[e] - v.coff;
             int s = c >> 2;
             float ps = ((c & 3) ? -third : 1.0f) * v.z[s];
@@ -591,8 +606,35 @@ __device__ __forceinline__ void cg_matvec_vertex(const V &v, int U) {
             a1 += ps * n.y;
             a2 += ps * n.z;
         }
+    };
+    for (int j = Gp::rank(); j < U; j += Gp::size()) {
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+        const int e0 = (int)v.seg[j] - v.eoff, e1 = (int)v.seg[j + 1] - v.eoff;
+        if (hubs && e1 - e0 > HUB_LIST) continue;
+        sum(e0, e1, 1, a0, a1, a2);
         float w = v.winv[j];
         v.u[j] = make_float4(w * a0, w * a1, w * a2, 0.f);
+    }
+    if (!hubs) return;
+    const int lane = threadIdx.x & 31;
+    for (int j0 = Gp::rank() - lane; j0 < U; j0 += Gp::size()) {
+        const int j = j0 + lane;
+        const int e0 = j < U ? (int)v.seg[j] - v.eoff : 0, e1 = j < U ? (int)v.seg[j + 1] - v.eoff : 0;
+        for (unsigned m = __ballot_sync(0xffffffffu, e1 - e0 > HUB_LIST); m; m &= m - 1u) {
+            const int o = __ffs(m) - 1, h0 = __shfl_sync(0xffffffffu, e0, o), h1 = __shfl_sync(0xffffffffu, e1, o);
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+            sum(h0 + lane, h1, 32, a0, a1, a2);
+#pragma unroll
+            for (int q = 16; q; q >>= 1) {
+                a0 += __shfl_xor_sync(0xffffffffu, a0, q);
+                a1 += __shfl_xor_sync(0xffffffffu, a1, q);
+                a2 += __shfl_xor_sync(0xffffffffu, a2, q);
+            }
+            if (lane == o) {
+                float w = v.winv[j];
+                v.u[j] = make_float4(w * a0, w * a1, w * a2, 0.f);
+            }
+        }
     }
 }
 
@@ -618,13 +660,14 @@ template <class Gp, class V>
 __device__ __forceinline__ int cg_cg_loop(const V &v, int k, int U, int maxit, float tol,
                                           float *red) {
     const int tid = Gp::rank(), nt = Gp::size();
+    const bool hubs = cg_hubs<Gp>(v, U);
     if (v.bperm) {
         cg_precond_blocks<Gp>(v, k);
     } else {
         for (int g = tid; g < v.G; g += nt) cg_precond_group(v, g);
     }
     Gp::sync();
-    cg_matvec_vertex<Gp>(v, U);
+    cg_matvec_vertex<Gp>(v, U, hubs);
     Gp::sync();
     float ga = 0.f, de = 0.f, rh = 0.f;
     for (int s = tid; s < k; s += nt) {
@@ -669,7 +712,7 @@ __device__ __forceinline__ int cg_cg_loop(const V &v, int k, int U, int maxit, f
             }
         }
         Gp::sync();
-        cg_matvec_vertex<Gp>(v, U);
+        cg_matvec_vertex<Gp>(v, U, hubs);
         Gp::sync();
         ga = 0.f;
         de = 0.f;
@@ -1746,6 +1789,26 @@ __device__ __forceinline__ int solve_zone_rows(const ZoneArgs &a, int z, char *b
         }
         return n;
     };
+    // a row has at least the entries of its longest list: the rows of a hub, on
+    // which merging is slow, are found too long before they are merged (700 rows
+    // took 130 us to find it out, 1,300 half a millisecond)
+#pragma unroll
+    for (int v = 0; v < RPT; ++v) {
+        const int t = tid + v * NT;
+        int most = 0;
+        if (t < k) {
+            const ushort4 g = vidx[t];
+            most = max(max(seg[g.x + 1] - seg[g.x], seg[g.y + 1] - seg[g.y]),
+                       max(seg[g.z + 1] - seg[g.z], seg[g.w + 1] - seg[g.w]));
+        }
+        most = (int)__reduce_max_sync(0xffffffffu, (unsigned)most);
+        if (lane == 0) sl[wq + v * (NT / 32)] = most;
+    }
+    Gp::sync();
+    int least = 0;
+    for (int q = 0; q < NS; ++q) least += sl[q];
+    if (fixed - 64 + 256ll * least > bytes) return 1;
+    Gp::sync();
     int off[RPT], len[RPT];
 #pragma unroll
     for (int v = 0; v < RPT; ++v) {
