@@ -993,24 +993,64 @@ __device__ __forceinline__ void store_inv_row(double4_32a *p, const double *row)
     *p = make_double4_32a(row[0], row[1], row[2], row[3]);
 }
 
-// Groups first + i (i = 0, step, ...) below n, eight per warp: the four lanes
-// of a quad hold the block's rows and run Gauss-Jordan with partial pivoting
-// in registers, exchanging rows by shuffles.  A (near-)singular block falls
-// back to the inverse of its diagonal.  Called by whole warps; gi: the
-// warp's first group, step: the groups of all warps taking part.  Bound by
-// the latency of the loads and of float64 arithmetic: one thread per group
-// with the block in local memory took 33 us (1,000 to 2,000 groups), a quad
-// 14 us.  R: float4 rows for the mixed solver, double4_32a rows for the
-// float64 one; perm: row t is row perm[t] of ids and n64.
+// w / 9, without the division where there are no masses
+__device__ __forceinline__ double ninth(double w) { return w == 1.0 ? 1.0 / 9.0 : w / 9.0; }
+
+// Groups first .. n - 1, shared out over nw warps (this is warp wi), eight per
+// warp: the four lanes of a quad hold the block's rows and run Gauss-Jordan with
+// partial pivoting in registers, exchanging rows by shuffles.  A (near-)
+// singular block falls back to the inverse of its diagonal.  Called by whole
+// warps.  Bound by the latency of the loads and of float64 arithmetic: one
+// thread per group with the block in local memory took 33 us (1,000 to 2,000
+// groups), a quad 14 us.  Where few warps have many groups each (the
+// cooperative setup just above what one CTA sets up), 32 groups of one row are
+// taken at once, a lane each, with the bits of the quads: a response to 4,097
+// stencils 528 -> 483 us.  R: float4 rows for the mixed solver, double4_32a rows
+// for the float64 one; perm: row t is row perm[t] of ids and n64.
 template <class G, typename R>
-__device__ __forceinline__ void group_inverses(int gi, int step, int n, const int *gst, const int4 *ids,
+__device__ __forceinline__ void group_inverses(int first, int wi, int nw, int n, const int *gst, const int4 *ids,
                                                const double4_32a *n64, int nA, const float *wA,
                                                const float *wB, R *pinv, const int *perm = nullptr) {
     static_assert(GMAX == 4, "a quad holds one block");
     constexpr unsigned ALL = 0xffffffffu;
     const int lane = threadIdx.x & 31, a = lane & 3, q0 = lane & ~3;
-    for (; gi < n; gi += step) {
-        const int g = gi + (lane >> 2);
+    const int per = n - first > 24 * nw ? 32 : 8;
+    for (int g8 = first + per * wi; g8 < n;) {
+        if (per == 32 && (g8 - first) % 32 == 0) {
+            const int g = g8 + lane;
+            const int a0 = g < n ? G::ld(gst + g) : 0, m = g < n ? G::ld(gst + g + 1) - a0 : 0;
+            if (!__any_sync(ALL, m > 1)) {
+                if (m == 1) {
+                    const int t = perm ? G::ld(perm + a0) : a0;
+                    const int4 v = G::ld(ids + t);
+                    const double4_32a nv = ld_n64<G>(n64 + t);
+                    const double w0 = inv_mass_of(v.x, nA, wA, wB), w1 = inv_mass_of(v.y, nA, wA, wB),
+                                 w2 = inv_mass_of(v.z, nA, wA, wB), w3 = inv_mass_of(v.w, nA, wA, wB);
+                    const int f[3] = {v.y, v.z, v.w};
+                    const double d[3] = {ninth(w1), ninth(w2), ninth(w3)};
+                    double w = w0;
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+#pragma unroll
+                        for (int q = 0; q < 3; ++q)
+                            if (f[p] == f[q]) w += d[p];
+                    const double A = (nv.x * nv.x + nv.y * nv.y + nv.z * nv.z) * w;
+                    double row[GMAX] = {0.0, 0.0, 0.0, 0.0};
+                    if (fabs(A) > 1e-12 * fabs(A)) {
+                        row[0] = 1.0 / A;
+                    } else {
+                        const double x = w0 + (w1 + w2 + w3) / 9.0;
+                        row[0] = x > 0.0 ? 1.0 / x : 0.0;
+                    }
+                    store_inv_row(pinv + a0, row);
+                }
+                g8 += 32 * nw;
+                continue;
+            }
+        }
+        const int g = g8 + (lane >> 2);
+        // eight groups further, behind the last of this warp's 32 (or 8) its next ones
+        g8 += (g8 - first) % per == per - 8 ? per * nw - per + 8 : 8;
         const int a0 = g < n ? G::ld(gst + g) : 0, m = g < n ? G::ld(gst + g + 1) - a0 : 0;
         const int mmax = (int)__reduce_max_sync(ALL, (unsigned)m);
         int4 v = make_int4(0, 0, 0, 0);
@@ -1025,7 +1065,6 @@ __device__ __forceinline__ void group_inverses(int gi, int step, int n, const in
             w2 = inv_mass_of(v.z, nA, wA, wB);
             w3 = inv_mass_of(v.w, nA, wA, wB);
         }
-        auto ninth = [](double w) { return w == 1.0 ? 1.0 / 9.0 : w / 9.0; };  // no division without masses
         const double d1 = ninth(w1), d2 = ninth(w2), d3 = ninth(w3);
         double A[2 * GMAX], diag = 0.0;
 #pragma unroll
@@ -1108,8 +1147,8 @@ __global__ void k_group_inverse(const int *d_ng, const int *gst, const int4 *ids
                                 float4 *pinv) {
     HFCR_PDL_WAIT();
     const int nw = blockDim.x >> 5;
-    group_inverses<PlainLd>(8 * (int)(blockIdx.x * nw + (threadIdx.x >> 5)), 8 * (int)gridDim.x * nw,
-                            *d_ng, gst, ids, n64, nA, wA, wB, pinv);
+    group_inverses<PlainLd>(0, (int)(blockIdx.x * nw + (threadIdx.x >> 5)), (int)gridDim.x * nw, *d_ng, gst,
+                            ids, n64, nA, wA, wB, pinv);
 }
 
 // float64 residual r = b - J M^-1 J^T lam of one zone (the float64 normals;
@@ -2629,8 +2668,8 @@ __global__ void __launch_bounds__(RESCUE ? RESCUE_THREADS : ZONE64_THREADS)
         const double bb = zone_start<CtaGroup>(a, s0, k, redd);  // lam = 0 on the zone's rows
         // the zone's block-Jacobi inverses in float64 (a block of nearly
         // dependent rows has a large inverse that float32 would not hold)
-        group_inverses<PlainLd>(g0 + 8 * (int)(threadIdx.x >> 5), 8 * (int)(blockDim.x >> 5), g0 + G,
-                                a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv64);
+        group_inverses<PlainLd>(g0, (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5), g0 + G, a.gst,
+                                a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv64);
         __syncthreads();  // the blocks, read by other threads below
         double *r = g.r + s0, *p = g.p + s0, *sv = g.s + s0, *w = g.w + s0, *zz = g.z + s0;
         double *x = a.lam + s0, *u = a.u64 + 3 * (size_t)j0;
@@ -3437,8 +3476,8 @@ constexpr int SETUP_READY = 1;
 // the inverse blocks of CTAs first .. first + n - 1 (consecutive groups on
 // different CTAs)
 __device__ __forceinline__ void setup_inverses(const SetupArgs &a, int first, int n) {
-    group_inverses<L2Ld>(8 * ((int)(threadIdx.x >> 5) * n + (int)blockIdx.x - first), 8 * n * (TPB / 32),
-                         __ldcg(a.d_ng), a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv);
+    group_inverses<L2Ld>(0, (int)(threadIdx.x >> 5) * n + (int)blockIdx.x - first, n * (TPB / 32), __ldcg(a.d_ng),
+                         a.gst, a.ids, a.n64, a.nA, a.wA, a.wB, a.pinv);
 }
 
 // a CTA not taking part in the phases (first = the first such CTA): waits
@@ -4070,7 +4109,7 @@ __device__ __forceinline__ void setup_rows(const SetupArgs &a, int k) {
         a.n32[t] = a.n32_raw[src];
         a.b[t] = a.b_raw[src];
     }
-    group_inverses<PlainLd>(8 * wi, 8 * nw, *a.d_ng, a.gst, a.ids_raw, a.n64_raw, a.nA,
+    group_inverses<PlainLd>(0, wi, nw, *a.d_ng, a.gst, a.ids_raw, a.n64_raw, a.nA,
                             a.wA, a.wB, a.pinv, a.zsrc);
 }
 

@@ -32,3 +32,12 @@ def test_a_large_zone_among_others(switch, monkeypatch):
     monkeypatch.setattr(api, "Context", lambda **kw: context(block_switch_iters=switch, **kw))
     monkeypatch.setattr(base, "SYSTEMS", {"mixed": ([130, 20], [1300, 300, 40, 1200] + [5] * 30, 2)})
     base.test_paths_identical("mixed", True)
+
+
+# more groups than a few warps take eight at a time: of one row, of several, mixed
+@pytest.mark.parametrize("masses", [False, True], ids=["unit", "masses"])
+@pytest.mark.parametrize("strips,share", [([17] * 242, 1), ([4200], 1), ([9000], 1), ([5000], 2), ([6000], 7), ([5001], 5),
+                                          ([3000, 40, 3000], 3), ([1] * 9000, 1)])
+def test_many_groups(strips, share, masses, monkeypatch):
+    monkeypatch.setattr(base, "SYSTEMS", {"groups": ([], strips, share)})
+    base.test_paths_identical("groups", masses)
