@@ -580,8 +580,8 @@ __device__ __forceinline__ void cg_precond_blocks(const V &v, int k) {
 // entries) by its warp: a response around a hub of 300 rows 460 -> 365 us, of
 // 1,300 2,510 -> 1,420 (with the early rejection of its matrix, solve_zone_rows).
 // A warp sums its hubs one after another, so shorter lists stay with the
-// threads, which sum 32 at a time (with 32 here 1,024 pairs of spheres, whose
-// coarse ones have lists of 40 to 60, took 140 us more).
+// threads, which sum 32 at a time (with 32 here a repair step of 1,024 pairs of
+// spheres, whose coarse ones have lists of 40 to 60, took 2,048 us for 1,938).
 constexpr int HUB_LIST = 128;
 
 // whether one of this warp's vertices is a hub
